@@ -83,7 +83,7 @@ int check_common(const ctqw_hamiltonian *h, int dtype, const void *psi, double d
 // otherwise one launch per stage.
 int taylor_step_plain(const ctqw_hamiltonian *h, int dtype, const void *in, void *out, void *phiA,
                       void *phiB, double dt, int K, cudaStream_t s) {
-    const int tshape = tiled_default_shape(K);
+    const int tshape = tiled_default_shape(h, K);
     if (dtype == CTQW_C64 && tiled_supported(h, dtype, tshape)) {
         const int D = tiled_depth(tshape);
         const void *w = in;
@@ -744,7 +744,7 @@ static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double
         if (st == CTQW_OK) {
             void *const bufs[3] = {psi_dev, w + sb, w + 2 * sb};
             st = tiled_steps(h, bufs, lo, dt, K, n_steps, obs_every, P_mean_dev, norm_dev, energy_dev, comp,
-                             tiled_default_shape(K), SwitchSpec{}, R_f, R_t, side);
+                             tiled_default_shape(h, K), SwitchSpec{}, R_f, R_t, side);
         }
         // joined even after an error: nothing of this call stays behind the caller's stream
         if (cudaEventRecord(h->join_ev, side) != cudaSuccess || cudaStreamWaitEvent(s, h->join_ev, 0) != cudaSuccess)
@@ -792,9 +792,9 @@ static int propagate_taylor_impl(const ctqw_hamiltonian *h, int32_t dtype, void 
     // (N > 256, ragged sizes, other N): the temporally blocked tiled kernel
     // with the iterate in registers, at the depth that needs the fewest
     // launches a step (depth 8 was the fastest measured of 2, 4, 8)
-    if (!fused && !(flags & CTQW_FLAG_PLAIN) && shape == 0 && tiled_supported(h, dtype, tiled_default_shape(K)))
+    if (!fused && !(flags & CTQW_FLAG_PLAIN) && shape == 0 && tiled_supported(h, dtype, tiled_default_shape(h, K)))
         return propagate_tiled(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,
-                               energy_dev, flags, tiled_default_shape(K), workspace_dev,
+                               energy_dev, flags, tiled_default_shape(h, K), workspace_dev,
                                workspace_bytes, s);
     if (!fused) {
         const size_t need = 3 * (size_t)h->total_amp * elem_bytes(dtype);
@@ -842,7 +842,7 @@ static int propagate_switching_impl(const ctqw_hamiltonian *h, int32_t dtype, vo
     sw.on = true;
     sw.seed = seed;
     sw.p = p_switch;
-    const int tshape = tiled_default_shape(K);
+    const int tshape = tiled_default_shape(h, K);
     if (!(flags & CTQW_FLAG_PLAIN) && tiled_supported(h, dtype, tshape))
         return propagate_tiled(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,
                                energy_dev, flags, tshape, workspace_dev, workspace_bytes, s, sw);

@@ -465,14 +465,15 @@ int rows_clusters(const RowsShape &f, int *clusters) {
 }  // namespace
 
 // Tiled-to-fused throughput ratio per SM, measured on two bosons at N = 256,
-// K = 16 (register tiles at depth 8 against the full-row clusters).
-static constexpr double kTiledPerSmRatio = 0.25;
+// K = 16: register tiles 4.43e11 site-updates/s on 152 SMs, the full-row
+// clusters 8.74e11 on the 112 that hold them.
+static constexpr double kTiledPerSmRatio = 0.37;
 
 int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) {
     *R_tiled = 0;
     RowsShape f;
     if (!fused_rows_supported(h, CTQW_C64) || !rows_shape_for(h->Nmax, shape, f) ||
-        !tiled_supported(h, CTQW_C64, tiled_default_shape(K)) || h->group_N.size() != 1)
+        !tiled_supported(h, CTQW_C64, tiled_default_shape(h, K)) || h->group_N.size() != 1)
         return CTQW_OK;
     CTQW_TRY(set_rows_attributes(f));
     int clusters = 0, per_sm = 0, n_sm = 0;

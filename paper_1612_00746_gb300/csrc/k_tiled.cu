@@ -21,6 +21,9 @@
 // its rounding error carried in a second FP32 word (lo, in place: every
 // element is read and written by its own tile only), and the new psi goes to
 // a separate buffer because other tiles still read the old psi as halo.
+#include <algorithm>
+#include <type_traits>
+
 #include "ctqw_internal.cuh"
 #include "fused_common.cuh"
 
@@ -55,6 +58,7 @@ struct TiledArgs {
     int n_stages;            // D, or fewer for the last launch of a step
     int final;               // the launch's last stage is j = 1 (state update)
     int compensated;
+    int aligned16;           // every buffer starts on a 16-byte boundary
 };
 
 
@@ -244,14 +248,71 @@ __global__ void __launch_bounds__(256) taylor_tiled_kernel(const __grid_constant
 // __syncthreads).  psi of the region stays in shared memory.  The shuffles
 // wrap from column 63 to 0 and the outermost warps read zero rows: both
 // only touch the halo's outer ring, which stage 1 already leaves inexact.
+//
+// Everything a block reads from HBM is requested before its first stage:
+// psi of the region and, for a final launch, the carried error word of the
+// tile, both by cp.async into shared memory (a lane reads back only slots it
+// filled itself, so they need no barrier).  The row coefficients are 8-byte
+// broadcasts: 16-byte ones cost twice the shared-memory wavefronts, and that
+// pipe is the bound (78% busy; 8 warps x 3 blocks an SM).  The ragged batch
+// of 512 realizations, N = 128..1024, K = 8, 20 steps: 97.5 ms with the
+// error words read in the final stage and psi read twice, 79.9 ms with both
+// fetched at the start, 74.2 ms with the 8-byte coefficients and the regions
+// that tiled_default_shape picks.
+template <int D, int W>
+struct RegTile {
+    static constexpr int RS = 8 * W, RL = 8;              // region rows, rows a warp
+    static constexpr int T = RS - 2 * D, T2 = 64 - 2 * D;   // tile rows and columns
+    static constexpr size_t q_bytes = sizeof(float4) * RS * 32;
+    static constexpr size_t lo_bytes = (sizeof(float2) * T * T2 + 15) / 16 * 16;
+    static constexpr size_t edge_bytes = sizeof(float4) * 2 * W * 2 * 32;
+    static constexpr size_t smem = q_bytes + lo_bytes + edge_bytes + sizeof(float4) * 32 + sizeof(float2) * (RS + 1) + sizeof(int) * RS;
+};
+
+// One stencil stage of a warp's 8 x 64 block: y = dt H P, then
+//   !FINAL: P <- psi + (-i / j) y;
+//   FINAL: psi + (-i) y on the tile, with the rounding error carried in lo.
+// u4, d4: the rows above and below; Q: this lane's psi (row stride 32
+// float4); diag: bit (2 i + k) set where row i, column k is on x1 = x2
+// (DIAG: some bit of the warp is set).
+template <bool DIAG>
+__device__ __forceinline__ void reg_stencil_row(const float2 (&P)[8][2], int i, const float2 (&prev)[2], float4 d4,
+                                                float2 rc, float2 rn, const float2 (&ec)[2], const float2 (&nJc)[3],
+                                                float2 dU, unsigned diag, int from_left, int from_right,
+                                                float2 &y0, float2 &y1) {
+    const float2 c0 = P[i][0], c1 = P[i][1];
+    const float2 lft = shfl2(c1, from_left), rgt = shfl2(c0, from_right);
+    const float2 n0 = i < 7 ? P[i < 7 ? i + 1 : 7][0] : make_float2(d4.x, d4.y);
+    const float2 n1 = i < 7 ? P[i < 7 ? i + 1 : 7][1] : make_float2(d4.z, d4.w);
+    const float2 er = make_float2(rc.x, rc.x), jup = make_float2(rc.y, rc.y), jdn = make_float2(rn.y, rn.y);
+    y0 = __fmul2_rn(ec[0], c0);
+    y1 = __fmul2_rn(ec[1], c1);
+    y0 = __ffma2_rn(er, c0, y0);
+    y1 = __ffma2_rn(er, c1, y1);
+    y0 = __ffma2_rn(jup, prev[0], y0);
+    y1 = __ffma2_rn(jup, prev[1], y1);
+    y0 = __ffma2_rn(jdn, n0, y0);
+    y1 = __ffma2_rn(jdn, n1, y1);
+    y0 = __ffma2_rn(nJc[0], lft, y0);
+    y1 = __ffma2_rn(nJc[1], c0, y1);
+    y0 = __ffma2_rn(nJc[1], c1, y0);
+    y1 = __ffma2_rn(nJc[2], rgt, y1);
+    if (DIAG) {
+        if (diag & (1u << (2 * i))) y0 = __ffma2_rn(dU, c0, y0);
+        if (diag & (1u << (2 * i + 1))) y1 = __ffma2_rn(dU, c1, y1);
+    }
+}
+
 template <int D, int W>
 __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kernel(const __grid_constant__ TiledArgs a) {
-    constexpr int RS = 8 * W, T = RS - 2 * D, T2 = 64 - 2 * D, RL = 8;   // rows x 64 columns
+    using Tile = RegTile<D, W>;
+    constexpr int RS = Tile::RS, T = Tile::T, T2 = Tile::T2, RL = Tile::RL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4 *Q = reinterpret_cast<float4 *>(smem_raw);            // [RS][32] psi, (row, lane) -> 2 columns
-    float4 *edge = Q + RS * 32;                                   // [2 parity][W warps][2][32]
+    float4 *Q = reinterpret_cast<float4 *>(smem_raw);                        // [RS][32] psi, (row, lane) -> 2 columns
+    float2 *los = reinterpret_cast<float2 *>(smem_raw + Tile::q_bytes);      // [T][T2] carried error of the tile
+    float4 *edge = reinterpret_cast<float4 *>(smem_raw + Tile::q_bytes + Tile::lo_bytes);   // [2 parity][W warps][2][32]
     float4 *zero = edge + 2 * W * 2 * 32;                         // [32] a row of zeros
-    float4 *rowc = zero + 32;                                     // [RS + 1] (dt eps, dt eps, -dt J_up, -dt J_up)
+    float2 *rowc = reinterpret_cast<float2 *>(zero + 32);         // [RS + 1] (dt eps, -dt J of the bond above)
     int *x_row = reinterpret_cast<int *>(rowc + RS + 1);          // [RS]
 
     const TileItem item = tile_item(a);
@@ -263,137 +324,225 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kerne
     const float dt = a.dt;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r0 = warp * RL;
+    auto wrap = [N](int x) { return x < 0 || x >= N ? (x % N + N) % N : x; };
 
+    // this warp's rows (a row index of its own: no barrier before the loads)
+    if (lane < RL) x_row[r0 + lane] = wrap(x1_0 + r0 + lane);
+    __syncwarp();
+    int X2[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) X2[k] = wrap(x2_0 + 2 * lane + k);
+    // pairs of columns are 16 bytes apart and never straddle the wrap
+    const bool vec = a.aligned16 && D % 2 == 0 && ((N | (int)(base & 1)) & 1) == 0;
+    // the tile's part of this lane and warp
+    bool col_in[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int ck = 2 * lane + k;
+        col_in[k] = ck >= D && ck < D + T2 && x2_0 + ck < N;
+    }
+    auto row_in = [&](int ri) { return ri >= D && ri < D + T && x1_0 + ri < N; };
+
+    const float2 *win = a.w_in + base, *gpsi = a.psi + base;
+    const bool carried = a.final && a.compensated;
+    const uint32_t sQ = smem_u32(Q) + (uint32_t)(r0 * 32 + lane) * 16u;
+    // slot of (row, column) of the tile: negative rows and columns are never touched
+    const int lo_at = (r0 - D) * T2 + 2 * lane - D;
+    const uint32_t sL = smem_u32(los);
+    float2 P[RL][2];
+    if (vec) {
+#pragma unroll
+        for (int i = 0; i < RL; ++i)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sQ + i * 512u),
+                         "l"(gpsi + (int64_t)x_row[r0 + i] * N + X2[0])
+                         : "memory");
+    } else {
+#pragma unroll
+        for (int i = 0; i < RL; ++i) {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sQ + i * 512u + 8u * k),
+                             "l"(gpsi + (int64_t)x_row[r0 + i] * N + X2[k])
+                             : "memory");
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (carried) {
+        const float2 *glo = a.lo + base;
+#pragma unroll
+        for (int i = 0; i < RL; ++i) {
+            if (!row_in(r0 + i)) continue;
+            const int64_t grow = (int64_t)x_row[r0 + i] * N;
+            if (vec) {
+                if (col_in[0])
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sL + (uint32_t)(lo_at + i * T2) * 8u),
+                                 "l"(glo + grow + X2[0])
+                                 : "memory");
+            } else {
+#pragma unroll
+                for (int k = 0; k < 2; ++k)
+                    if (col_in[k])
+                        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sL + (uint32_t)(lo_at + i * T2 + k) * 8u),
+                                     "l"(glo + grow + X2[k])
+                                     : "memory");
+            }
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const bool own_w = a.w_in != a.psi;   // the launch starts from an iterate of its own
+    if (own_w) {
+#pragma unroll
+        for (int i = 0; i < RL; ++i) {
+            const float2 *g = win + (int64_t)x_row[r0 + i] * N;
+            if (vec) {
+                const float4 v = *reinterpret_cast<const float4 *>(g + X2[0]);
+                P[i][0] = make_float2(v.x, v.y);
+                P[i][1] = make_float2(v.z, v.w);
+            } else {
+                P[i][0] = g[X2[0]];
+                P[i][1] = g[X2[1]];
+            }
+        }
+    }
+    // coefficients of the region's rows and of this lane's columns
     for (int i = threadIdx.x; i <= RS; i += blockDim.x) {
-        const int X1 = ((x1_0 + i) % N + N) % N;
-        if (i < RS) x_row[i] = X1;
+        const int X1 = wrap(x1_0 + i);
         const float e = i < RS ? dt * a.eps[po + X1] : 0.f;
-        const float j = -dt * a.J[po + (X1 + N - 1) % N];
-        rowc[i] = make_float4(e, e, j, j);
+        const float j = -dt * a.J[po + (X1 == 0 ? N - 1 : X1 - 1)];
+        rowc[i] = make_float2(e, j);
     }
     if (threadIdx.x < 32) zero[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-    // this lane's columns and their coefficients
-    int X2[2];
     float2 ec[2], nJc[3];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        X2[k] = ((x2_0 + 2 * lane + k) % N + N) % N;
         const float v = dt * a.eps[po + X2[k]];
         ec[k] = make_float2(v, v);
     }
 #pragma unroll
-    for (int k = 0; k <= 2; ++k) {
-        const int X = ((x2_0 + 2 * lane + k - 1) % N + N) % N;   // bond left of column 2 lane + k
+    for (int k = 0; k <= 2; ++k) {   // bond left of column 2 lane + k
+        const int X = k < 2 ? (X2[k] == 0 ? N - 1 : X2[k] - 1) : X2[1];
         const float v = -dt * a.J[po + X];
         nJc[k] = make_float2(v, v);
     }
-    __syncthreads();
-    // psi of the region (asynchronous) and the input iterate into registers
-    const float2 *win = a.w_in + base, *gpsi = a.psi + base;
-    const uint32_t sQ = smem_u32(Q);
-    for (int i = warp; i < RS; i += W) {
-        const int64_t grow = (int64_t)x_row[i] * N;
+    unsigned diag = 0;
+    if (a.dtU != 0.f) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sQ + (uint32_t)((i * 32 + lane) * 16 + 8 * k)),
-                         "l"(gpsi + grow + X2[k])
-                         : "memory");
+        for (int i = 0; i < RL; ++i) {
+            const int X1 = x_row[r0 + i];
+            diag |= (X1 == X2[0] ? 1u << (2 * i) : 0u) | (X1 == X2[1] ? 2u << (2 * i) : 0u);
+        }
     }
-    float2 P[RL][2];
+    const bool any_diag = __any_sync(0xffffffffu, diag != 0);
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    if (!own_w) {
 #pragma unroll
-    for (int i = 0; i < RL; ++i) {
-        const int64_t grow = (int64_t)x_row[r0 + i] * N;
-        P[i][0] = win[grow + X2[0]];
-        P[i][1] = win[grow + X2[1]];
+        for (int i = 0; i < RL; ++i) {
+            const float4 q = Q[(r0 + i) * 32 + lane];
+            P[i][0] = make_float2(q.x, q.y);
+            P[i][1] = make_float2(q.z, q.w);
+        }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
 
     const float2 dU = make_float2(a.dtU, a.dtU);
     const int from_left = (lane + 31) & 31, from_right = (lane + 1) & 31;
-#pragma unroll 1
-    for (int d = 1; d <= a.n_stages; ++d) {
-        const int par = d & 1;
-        const int j = a.j0 - d + 1;
-        const bool last_final = a.final && d == a.n_stages;   // j == 1
-        const float inv_j = 1.0f / (float)j;
-        // publish this warp's first and last rows
+    const int n_mid = a.final ? a.n_stages - 1 : a.n_stages;   // stages that update the iterate
+    const float4 *Ql = Q + r0 * 32 + lane;
+    // publish the warp's first and last rows; the rows above and below it
+    float4 u4, d4;
+    auto exchange = [&](int par) {
         float4 *eb = edge + (par * W + warp) * 2 * 32;
         eb[lane] = make_float4(P[0][0].x, P[0][0].y, P[0][1].x, P[0][1].y);
         eb[32 + lane] = make_float4(P[RL - 1][0].x, P[RL - 1][0].y, P[RL - 1][1].x, P[RL - 1][1].y);
         __syncthreads();
-        const float4 u4 = warp > 0 ? edge[(par * W + warp - 1) * 2 * 32 + 32 + lane] : zero[lane];
-        const float4 d4 = warp < W - 1 ? edge[(par * W + warp + 1) * 2 * 32 + lane] : zero[lane];
+        u4 = warp > 0 ? edge[(par * W + warp - 1) * 2 * 32 + 32 + lane] : zero[lane];
+        d4 = warp < W - 1 ? edge[(par * W + warp + 1) * 2 * 32 + lane] : zero[lane];
+    };
+    auto mid = [&](auto diag_tag, float inv_j) {
         float2 prev[2] = {make_float2(u4.x, u4.y), make_float2(u4.z, u4.w)};
-        float4 rc = rowc[r0];
+        float2 rc = rowc[r0];
 #pragma unroll
         for (int i = 0; i < RL; ++i) {
-            const float2 c0 = P[i][0], c1 = P[i][1];
-            const float2 lft = shfl2(c1, from_left), rgt = shfl2(c0, from_right);
-            const float2 n0 = i < RL - 1 ? P[i + 1][0] : make_float2(d4.x, d4.y);
-            const float2 n1 = i < RL - 1 ? P[i + 1][1] : make_float2(d4.z, d4.w);
-            const float4 rn = rowc[r0 + i + 1];
-            const float2 er = make_float2(rc.x, rc.y), jup = make_float2(rc.z, rc.w), jdn = make_float2(rn.z, rn.w);
+            const float2 rn = rowc[r0 + i + 1];
+            float2 y0, y1;
+            reg_stencil_row<decltype(diag_tag)::value>(P, i, prev, d4, rc, rn, ec, nJc, dU, diag, from_left, from_right,
+                                                       y0, y1);
             rc = rn;
-            float2 y0 = __fmul2_rn(ec[0], c0), y1 = __fmul2_rn(ec[1], c1);
-            y0 = __ffma2_rn(er, c0, y0);
-            y1 = __ffma2_rn(er, c1, y1);
-            y0 = __ffma2_rn(jup, prev[0], y0);
-            y1 = __ffma2_rn(jup, prev[1], y1);
-            y0 = __ffma2_rn(jdn, n0, y0);
-            y1 = __ffma2_rn(jdn, n1, y1);
-            y0 = __ffma2_rn(nJc[0], lft, y0);
-            y1 = __ffma2_rn(nJc[1], c0, y1);
-            y0 = __ffma2_rn(nJc[1], c1, y0);
-            y1 = __ffma2_rn(nJc[2], rgt, y1);
-            const int X1w = x_row[r0 + i];
-            if (X1w == X2[0]) y0 = __ffma2_rn(dU, c0, y0);   // dt U on x1 = x2
-            if (X1w == X2[1]) y1 = __ffma2_rn(dU, c1, y1);
-            prev[0] = c0;
-            prev[1] = c1;
-            const float4 q = Q[(r0 + i) * 32 + lane];
-            if (!last_final) {
-                P[i][0] = make_float2(fmaf(inv_j, y0.y, q.x), fmaf(-inv_j, y0.x, q.y));
-                P[i][1] = make_float2(fmaf(inv_j, y1.y, q.z), fmaf(-inv_j, y1.x, q.w));
-            } else {
-                // psi(t+dt) = psi + (-i) y on the tile, rounding error carried in lo
-                const int ri = r0 + i;
-                if (ri >= D && ri < D + T && x1_0 + ri < N) {
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const int ck = 2 * lane + k;
-                        if (ck < D || ck >= D + T2 || x2_0 + ck >= N) continue;
-                        const int64_t g = base + (int64_t)X1w * N + X2[k];
-                        const float2 yk = k ? y1 : y0;
-                        float2 h = k ? make_float2(q.z, q.w) : make_float2(q.x, q.y);
-                        const float2 inc = make_float2(yk.y, -yk.x);
-                        if (a.compensated) {
-                            float2 l = a.lo[g];
-                            compensated_add(h.x, l.x, inc.x);
-                            compensated_add(h.y, l.y, inc.y);
-                            a.lo[g] = l;
-                        } else {
-                            h.x += inc.x;
-                            h.y += inc.y;
-                        }
-                        a.w_out[g] = h;
-                    }
-                }
-            }
+            prev[0] = P[i][0];
+            prev[1] = P[i][1];
+            const float4 q = Ql[i * 32];
+            P[i][0] = make_float2(fmaf(inv_j, y0.y, q.x), fmaf(-inv_j, y0.x, q.y));
+            P[i][1] = make_float2(fmaf(inv_j, y1.y, q.z), fmaf(-inv_j, y1.x, q.w));
         }
+    };
+#pragma unroll 1
+    for (int d = 1; d <= n_mid; ++d) {
+        exchange(d & 1);
+        const float inv_j = 1.0f / (float)(a.j0 - d + 1);
+        if (any_diag)
+            mid(std::true_type(), inv_j);
+        else
+            mid(std::false_type(), inv_j);
     }
     if (!a.final) {
         // the tile of the launch's last iterate
 #pragma unroll
         for (int i = 0; i < RL; ++i) {
-            const int ri = r0 + i;
-            if (ri < D || ri >= D + T || x1_0 + ri >= N) continue;
-            const int64_t grow = base + (int64_t)x_row[ri] * N;
+            if (!row_in(r0 + i)) continue;
+            float2 *g = a.w_out + base + (int64_t)x_row[r0 + i] * N;
+            if (vec) {
+                if (col_in[0])
+                    *reinterpret_cast<float4 *>(g + X2[0]) = make_float4(P[i][0].x, P[i][0].y, P[i][1].x, P[i][1].y);
+            } else {
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const int ck = 2 * lane + k;
-                if (ck >= D && ck < D + T2 && x2_0 + ck < N) a.w_out[grow + X2[k]] = P[i][k];
+                for (int k = 0; k < 2; ++k)
+                    if (col_in[k]) g[X2[k]] = P[i][k];
             }
+        }
+        return;
+    }
+    // the final stage: psi(t+dt) = psi + (-i) y on the tile, rounding error carried in lo
+    exchange(a.n_stages & 1);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    float2 prev[2] = {make_float2(u4.x, u4.y), make_float2(u4.z, u4.w)};
+    float2 rc = rowc[r0];
+#pragma unroll
+    for (int i = 0; i < RL; ++i) {
+        const float2 rn = rowc[r0 + i + 1];
+        float2 y0, y1;
+        reg_stencil_row<true>(P, i, prev, d4, rc, rn, ec, nJc, dU, diag, from_left, from_right, y0, y1);
+        rc = rn;
+        prev[0] = P[i][0];
+        prev[1] = P[i][1];
+        if (!row_in(r0 + i)) continue;
+        const float4 q = Ql[i * 32];
+        float2 h[2] = {make_float2(q.x, q.y), make_float2(q.z, q.w)};
+        const float2 inc[2] = {make_float2(y0.y, -y0.x), make_float2(y1.y, -y1.x)};
+        const int64_t g = base + (int64_t)x_row[r0 + i] * N;
+        float2 l[2] = {};
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (!col_in[k]) continue;
+            if (a.compensated) {
+                l[k] = los[lo_at + i * T2 + k];
+                compensated_add2(h[k], l[k], inc[k]);
+            } else {
+                h[k].x += inc[k].x;
+                h[k].y += inc[k].y;
+            }
+        }
+        if (vec) {
+            if (col_in[0]) {
+                if (a.compensated)
+                    *reinterpret_cast<float4 *>(a.lo + g + X2[0]) = make_float4(l[0].x, l[0].y, l[1].x, l[1].y);
+                *reinterpret_cast<float4 *>(a.w_out + g + X2[0]) = make_float4(h[0].x, h[0].y, h[1].x, h[1].y);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (col_in[k]) {
+                    if (a.compensated) a.lo[g + X2[k]] = l[k];
+                    a.w_out[g + X2[k]] = h[k];
+                }
         }
     }
 }
@@ -607,13 +756,13 @@ TiledShape tiled_shape() {
 
 template <int D, int W = 8>
 TiledShape tiled_reg_shape() {
-    constexpr int RS = 8 * W;
+    using Tile = RegTile<D, W>;
     TiledShape s;
-    s.TMAX = RS - 2 * D;
-    s.TMAX2 = 64 - 2 * D;
+    s.TMAX = Tile::T;
+    s.TMAX2 = Tile::T2;
     s.D = D;
     s.kern = taylor_tiled_reg_kernel<D, W>;
-    s.smem = sizeof(float4) * (RS * 32 + 2 * W * 2 * 32 + 32 + RS + 1) + sizeof(int) * RS;
+    s.smem = Tile::smem;
     s.fixed_tile = true;
     s.threads = 32 * W;
     return s;
@@ -673,13 +822,50 @@ int tiled_depth(int shape) {
     return tiled_shape_for(shape, s) ? s.D : 0;
 }
 
-int tiled_default_shape(int K) {
-    // the fewest launches a step at depth <= 8, with the stages split evenly
-    // between them (a larger tile for the same launch count)
-    const int launches = (K + 7) / 8;
-    const int D = (K + launches - 1) / launches;
-    static const int by_depth[9] = {4, 10, 5, 9, 3, 8, 7, 6, 4};
-    return by_depth[D < 1 ? 1 : (D > 8 ? 8 : D)];
+// The register tiles' depth (and region) for this handle and order: the
+// least of launches x tiles x (kTileFixed + 8 kRowStage stages), the warp
+// instructions of a tile, over the depths 1..8.  A tile costs a fixed part
+// (loads, coefficients, the compensated update) and its rows' stages; deeper
+// launches are fewer but leave a smaller tile, and where N is little more
+// than a whole number of tiles the next shallower one covers it with fewer.
+// The two constants are from the 64 x 64 tiles' counters at depths 8 and 4
+// (2918 and 2049 warp instructions a tile and warp).  Measured, K = 16
+// (site-updates/s at depths 8 / 4): N = 1024 5.16e11 / 5.02e11, N = 256
+// 4.20e11 / 4.43e11, N = 128 4.02e11 / 3.11e11, N = 100 2.45e11 / 3.73e11.
+// The 96 x 64 regions (depth 7 and 8 only) run at 0.94 of the rate a region
+// point and are taken where they save more than that: N = 1024 5.44e11,
+// N = 512 4.99e11 against 5.03e11.
+int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
+    static const int by_depth[9] = {4, 10, 5, 9, 3, 8, 7, 6, 4};   // 64 x 64 regions
+    constexpr double kTileFixed = 1180.0, kRowStage = 27.0, kTallRate = 0.94;
+    int best = by_depth[8];
+    double best_cost = 0.0;
+    auto consider = [&](int shape) {
+        TiledShape f;
+        if (!tiled_shape_for(shape, f)) return;
+        double tiles = 0.0;
+        for (size_t g = 0; g < h->group_N.size(); ++g) {
+            const int N = h->group_N[g];
+            tiles += (double)h->group_count[g] * ((N + f.TMAX - 1) / f.TMAX) * ((N + f.TMAX2 - 1) / f.TMAX2);
+        }
+        const int launches = (K + f.D - 1) / f.D;
+        double cost = tiles * (f.threads / 256.0) * (launches * kTileFixed + 8.0 * kRowStage * K);
+        if (f.threads > 256) cost /= kTallRate;
+        if (best_cost == 0.0 || cost < best_cost) {
+            best = shape;
+            best_cost = cost;
+        }
+    };
+    for (int d = 8; d >= 1; --d) {
+        // only depths that split the stages evenly: another one does the same
+        // launches on smaller tiles
+        const int launches = (K + d - 1) / d;
+        if ((K + launches - 1) / launches == d) consider(by_depth[d]);
+    }
+    const int launches = (K + 7) / 8, even = (K + launches - 1) / launches;
+    if (even == 8) consider(13);
+    if (even == 7) consider(14);
+    return best;
 }
 
 int launch_taylor_tiled_range(const ctqw_hamiltonian *h, int shape, const void *w_in, const void *psi,
@@ -715,6 +901,7 @@ int launch_taylor_tiled_range(const ctqw_hamiltonian *h, int shape, const void *
     a.n_stages = n_stages;
     a.final = final;
     a.compensated = compensated;
+    a.aligned16 = (((uintptr_t)w_in | (uintptr_t)psi | (uintptr_t)w_out | (uintptr_t)lo) & 15) == 0;
     CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)f.smem));
     const int G = (int)h->group_N.size();
