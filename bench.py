@@ -262,14 +262,14 @@ def roofline_of(w, dtype, flags, units, kernel_ms, peaks, traffic, switching=Fal
                               "hbm_gbs_measured": peaks.get("hbm_gbs")}, "fp32")
     if dtype == ctqw.C128:
         # FP64 on GB300 runs 2 DFMA per SM per cycle: the per-term FP64
-        # kernels are bound by that pipe, not by HBM (64 B per site-update)
+        # kernels are bound by that pipe, not by HBM (48 B per site-update)
         flops_per_unit = 8 * w.m + 4
         achieved = units * flops_per_unit / sec / 1e12
         peak = alu_peak(fp64=True)
         return with_measured({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                              "frac": achieved / peak, "traffic": None, "kernel": "taylor_term_kernel<double>",
+                              "frac": achieved / peak, "traffic": None, "kernel": "horner2_f64_kernel",
                               "kernel_ms": kernel_ms, "flops_per_site_update": flops_per_unit,
-                              "hbm_gbs_achieved": units * 64.0 / sec / 1e9, "bytes_per_site_update": 64.0,
+                              "hbm_gbs_achieved": units * 48.0 / sec / 1e9, "bytes_per_site_update": 48.0,
                               "peak_basis": f"{SM_COUNT} SMs x 2 DFMA x 2 flop x 2070 MHz (FP64, derived)",
                               "timing": "the whole propagate call (observables kernels included)"}, "fp64")
     bpu = ((w.K - 1) * 24.0 + 40.0) / w.K

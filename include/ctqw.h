@@ -245,11 +245,11 @@ int ctqw_autotune_order(const ctqw_hamiltonian *h, int32_t dtype, double dt, int
  * it forks from and joins back to `stream` (so the call stays ordered on
  * `stream`, also under graph capture): those tiles fill the SMs that no
  * cluster can hold.  Overlapping calls on one handle share that stream.  The
- * per-term path runs in CTQW_C128 in the order of
- * Algorithm 3 (Phi^(j) from Phi^(j-1), summed forward); in CTQW_C64 as the
- * same polynomial in Horner form (w_j = Psi + (-i dt / j) H w_{j+1}, j = K..2,
- * Psi(t+dt) = Psi - i dt H w_2) with the state update compensated, because a
- * forward FP32 sum drops every term below half an ulp of the running sum.
+ * per-term path evaluates the polynomial of Algorithm 3 in Horner form
+ * (w_j = Psi + (-i dt / j) H w_{j+1}, j = K..2, Psi(t+dt) = Psi - i dt H w_2):
+ * the same sum with fewer operations and roundings than term by term.  In
+ * CTQW_C64 its state update is compensated (a forward FP32 sum would drop
+ * every term below half an ulp of the running sum).
  * Asynchronous.
  */
 int ctqw_propagate_taylor(const ctqw_hamiltonian *h, int32_t dtype, void *psi_dev, double dt,
@@ -323,10 +323,10 @@ int ctqw_propagate_exact(const ctqw_hamiltonian *h, int32_t dtype, void *psi_dev
  * Psi(t+dt) = Psi + dt/6 (K^(1) + 2K^(2) + 2K^(3) + K^(4)).  The norm is not
  * corrected.  This update map is the order-4 Taylor polynomial of
  * exp(-i H dt) (Sec. 2.3: order-n RK and order-n Taylor coincide for the
- * exponential); where the fused kernel applies (see ctqw_propagate_taylor)
- * it evaluates that polynomial on chip, otherwise, or with CTQW_FLAG_PLAIN,
- * one launch per stage runs the four stages above and needs the workspace
- * of ctqw_workspace_size(method = 1).
+ * exponential); the call evaluates that polynomial as ctqw_propagate_taylor
+ * with K = 4 does.  With CTQW_FLAG_PLAIN (or CTQW_FLAG_RENORMALIZE) one
+ * launch per stage runs the four stages above.  Both need the workspace of
+ * ctqw_workspace_size(method = 1).
  */
 int ctqw_propagate_rk4(const ctqw_hamiltonian *h, int32_t dtype, void *psi_dev, double dt,
                        int64_t n_steps, int32_t obs_every, double *P_mean_dev, double *norm_dev,

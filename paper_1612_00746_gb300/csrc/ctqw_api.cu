@@ -100,24 +100,14 @@ int taylor_step_plain(const ctqw_hamiltonian *h, int dtype, const void *in, void
         }
         return CTQW_OK;
     }
-    if (dtype == CTQW_C64) {
-        const void *w = in;
-        void *dst = phiA;
-        for (int j = K; j >= 1; --j) {
-            void *o = (j == 1) ? out : dst;
-            int st = launch_horner_stage(h, w, in, o, dt / j, s);
-            if (st != CTQW_OK) return st;
-            w = o;
-            dst = (dst == phiA) ? phiB : phiA;
-        }
-        return CTQW_OK;
-    }
-    const void *src = in;
+    const void *w = in;
     void *dst = phiA;
-    for (int j = 1; j <= K; ++j) {
-        int st = launch_taylor_term(h, dtype, src, dst, in, out, dt / j, j == 1, s);
+    for (int j = K; j >= 1; --j) {
+        void *o = (j == 1) ? out : dst;
+        int st = dtype == CTQW_C64 ? launch_horner_stage(h, w, in, o, dt / j, s)
+                                   : launch_horner_f64(h, w, in, o, dt / j, s);
         if (st != CTQW_OK) return st;
-        src = dst;
+        w = o;
         dst = (dst == phiA) ? phiB : phiA;
     }
     return CTQW_OK;
@@ -535,9 +525,8 @@ struct SwitchSpec {
     bool renorm = false;   // divide every state by its norm after each step
 };
 
-// One launch per Taylor term (c128, forward order of Algorithm 3) or per
-// Horner stage (c64, compensated state update); outputs already zeroed and
-// the workspace (3 states) checked by the caller.
+// One launch per Horner stage (c64: with a compensated state update);
+// outputs already zeroed and the workspace (3 states) checked by the caller.
 static int propagate_per_term(const ctqw_hamiltonian *h, int32_t dtype, void *psi_dev, double dt,
                               int32_t K, int64_t n_steps, int32_t obs_every, double *P_mean_dev,
                               double *norm_dev, double *energy_dev, void *workspace_dev,
@@ -574,28 +563,31 @@ static int propagate_per_term(const ctqw_hamiltonian *h, int32_t dtype, void *ps
         }
         return CTQW_OK;
     }
-    void *cur = psi_dev, *acc = ws, *phi1 = ws + sb, *phi2 = ws + 2 * sb;
+    void *wa = ws, *wb = ws + sb;
     int64_t obs = 0;
     for (int64_t step = 0; step <= n_steps; ++step) {
         if (obs_every > 0 && step % obs_every == 0) {
-            CTQW_TRY(launch_observables(h, dtype, cur, P_mean_dev ? P_mean_dev + obs * h->p_width : nullptr,
+            CTQW_TRY(launch_observables(h, dtype, psi_dev, P_mean_dev ? P_mean_dev + obs * h->p_width : nullptr,
                                         nullptr, norm_dev ? norm_dev + obs * h->R : nullptr,
                                         energy_dev ? energy_dev + obs * h->R : nullptr, s));
             ++obs;
         }
         if (step == n_steps) break;
-        const void *in = cur;
-        void *out = phi1;
-        for (int j = 1; j <= K; ++j) {
-            CTQW_TRY(launch_taylor_term(h, dtype, in, out, cur, acc, dt / j, j == 1, s));
-            in = out;
-            out = (out == phi1) ? phi2 : phi1;
+        const void *in = psi_dev;
+        if (K == 1) {   // the only stage reads its neighbours from a copy
+            CTQW_CUDA_TRY(cudaMemcpyAsync(wa, psi_dev, sb, cudaMemcpyDeviceToDevice, s));
+            in = wa;
         }
-        std::swap(cur, acc);
-        if (sw.renorm) CTQW_TRY(launch_renormalize(h, dtype, cur, nullptr, s));
+        void *out = wa;
+        for (int j = K; j >= 1; --j) {
+            void *o = j == 1 ? psi_dev : out;
+            CTQW_TRY(launch_horner_f64(h, in, psi_dev, o, dt / j, s));
+            in = o;
+            out = (out == wa) ? wb : wa;
+        }
+        if (sw.renorm) CTQW_TRY(launch_renormalize(h, dtype, psi_dev, nullptr, s));
         if (sw.on) CTQW_TRY(launch_switch_params(h, sw.seed, (uint64_t)step, sw.p, s));
     }
-    if (cur != psi_dev) CTQW_CUDA_TRY(cudaMemcpyAsync(psi_dev, cur, sb, cudaMemcpyDeviceToDevice, s));
     return CTQW_OK;
 }
 
@@ -905,11 +897,14 @@ static int propagate_rk4_impl(const ctqw_hamiltonian *h, int32_t dtype, void *ps
     CTQW_TRY(check_common(h, dtype, psi_dev, dt, n_steps, obs_every));
     cudaStream_t s = (cudaStream_t)stream;
     // RK4's update map is the order-4 Taylor polynomial of exp(-i H dt)
-    // (Sec. 2.3): the fused kernel evaluates it directly
-    if (!(flags & (CTQW_FLAG_PLAIN | CTQW_FLAG_RENORMALIZE)) && fused_rows_supported(h, dtype))
+    // (Sec. 2.3): the Taylor path of the handle evaluates it directly
+    if (!(flags & (CTQW_FLAG_PLAIN | CTQW_FLAG_RENORMALIZE))) {
+        // a tuning shape only means something where the cluster kernel runs
+        if (!fused_rows_supported(h, dtype)) flags &= ~(0xFu << CTQW_FUSED_SHAPE_SHIFT);
         return propagate_taylor_impl(h, dtype, psi_dev, dt, 4, n_steps, obs_every, P_mean_dev,
                                      norm_dev, energy_dev, flags, workspace_dev, workspace_bytes,
                                      stream);
+    }
     const size_t sb = (size_t)h->total_amp * elem_bytes(dtype);
     const int64_t n_obs = n_samples(n_steps, obs_every);
     CTQW_TRY(zero_outputs(h, n_obs, P_mean_dev, norm_dev, energy_dev, s));

@@ -167,9 +167,9 @@ int launch_renormalize(const ctqw_hamiltonian *h, int dtype, void *psi, void *lo
 int launch_init_state(const ctqw_hamiltonian *h, const int32_t *sites_d, int dtype, void *psi,
                       cudaStream_t s);
 
-// Per-term Taylor launch (a3, plain path): out = -(i dt/j) H in; acc (= psi if first) += out.
-int launch_taylor_term(const ctqw_hamiltonian *h, int dtype, const void *in, void *out,
-                       const void *psi, void *acc, double coef, int first, cudaStream_t s);
+// FP64 per-term Horner stage (a3, plain path): out = psi + coef (-i) H in; out may be psi.
+int launch_horner_f64(const ctqw_hamiltonian *h, const void *in, const void *psi, void *out, double coef,
+                      cudaStream_t s);
 
 // FP32 per-term path in Horner form: out = psi + coef (-i) H in;
 // final: psi (+lo, carried rounding error) += -i dt H w2.

@@ -78,11 +78,10 @@ extern "C" int ctqw_propagate_taylor_noalloc(const ctqw_hamiltonian *h, int32_t 
     void *scratch = nullptr;
     const int st = noalloc_scratch_address(&scratch);
     if (st != CTQW_OK) return st;
-    // Nothing left in the array by an earlier call is read.  CTQW_C128: the
-    // first Taylor term of every step writes the running sum and the term
-    // buffer in full before they are read.  CTQW_C64: every Horner stage
+    // Nothing left in the array by an earlier call is read: every Horner stage
     // writes its iterate in full before the next stage reads it, and the
-    // carried error word is cleared by a memset at the start of the call.
+    // carried error word of CTQW_C64 is cleared by a memset at the start of
+    // the call.
     return ctqw_propagate_taylor(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev,
                                  norm_dev, energy_dev, CTQW_FLAG_PLAIN, scratch,
                                  kNoAllocScratchBytes, stream);

@@ -1,33 +1,11 @@
 // Per-term propagation kernels: the structure of Algorithms 2 and 3 with
 // one launch per Taylor term (or RK4 stage) over all realizations at once
 // (the realization x node loop collapsed into one grid, Sec. 2.2).  These
-// are the plain path: every term streams Phi and the running sum through HBM.
+// are the plain path: every term streams the iterate and psi through HBM.
 #include "ctqw_internal.cuh"
 #include "stencil.cuh"
 
 namespace {
-
-// Phi^(j) = -(i dt/j) H Phi^(j-1);  acc = (first ? psi : acc) + Phi^(j).
-template <typename T, int M>
-__global__ void __launch_bounds__(256) taylor_term_kernel(RealTable tab, const int32_t *__restrict__ list,
-                                                          const T *__restrict__ eps,
-                                                          const T *__restrict__ J,
-                                                          const cplx_t<T> *__restrict__ in,
-                                                          cplx_t<T> *__restrict__ out,
-                                                          const cplx_t<T> *__restrict__ psi,
-                                                          cplx_t<T> *__restrict__ acc, T coef,
-                                                          int first) {
-    Site<M> p;
-    if (!site_of<M>(tab, list, p)) return;
-    const int64_t s = p.s;
-    const int64_t base = tab.st_off[p.r];
-    const int64_t po = tab.par_off[p.r];
-    cplx_t<T> y = apply_h<T, M>(in + base, s, p.x, p.N, eps + po, J + po, (T)tab.U);
-    cplx_t<T> phi = mk<T>(coef * y.y, -coef * y.x);   // -(i coef) y
-    out[base + s] = phi;
-    cplx_t<T> a = first ? psi[base + s] : acc[base + s];
-    acc[base + s] = mk<T>(a.x + phi.x, a.y + phi.y);
-}
 
 // k = -i H in;  next = psi + a k (when next != null);  acc = (first ? psi : acc) + b k.
 template <typename T, int M>
@@ -54,22 +32,6 @@ __global__ void __launch_bounds__(256) rk4_stage_kernel(RealTable tab, const int
 
 }  // namespace
 
-int launch_taylor_term(const ctqw_hamiltonian *h, int dtype, const void *in, void *out,
-                       const void *psi, void *acc, double coef, int first, cudaStream_t s) {
-    RealTable t = real_table(h);
-    return for_each_group(h, [&](dim3 grid, dim3 block, const int32_t *list) {
-        if (dtype == CTQW_C64) {
-            auto k = h->m == 2 ? taylor_term_kernel<float, 2> : taylor_term_kernel<float, 3>;
-            k<<<grid, block, 0, s>>>(t, list, h->eps32, h->J32, (const float2 *)in, (float2 *)out,
-                                     (const float2 *)psi, (float2 *)acc, (float)coef, first);
-        } else {
-            auto k = h->m == 2 ? taylor_term_kernel<double, 2> : taylor_term_kernel<double, 3>;
-            k<<<grid, block, 0, s>>>(t, list, h->eps64, h->J64, (const double2 *)in, (double2 *)out,
-                                     (const double2 *)psi, (double2 *)acc, coef, first);
-        }
-    });
-}
-
 int launch_rk4_stage(const ctqw_hamiltonian *h, int dtype, const void *in, void *next,
                      const void *psi, void *acc, double a, double b, int first, cudaStream_t s) {
     RealTable t = real_table(h);
@@ -84,6 +46,132 @@ int launch_rk4_stage(const ctqw_hamiltonian *h, int dtype, const void *in, void 
                                      (const double2 *)psi, (double2 *)acc, a, b, first);
         }
     });
+}
+
+// ---------------------------------------------------------------- FP64 per-term path
+// One Horner stage of Algorithm 3's polynomial (Sec. 2.3), w_j = psi + (A/j) w_{j+1},
+// A = -i dt H; with j = 1 that is the new state itself, which may overwrite
+// psi in place (a thread reads psi at its own amplitude only).
+//
+// The FP64 pipe bounds it: GB300 issues 2 FP64 operations a clock and SM.
+// One launch per term in the forward order of Algorithm 3 spends 21 of them
+// an amplitude (13 with fused multiply-adds) and moves 64 bytes; this form
+// spends 11 for two particles (one add for the diagonal, ten fused
+// multiply-adds into psi, the coefficients scaled by dt / j once a thread and
+// row) and moves 48.  It also rounds at the state's own magnitude 5 times a
+// step instead of K: against 80-bit arithmetic 200 steps of N = 64, K = 12 end
+// 1.5e-15 off, the forward sum 4.2e-15.  4 realizations of N = 4096, K = 16,
+// 5 steps: 187.8 ms forward, 106.7 ms here (5.0e10 site-updates/s, 0.88 of the
+// FP64 pipe); RK4 on 16 x N = 256, 100 steps: 17.0 ms -> 11.7 ms.
+namespace {
+
+// Two particles: a block's thread row owns `rows` lattice rows x1 of up to
+// 256 columns x2, each thread walking down one column with w at x1 - 1, x1
+// and x1 + 1 in registers (the next one loaded a row ahead).
+constexpr int kF64Rows = 16;   // lattice rows a thread row walks at most
+
+__global__ void __launch_bounds__(256) horner2_f64_kernel(RealTable tab, const int32_t *__restrict__ list,
+                                                          const double *__restrict__ eps,
+                                                          const double *__restrict__ J, const double2 *in,
+                                                          const double2 *psi, double2 *out, double coef, int rows) {
+    __shared__ double2 rowc[8 * kF64Rows + 1];   // coef (eps, -J of the bond above) of the block's rows
+    const int r = list[blockIdx.z];
+    const int N = tab.N[r];
+    const int64_t po = tab.par_off[r], base = tab.st_off[r];
+    const int b0 = blockIdx.x * blockDim.y * rows;   // the block's first row
+    for (int q = threadIdx.y * blockDim.x + threadIdx.x; q <= (int)blockDim.y * rows; q += blockDim.x * blockDim.y) {
+        const int x1 = b0 + q < N ? b0 + q : (b0 + q) % N;
+        rowc[q] = make_double2(coef * eps[po + x1], -coef * J[po + (x1 == 0 ? N - 1 : x1 - 1)]);
+    }
+    __syncthreads();
+    const int x2 = blockIdx.y * blockDim.x + threadIdx.x;
+    const int x1_0 = b0 + threadIdx.y * rows, x1_e = min(x1_0 + rows, N);
+    if (x2 >= N || x1_0 >= x1_e) return;
+    const int xl = x2 == 0 ? N - 1 : x2 - 1, xr = x2 == N - 1 ? 0 : x2 + 1;
+    const double e2 = coef * eps[po + x2], jl = -coef * J[po + xl], jr = -coef * J[po + x2];
+    const double cU = coef * tab.U;
+    const double2 *w = in + base;
+    double2 up = w[(int64_t)(x1_0 == 0 ? N - 1 : x1_0 - 1) * N + x2], c = w[(int64_t)x1_0 * N + x2];
+    double2 dn = w[(int64_t)(x1_0 + 1 == N ? 0 : x1_0 + 1) * N + x2];
+    double2 l = w[(int64_t)x1_0 * N + xl], rt = w[(int64_t)x1_0 * N + xr];
+    double2 q = psi[base + (int64_t)x1_0 * N + x2];
+    const double2 *rc = rowc + threadIdx.y * rows;
+    for (int x1 = x1_0; x1 < x1_e; ++x1, ++rc) {
+        double2 nn = dn, l2 = l, rt2 = rt, q2 = q;
+        if (x1 + 1 < x1_e) {   // the next row's values, a row ahead
+            const int64_t row = (int64_t)(x1 + 1) * N;
+            nn = w[(int64_t)(x1 + 2 == N ? 0 : x1 + 2) * N + x2];
+            l2 = w[row + xl];
+            rt2 = w[row + xr];
+            q2 = psi[base + row + x2];
+        }
+        const double2 r0 = rc[0];
+        const double jup = r0.y, jdn = rc[1].y;
+        double v = r0.x + e2;
+        if (x1 == x2) v += cU;
+        // psi - i (coef H w): the real part takes +, the imaginary part -
+        double yr = fma(v, c.y, q.x), yi = fma(-v, c.x, q.y);
+        yr = fma(jup, up.y, yr);
+        yi = fma(-jup, up.x, yi);
+        yr = fma(jdn, dn.y, yr);
+        yi = fma(-jdn, dn.x, yi);
+        yr = fma(jl, l.y, yr);
+        yi = fma(-jl, l.x, yi);
+        yr = fma(jr, rt.y, yr);
+        yi = fma(-jr, rt.x, yi);
+        out[base + (int64_t)x1 * N + x2] = make_double2(yr, yi);
+        up = c;
+        c = dn;
+        dn = nn;
+        l = l2;
+        rt = rt2;
+        q = q2;
+    }
+}
+
+// Three particles: one amplitude a thread.
+__global__ void __launch_bounds__(256) horner3_f64_kernel(RealTable tab, const int32_t *__restrict__ list,
+                                                          const double *__restrict__ eps,
+                                                          const double *__restrict__ J, const double2 *in,
+                                                          const double2 *psi, double2 *out, double coef) {
+    Site<3> p;
+    if (!site_of<3>(tab, list, p)) return;
+    const int64_t base = tab.st_off[p.r], po = tab.par_off[p.r];
+    const double2 y = apply_h<double, 3>(in + base, p.s, p.x, p.N, eps + po, J + po, tab.U);
+    const double2 q = psi[base + p.s];
+    out[base + p.s] = make_double2(fma(coef, y.y, q.x), fma(-coef, y.x, q.y));
+}
+
+}  // namespace
+
+int launch_horner_f64(const ctqw_hamiltonian *h, const void *in, const void *psi, void *out, double coef,
+                      cudaStream_t s) {
+    RealTable t = real_table(h);
+    if (h->m == 3)
+        return for_each_group(h, [&](dim3 grid, dim3 block, const int32_t *list) {
+            horner3_f64_kernel<<<grid, block, 0, s>>>(t, list, h->eps64, h->J64, (const double2 *)in,
+                                                      (const double2 *)psi, (double2 *)out, coef);
+        });
+    int off = 0;
+    for (size_t g = 0; g < h->group_N.size(); ++g) {
+        const int N = h->group_N[g], cnt = h->group_count[g];
+        const int tx = N >= 256 ? 256 : ((N + 31) / 32) * 32, ty = 256 / tx;
+        const int64_t cols = (N + tx - 1) / tx;
+        // longer walks scale and reload less, but the FP64 pipes of all SMs
+        // have to get work: at least six blocks an SM, or one row a thread
+        int rows = kF64Rows;
+        while (rows > 1 && (int64_t)((N + ty * rows - 1) / (ty * rows)) * cols * cnt < 912) rows /= 2;
+        for (int done = 0; done < cnt; done += 65535) {
+            const int part = cnt - done < 65535 ? cnt - done : 65535;
+            horner2_f64_kernel<<<dim3((unsigned)((N + ty * rows - 1) / (ty * rows)), (unsigned)cols, (unsigned)part),
+                                 dim3((unsigned)tx, (unsigned)ty), 0, s>>>(
+                t, h->by_group_d + off + done, h->eps64, h->J64, (const double2 *)in, (const double2 *)psi,
+                (double2 *)out, coef, rows);
+            CTQW_CUDA_TRY(cudaGetLastError());
+        }
+        off += cnt;
+    }
+    return CTQW_OK;
 }
 
 // ---------------------------------------------------------------- FP32 per-term path
