@@ -227,19 +227,20 @@ int ctqw_autotune_order(const ctqw_hamiltonian *h, int32_t dtype, double dt, int
  * Precision: CTQW_C128 propagates in FP64; CTQW_C64 propagates in FP32 and
  * carries the rounding error of every state update in a second FP32 word
  * (compensated summation).
- * Path: m = 2 chains with N a multiple of 64 up to 256 in CTQW_C64 run the
- * fused cluster kernel (every Taylor term of every step on chip; halo rows move between the CTAs
+ * Path: m = 2 chains of one size N <= 256 in CTQW_C64 (rings: N a multiple
+ * of 4 that 2, 4, 6 or 8 adjacent columns on at most 32 lanes cover exactly)
+ * run the fused cluster kernel (every Taylor term of every step on chip; halo rows move between the CTAs
  * of a cluster point to point, see ctqw_check_status); other m = 2 handles
- * in CTQW_C64 (N > 256, ragged sizes) run the temporally blocked tiled
- * kernel with the iterate in registers, ceil(K / 8) launches a step with the
- * stages split evenly between them; everything
+ * in CTQW_C64 (N > 256, ragged sizes, other rings) run the temporally blocked
+ * tiled kernel with the iterate in registers, at the tile and depth that
+ * cost the fewest instructions; everything
  * else, or CTQW_FLAG_PLAIN, runs one launch per Taylor term.  Every path
  * needs the workspace of ctqw_workspace_size (3 states).  The fused path
  * keeps the carried error in the first state and stores the state at
  * sample points into the others (S = workspace_bytes / state bytes - 1
  * slots); one launch covers S + 1 sampling intervals, so a larger
  * workspace means fewer launches.  Given no workspace, the fused path
- * allocates its 3 states stream-ordered.  With S >= 2 and enough
+ * allocates its 3 states stream-ordered (N a multiple of 64 only).  With S >= 2 and enough
  * realizations, the fused path also runs the last ctqw_fused_split
  * realizations on the register tiles, on a second stream of the handle that
  * it forks from and joins back to `stream` (so the call stays ordered on

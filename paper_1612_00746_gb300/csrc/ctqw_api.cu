@@ -337,6 +337,7 @@ int ctqw_build_hamiltonian(const ctqw_lattice_desc *d, void *stream, ctqw_hamilt
         cudaMemcpyAsync(h->J64_0, h->J64, pb, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return fail(CTQW_ECUDA);
     if (fused_rows_supported(h, CTQW_C64)) {
+        if ((st = plan_fused_rows(h))) return fail(st);
         // the fused path's second stream, at the lowest priority so that the
         // clusters go first when both have work waiting
         int least = 0, greatest = 0;
@@ -779,19 +780,21 @@ static int propagate_taylor_impl(const ctqw_hamiltonian *h, int32_t dtype, void 
                                energy_dev, flags, tiled_public[shape - CTQW_SHAPE_TILED(0)],
                                workspace_dev, workspace_bytes, s);
     }
-    const bool fused = !(flags & CTQW_FLAG_PLAIN) && fused_rows_supported(h, dtype);
+    // the cluster kernel takes every uniform N it can lay out; the tuning
+    // shapes and a missing workspace only go with the sizes of the banded kernel
+    const bool tuned_size = fused_taylor_supported(h, dtype);
+    const bool fused = !(flags & CTQW_FLAG_PLAIN) && fused_rows_supported(h, dtype) && (tuned_size || shape == 0);
     // two particles in FP32 that the cluster-resident kernel cannot hold
-    // (N > 256, ragged sizes, other N): the temporally blocked tiled kernel
-    // with the iterate in registers, at the depth that needs the fewest
-    // launches a step (depth 8 was the fastest measured of 2, 4, 8)
+    // (N > 256, ragged sizes, some rings): the temporally blocked tiled kernel
+    // with the iterate in registers, at the region and depth of least cost
     if (!fused && !(flags & CTQW_FLAG_PLAIN) && shape == 0 && tiled_supported(h, dtype, tiled_default_shape(h, K)))
         return propagate_tiled(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,
                                energy_dev, flags, tiled_default_shape(h, K), workspace_dev,
                                workspace_bytes, s);
-    if (!fused) {
+    if (!fused || !tuned_size) {
         const size_t need = 3 * (size_t)h->total_amp * elem_bytes(dtype);
         if (!workspace_dev || workspace_bytes < need) {
-            ctqw_set_error("plain path needs a workspace of %zu bytes (got %zu)", need, workspace_bytes);
+            ctqw_set_error("this path needs a workspace of %zu bytes (got %zu)", need, workspace_bytes);
             return CTQW_EINVAL;
         }
     }
@@ -899,8 +902,8 @@ static int propagate_rk4_impl(const ctqw_hamiltonian *h, int32_t dtype, void *ps
     // RK4's update map is the order-4 Taylor polynomial of exp(-i H dt)
     // (Sec. 2.3): the Taylor path of the handle evaluates it directly
     if (!(flags & (CTQW_FLAG_PLAIN | CTQW_FLAG_RENORMALIZE))) {
-        // a tuning shape only means something where the cluster kernel runs
-        if (!fused_rows_supported(h, dtype)) flags &= ~(0xFu << CTQW_FUSED_SHAPE_SHIFT);
+        // a tuning shape only means something at the sizes that have them
+        if (!fused_taylor_supported(h, dtype)) flags &= ~(0xFu << CTQW_FUSED_SHAPE_SHIFT);
         return propagate_taylor_impl(h, dtype, psi_dev, dt, 4, n_steps, obs_every, P_mean_dev,
                                      norm_dev, energy_dev, flags, workspace_dev, workspace_bytes,
                                      stream);

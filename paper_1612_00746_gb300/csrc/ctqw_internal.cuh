@@ -44,6 +44,9 @@ struct ctqw_hamiltonian {
     double *renorm_d = nullptr;     // [R] norms of the per-step renormalization
     int32_t *sites_d = nullptr;     // [R][m] initial sites (ctqw_init_state)
     double norm_drift_tol = 0.0;    // norm check: |norm - norm at step 0| above this fails (0: finiteness only)
+    // the cluster kernel's layout for this handle (plan_fused_rows, at the
+    // build): warps a CTA, CTAs a cluster, resident clusters, CTAs an SM
+    int rows_W = 0, rows_C = 0, rows_clusters = 0, rows_per_sm = 0;
     int density_method = 0;         // one-body density: 0 tensor cores where supported, 1 CUDA cores
     // second stream of the fused path (the realizations on the SMs that hold
     // no cluster) and the events that fork it from and join it to the caller's
@@ -248,6 +251,9 @@ int launch_group_sum(const ctqw_hamiltonian *h, const double *grad, double *out,
 // clusters take the realizations one at a time from the handle's ticket
 // counter (work_counter), which the launch zeroes on its stream.
 bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype);
+// Picks the split of a lattice over warps, CTAs and the cluster for the
+// handle's N and R (rows_* of the handle); a no-op where the kernel does not apply.
+int plan_fused_rows(ctqw_hamiltonian *h);
 // How many realizations (the last ones) to run on the register tiles on the
 // handle's side stream while the clusters run the rest: the SMs that hold no
 // cluster (a 16-CTA cluster needs 8 SMs of one GPC) take a share matched to

@@ -48,6 +48,16 @@ static __device__ __forceinline__ void mbar_init(uint32_t mb, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(count) : "memory");
 }
 
+static __device__ __forceinline__ void mbar_arrive(uint32_t mb) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mb) : "memory");
+}
+
+// One arrival per warp, from its first lane (no branch).
+static __device__ __forceinline__ void mbar_arrive_lane0(uint32_t mb, int lane) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, %1, 0;\n\t"
+                 "@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(mb), "r"(lane) : "memory");
+}
+
 static __device__ __forceinline__ void mbar_expect_tx(uint32_t mb, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(bytes)
                  : "memory");
@@ -62,6 +72,12 @@ static __device__ __forceinline__ void mbar_expect_tx2_if(uint32_t mb0, uint32_t
 }
 
 // 16-byte store into another CTA's shared memory, counted on its mbarrier.
+static __device__ __forceinline__ void st_async16(uint32_t raddr, unsigned long long lo, unsigned long long hi,
+                                                  uint32_t rmbar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];"
+                 ::"r"(raddr), "l"(lo), "l"(hi), "r"(rmbar) : "memory");
+}
+
 static __device__ __forceinline__ void st_async16(uint32_t raddr, float4 v, uint32_t rmbar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                  ::"r"(raddr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(rmbar) : "memory");
@@ -99,6 +115,42 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t mb, uint32_t parity,
 static __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mb, uint32_t parity,
                                                   unsigned long long limit_ns, int *status) {
     return mbar_try_wait(mb, parity) || mbar_wait_slow(mb, parity, limit_ns, status);
+}
+
+// An (re, im) pair of FP32 values in one 64-bit register pair.  The stencil
+// loops keep amplitudes in this form from load to store: as float2 members
+// the compiler re-packs an amplitude for every FFMA2 that uses it, which
+// measured 5 to 6 register moves an amplitude and stage.
+using pair_t = unsigned long long;
+
+static __device__ __forceinline__ pair_t pack2(float x, float y) {
+    pair_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+
+static __device__ __forceinline__ float2 unpack2(pair_t v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+
+static __device__ __forceinline__ pair_t fma2(pair_t a, pair_t b, pair_t c) {
+    pair_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+static __device__ __forceinline__ pair_t mul2(pair_t a, pair_t b) {
+    pair_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// psi + (-i c) y, the Horner update of one amplitude
+static __device__ __forceinline__ pair_t horner2(pair_t psi, pair_t y, float c) {
+    const float2 q = unpack2(psi), v = unpack2(y);
+    return pack2(fmaf(c, v.y, q.x), fmaf(-c, v.x, q.y));
 }
 
 static __device__ __forceinline__ float2 ffma2(float a, float2 b, float2 c) {

@@ -7,15 +7,18 @@
 // once, and each takes realization after realization from a ticket counter,
 // so the SMs a cluster holds stay its own until the launch ends.
 // The N x N tile is split into row slabs, one per CTA; every warp owns RL
-// whole rows and each lane CL = N/32 adjacent columns of them, so a warp
+// whole rows and each lane CL adjacent columns of them (N <= 32 CL), so a warp
 // covers full rows: neighbours along x2 are in the lane's registers or one
-// 64-bit rotate-shuffle away (the rotation wraps from column N-1 to 0, which
-// is the ring's bond and is multiplied by J[N-1] = 0 on an open chain).
+// 64-bit rotate-shuffle away.  The rotation runs over the lanes that hold
+// columns and wraps from column N-1 to 0, which is the ring's bond and is
+// multiplied by J[N-1] = 0 on an open chain; rings therefore need CL and RL
+// to divide N, open chains pad rows and columns with zeros behind bonds that
+// are zero.
 // Neighbours along x1 are in registers except for the warp's first and last
-// rows, which come from the adjacent warps through shared memory (one
-// __syncthreads per stage) or, at the slab's edges, are pushed by the
-// neighbour CTAs straight into this CTA's shared memory with st.async on an
-// mbarrier (bounded waits).
+// rows, which come from the adjacent warps through shared memory (an mbarrier
+// of the CTA's warps) or, at the slab's edges, are pushed by the neighbour
+// CTAs straight into this CTA's shared memory with st.async on an mbarrier
+// (bounded waits).
 //
 // Arithmetic: the same polynomial in Horner form with A = -i dt H applied to
 // (re, im) pairs with FFMA2:
@@ -26,12 +29,26 @@
 // of a row that owns the diagonal.  The increment A w_2 is added to the state
 // with its rounding error carried in a second FP32 word (lo), so hi + lo
 // holds the state to ~2^-48 relative.  lo sits in shared memory for the
-// launch (lane-major like hi) and in a state-sized buffer between launches.
+// launch and in a state-sized buffer between launches.
 //
-// Control flow: the diagonal offset of a warp's rows is fixed for the
-// kernel, and the Horner stages of a step are K - 1 middle stages and one
-// final one, so the step loop is compiled per offset with the stage mode a
-// compile-time constant: no per-stage dispatch.
+// What bounds it: the FP32 pipe takes 14 cycles an amplitude and warp (6
+// FFMA2 of two cycles, 2 FFMA); everything else is latency.  psi of the step
+// stays in registers beside the iterate (reading it from shared memory every
+// stage took half of that pipe), and the exchange of edge rows is hidden: a
+// stage publishes its edge rows, computes the rows between them into spare
+// registers, and only then waits for the neighbours' rows.  Two stages
+// alternate between the two register sets of the inner rows, so nothing is
+// moved between them.  Measured against psi in shared memory and a block
+// barrier a stage (K = 16, site-updates/s, one stream): N = 64 1.17e12 ->
+// 1.23e12, N = 128 1.27e12 -> 1.33e12, N = 192 1.01e12 -> 1.23e12, N = 256
+// 9.1e11 -> 1.11e12; N = 100, on the register tiles before, 4.4e11 -> 7.6e11;
+// one realization of N = 64, 10 steps: 129 us -> 76 us.
+//
+// Control flow: the stages of a step are a first one (from psi), middle ones
+// in pairs and a final one, with no per-stage dispatch.  A row tests the few
+// columns that the diagonal x1 = x2 can meet it in; a step loop compiled per
+// offset of the diagonal had the warps of an SM run different copies of it
+// and wait for instructions.
 //
 // Observables are not formed here.  At every snap_every-th step inside the
 // launch the kernel stores the state to a snapshot slot (row-major, the
@@ -39,12 +56,6 @@
 // observables kernel; a launch covers the steps between a sample and the
 // sample after its last snapshot.  Keeping that work out of the kernel
 // leaves the registers of the Horner loop to the stencil.
-//
-// Row layout in shared memory (and of the carried error in global memory):
-// lane-major, the k-th column pair of lane l at float4 slot (k/2)*32 + l of
-// the row, so that every 16-byte access of a warp touches 32 consecutive
-// slots (a plain row-major layout puts lanes CL*8 bytes apart, a 4-way bank
-// conflict for CL = 8).  Every reader uses the writer's lane mapping.
 #include <algorithm>
 #include <type_traits>
 
@@ -62,10 +73,12 @@ struct RowsArgs {
     const double *J;
     RealTable tab;
     float2 *psi;            // state in (start of the launch) and out (end)
-    float2 *lo;             // carried rounding error (lane-major rows), in and out
+    float2 *lo;             // carried rounding error, in and out
     float2 *snap;           // snapshot slots (states), or null
     double dt;
     float dtU;
+    int N, W;               // lattice sites; warps a CTA
+    int vec;                // rows of every buffer can be accessed 16 bytes at a time
     int K;
     long long n_steps;      // steps of this launch
     int snap_every;         // snapshot after every snap_every-th step (< n_steps), 0: none
@@ -79,120 +92,73 @@ struct RowsArgs {
     float inv_j[kMaxK + 1];
 };
 
-enum { kHorner = 0, kFinal = 1 };
-
-// Register state of one lane: RL rows x CL columns of the Horner iterate and
-// the per-column coefficient pairs (c, c) of dt H.  The per-row pairs are the
-// same for the whole warp and are read from shared memory (rowc) instead.
-template <int CL, int RL>
-struct Lane {
-    float2 P[RL][CL];
-    float2 ec[CL];        // dt eps_x2 per column
-    float2 nJc[CL + 1];   // -dt J of the bond left of column k (k = CL: right of the last)
-};
-
-// One stencil application y = (dt H) P on the lane's block, then
-//   kHorner: P <- Q + (-i/j) y;  kFinal: P <- -i y.
-// usrc/dsrc: the rows above the first and below the last row in shared memory
-// (this lane's first column), read when needed so they do not hold registers.
-// Q: psi of the step in shared memory (this lane's first element, row stride N).
-// OFF = (first row) mod CL, which fixes where the diagonal x1 = x2 falls.
-// rowc: per slab row (dt eps_x1, dt eps_x1, -dt J above, -dt J above) for this
-// warp's rows and the one below them (broadcast loads).
-template <int MODE, int CL, int RL, int N, int OFF>
-__device__ __forceinline__ void stage(Lane<CL, RL> &L, const float4 *__restrict__ rowc,
-                                      const float2 *__restrict__ usrc,
-                                      const float2 *__restrict__ dsrc, const float2 *__restrict__ Q,
-                                      int lane, int x1_0, float dtU, float inv_j) {
-    const int from_left = (lane + 31) & 31, from_right = (lane + 1) & 31;
-    const float2 dU = make_float2(dtU, dtU);
-    float4 rc = rowc[0];
-    float2 prev[CL];   // old row above the current one
+// y = dt H of one row of a warp from its values c and the rows up and dn.
+// rc, rn: (dt eps, -dt J above) of the row and of the one below it.  dt U on
+// x1 = x2: row I of the warp meets it in the lane's column I + d, d = x1 - x2
+// of the lane's first column and the warp's first row, a multiple of
+// gcd(4, CL); dU holds dt U for the d of this lane and zeros for the others.
+template <int CL, int I>
+__device__ __forceinline__ void stencil_row(const pair_t (&ec)[CL], const pair_t (&nJc)[CL + 1], float2 rc, float2 rn,
+                                            const pair_t (&up)[CL], const pair_t (&c)[CL], const pair_t (&dn)[CL],
+                                            const pair_t (&dU)[4], int from_left, int from_right,
+                                            pair_t (&y)[CL]) {
+    const pair_t er = pack2(rc.x, rc.x), jup = pack2(rc.y, rc.y), jdn = pack2(rn.y, rn.y);
+    const pair_t lft = __shfl_sync(0xffffffffu, c[CL - 1], from_left), rgt = __shfl_sync(0xffffffffu, c[0], from_right);
 #pragma unroll
-    for (int k = 0; k < CL; k += 2) {
-        const float4 u4 = *reinterpret_cast<const float4 *>(usrc + k * 32);
-        prev[k] = make_float2(u4.x, u4.y);
-        prev[k + 1] = make_float2(u4.z, u4.w);
-    }
+    for (int k = 0; k < CL; ++k) y[k] = mul2(ec[k], c[k]);
 #pragma unroll
-    for (int i = 0; i < RL; ++i) {
-        float2 c[CL];
+    for (int k = 0; k < CL; ++k) y[k] = fma2(er, c[k], y[k]);
 #pragma unroll
-        for (int k = 0; k < CL; ++k) c[k] = L.P[i][k];
-        const float2 lft = shfl2(c[CL - 1], from_left);
-        const float2 rgt = shfl2(c[0], from_right);
-        float2 dn[CL];   // old row below (read from shared memory for the last row)
-        if (i == RL - 1) {
+    for (int k = 0; k < CL; ++k) y[k] = fma2(jup, up[k], y[k]);
 #pragma unroll
-            for (int k = 0; k < CL; k += 2) {
-                const float4 d4 = *reinterpret_cast<const float4 *>(dsrc + k * 32);
-                dn[k] = make_float2(d4.x, d4.y);
-                dn[k + 1] = make_float2(d4.z, d4.w);
-            }
-        }
-        const float4 rn = rowc[i + 1];
-        const float2 er = make_float2(rc.x, rc.y), jup = make_float2(rc.z, rc.w);
-        const float2 jdn = make_float2(rn.z, rn.w);
-        rc = rn;
-        float2 y[CL];
+    for (int k = 0; k < CL; ++k) y[k] = fma2(jdn, dn[k], y[k]);
 #pragma unroll
-        for (int k = 0; k < CL; ++k) {
-            const float2 nb = (i < RL - 1) ? L.P[i + 1][k] : dn[k];   // old row below
-            const float2 l = (k == 0) ? lft : c[k - 1];
-            const float2 r = (k == CL - 1) ? rgt : c[k + 1];
-            float2 t = __fmul2_rn(L.ec[k], c[k]);
-            t = __ffma2_rn(er, c[k], t);
-            t = __ffma2_rn(jup, prev[k], t);
-            t = __ffma2_rn(jdn, nb, t);
-            t = __ffma2_rn(L.nJc[k], l, t);
-            t = __ffma2_rn(L.nJc[k + 1], r, t);
-            y[k] = t;
-        }
-        // dt U on the diagonal x2 = x1: column (OFF + i) % CL of the lane (x1_0 + i) / CL
-        {
-            const int kd = (OFF + i) % CL;   // a constant once the row loop is unrolled
-            if (lane == (x1_0 + i) / CL) y[kd] = __ffma2_rn(dU, c[kd], y[kd]);
-        }
-        if (MODE == kHorner) {
+    for (int k = 0; k < CL; ++k) y[k] = fma2(nJc[k], k == 0 ? lft : c[k == 0 ? 0 : k - 1], y[k]);
 #pragma unroll
-            for (int k = 0; k < CL; k += 2) {
-                const float4 q = *reinterpret_cast<const float4 *>(Q + i * N + k * 32);
-                L.P[i][k] = make_float2(fmaf(inv_j, y[k].y, q.x), fmaf(-inv_j, y[k].x, q.y));
-                L.P[i][k + 1] = make_float2(fmaf(inv_j, y[k + 1].y, q.z), fmaf(-inv_j, y[k + 1].x, q.w));
-            }
-        } else if (MODE == kFinal) {
+    for (int k = 0; k < CL; ++k) y[k] = fma2(nJc[k + 1], k == CL - 1 ? rgt : c[k == CL - 1 ? k : k + 1], y[k]);
+    constexpr int G = CL % 4 == 0 ? 4 : 2;
 #pragma unroll
-            for (int k = 0; k < CL; ++k) L.P[i][k] = make_float2(y[k].y, -y[k].x);
-        }
-#pragma unroll
-        for (int k = 0; k < CL; ++k) prev[k] = c[k];
-    }
+    for (int k = I % G; k < CL; k += G) y[k] = fma2(dU[(k - I + 2) / 2], c[k], y[k]);
 }
 
-// CL columns per lane (N = 32 CL), RL rows per warp, W warps per CTA.
-template <int CL, int RL, int W, int MINB>
-__global__ void __launch_bounds__(32 * W, MINB) taylor_fused_rows_kernel(const __grid_constant__ RowsArgs a) {
-    constexpr int N = 32 * CL;
-    constexpr int SR = RL * W;     // slab rows
-    constexpr int C = N / SR;      // CTAs per cluster
-    static_assert(N % SR == 0 && C >= 1 && C <= 16 && CL % 2 == 0, "unsupported shape");
+// out <- Q + (-i / j) y
+template <int CL>
+__device__ __forceinline__ void horner_row(pair_t (&out)[CL], const pair_t (&Q)[CL], const pair_t (&y)[CL], float inv_j) {
+#pragma unroll
+    for (int k = 0; k < CL; ++k) out[k] = horner2(Q[k], y[k], inv_j);
+}
+
+// CL columns per lane (N <= 32 CL), 4 rows a warp, up to MAXW warps a CTA.
+template <int CL, int MAXW>
+__global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const __grid_constant__ RowsArgs a) {
+    constexpr int RL = 4;
+    constexpr int RQ = 16 * CL;       // float4 (column pairs) a row in shared memory, lane-major
+    const int N = a.N, W = a.W, SR = RL * W;
+    const int units = (N + RL - 1) / RL;              // warps' row blocks of the lattice
+    const int C = (units + W - 1) / W;                // CTAs per cluster
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *hi = reinterpret_cast<float2 *>(smem_raw);      // [SR][N] psi of the step
-    float2 *halo = hi + SR * N;                             // [2 parity][2: above, below][N]
-    float2 *edge = halo + 2 * 2 * N;                        // [2 parity][W][2: first, last][N]
-    float4 *rowc = reinterpret_cast<float4 *>(edge + 2 * W * 2 * N);  // [SR + 1] row coefficient pairs
-    float2 *los = reinterpret_cast<float2 *>(rowc + SR + 1);          // [SR][N] carried error, lane-major
-    __shared__ __align__(8) unsigned long long mbar[2][2];
+    float4 *halo = reinterpret_cast<float4 *>(smem_raw);    // [2 parity][2: above, below][RQ]
+    float4 *edge = halo + 2 * 2 * RQ;                       // [2 parity][W][2: first, last][RQ]
+    float4 *los = edge + 2 * W * 2 * RQ;                    // [SR][RQ] carried error
+    float2 *rowc = reinterpret_cast<float2 *>(los + SR * RQ);   // [SR + 1] (dt eps, -dt J of the bond above)
+    __shared__ __align__(8) unsigned long long mbar[2][2];      // halo rows: [parity][above, below]
+    __shared__ __align__(8) unsigned long long mbar_edge;       // the CTA's warps have published a stage
     __shared__ __align__(8) unsigned long long mbar_never;
     __shared__ int next_r;
 
     const int rank = (int)cluster_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int unit = rank * W + warp;
+    const bool active = unit < units;                       // the last CTA may have idle warps
+    const int my_warps = min(W, units - rank * W);          // warps of this CTA that hold rows
+    const bool top = warp == 0, bottom = warp == my_warps - 1;
     const int lrow0 = warp * RL;
-    const int x1_0 = rank * SR + lrow0;
+    const int x1_0 = unit * RL;
     const int x2_0 = lane * CL;
+    const int lanes = (N + CL - 1) / CL;                    // lanes that hold columns
+    const int from_left = lane == 0 ? lanes - 1 : lane - 1, from_right = lane + 1 >= lanes ? 0 : lane + 1;
 
-    Lane<CL, RL> L;
+    pair_t P[RL][CL], Q[RL][CL], T[2][CL], ec[CL], nJc[CL + 1];
     // coefficients and state of realization r (every warp reads rowc, so the
     // caller orders this behind the previous realization's last stage)
     auto load_realization = [&](const int r) {
@@ -200,73 +166,85 @@ __global__ void __launch_bounds__(32 * W, MINB) taylor_fused_rows_kernel(const _
         const double *eps = a.eps + po, *J = a.J + po;
         const double dt = a.dt;
         for (int q = threadIdx.x; q <= SR; q += blockDim.x) {
-            const int x1 = rank * SR + q;   // q = SR: only the bond below the slab is used
-            const float e = q < SR ? (float)(dt * eps[x1]) : 0.f;
-            const float j = (float)(-dt * J[(x1 - 1 + N) % N]);
-            rowc[q] = make_float4(e, e, j, j);
+            const int x1 = rank * SR + q;
+            const float e = x1 < N ? (float)(dt * eps[x1]) : 0.f;
+            // the bond above row x1 (x1 = N: the ring's, below the last row)
+            const float j = x1 <= N ? (float)(-dt * J[x1 == 0 ? N - 1 : x1 - 1]) : 0.f;
+            rowc[q] = make_float2(e, j);
         }
 #pragma unroll
         for (int k = 0; k < CL; ++k) {
-            const float v = (float)(dt * eps[x2_0 + k]);
-            L.ec[k] = make_float2(v, v);
+            const float v = x2_0 + k < N ? (float)(dt * eps[x2_0 + k]) : 0.f;
+            ec[k] = pack2(v, v);
         }
 #pragma unroll
-        for (int k = 0; k <= CL; ++k) {
-            const float v = (float)(-dt * J[(x2_0 + k - 1 + N) % N]);
-            L.nJc[k] = make_float2(v, v);
+        for (int k = 0; k <= CL; ++k) {   // left of column x2_0 + k (N: the ring's)
+            const int x = x2_0 + k;
+            const float v = x2_0 < N && x <= N ? (float)(-dt * J[x == 0 ? N - 1 : x - 1]) : 0.f;
+            nJc[k] = pack2(v, v);
         }
-        // state in: hi = psi (shared), P = psi (registers), lo (shared, lane-major like hi)
-        const float2 *glo = a.lo + a.tab.st_off[r];
+        const int64_t base = a.tab.st_off[r];
 #pragma unroll
         for (int i = 0; i < RL; ++i) {
-#pragma unroll
-            for (int k = 0; k < CL; k += 2)
-                *reinterpret_cast<float4 *>(los + (lrow0 + i) * N + lane * 2 + k * 32) =
-                    *reinterpret_cast<const float4 *>(glo + (size_t)(x1_0 + i) * N + lane * 2 + k * 32);
-        }
-#pragma unroll
-        for (int i = 0; i < RL; ++i) {
+            const int64_t g = base + (int64_t)(x1_0 + i) * N + x2_0;
 #pragma unroll
             for (int k = 0; k < CL; k += 2) {
-                const float4 v = *reinterpret_cast<const float4 *>(a.psi + a.tab.st_off[r] + (size_t)(x1_0 + i) * N + x2_0 + k);
-                L.P[i][k] = make_float2(v.x, v.y);
-                L.P[i][k + 1] = make_float2(v.z, v.w);
-                *reinterpret_cast<float4 *>(hi + (lrow0 + i) * N + lane * 2 + k * 32) = v;
+                float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
+                if (x1_0 + i < N && x2_0 + k < N) {
+                    if (a.vec) {
+                        h = *reinterpret_cast<const float4 *>(a.psi + g + k);
+                        l = *reinterpret_cast<const float4 *>(a.lo + g + k);
+                    } else {
+                        const float2 h0 = a.psi[g + k], l0 = a.lo[g + k];
+                        h.x = h0.x; h.y = h0.y; l.x = l0.x; l.y = l0.y;
+                        if (x2_0 + k + 1 < N) {
+                            const float2 h1 = a.psi[g + k + 1], l1 = a.lo[g + k + 1];
+                            h.z = h1.x; h.w = h1.y; l.z = l1.x; l.w = l1.y;
+                        }
+                    }
+                }
+                Q[i][k] = pack2(h.x, h.y);
+                Q[i][k + 1] = pack2(h.z, h.w);
+                los[(lrow0 + i) * RQ + k * 16 + lane] = l;
             }
         }
     };
-    // state out (hi, and the carried error for the next launch); each thread
-    // reads back only the shared words it wrote
-    auto store_realization = [&](const int r) {
-        float2 *glo = a.lo + a.tab.st_off[r];
+    auto store_rows = [&](float2 *dst, const int r, bool with_lo) {
+        const int64_t base = a.tab.st_off[r];
 #pragma unroll
         for (int i = 0; i < RL; ++i) {
+            const int64_t g = base + (int64_t)(x1_0 + i) * N + x2_0;
 #pragma unroll
-            for (int k = 0; k < CL; k += 2)
-                *reinterpret_cast<float4 *>(glo + (size_t)(x1_0 + i) * N + lane * 2 + k * 32) =
-                    *reinterpret_cast<const float4 *>(los + (lrow0 + i) * N + lane * 2 + k * 32);
-        }
-#pragma unroll
-        for (int i = 0; i < RL; ++i) {
-#pragma unroll
-            for (int k = 0; k < CL; k += 2)
-                *reinterpret_cast<float4 *>(a.psi + a.tab.st_off[r] + (size_t)(x1_0 + i) * N + x2_0 + k) =
-                    *reinterpret_cast<const float4 *>(hi + (lrow0 + i) * N + lane * 2 + k * 32);
+            for (int k = 0; k < CL; k += 2) {
+                if (x1_0 + i >= N || x2_0 + k >= N) continue;
+                const float4 l = with_lo ? los[(lrow0 + i) * RQ + k * 16 + lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+                if (a.vec) {
+                    *reinterpret_cast<ulonglong2 *>(dst + g + k) = make_ulonglong2(Q[i][k], Q[i][k + 1]);
+                    if (with_lo) *reinterpret_cast<float4 *>(a.lo + g + k) = l;
+                } else {
+                    dst[g + k] = unpack2(Q[i][k]);
+                    if (with_lo) a.lo[g + k] = make_float2(l.x, l.y);
+                    if (x2_0 + k + 1 < N) {
+                        dst[g + k + 1] = unpack2(Q[i][k + 1]);
+                        if (with_lo) a.lo[g + k + 1] = make_float2(l.z, l.w);
+                    }
+                }
+            }
         }
     };
 
     const int rank_up = (rank + C - 1) % C, rank_dn = (rank + 1) % C;
-    const uint32_t send_up = map_rank(smem_u32(halo + N + lane * 2), rank_up);    // their "row below" slot
+    const uint32_t send_up = map_rank(smem_u32(halo + RQ + lane), rank_up);    // their "row below" slot
     const uint32_t send_up_mb = map_rank(smem_u32(&mbar[0][1]), rank_up);
-    const uint32_t send_dn = map_rank(smem_u32(halo + lane * 2), rank_dn);        // their "row above" slot
+    const uint32_t send_dn = map_rank(smem_u32(halo + lane), rank_dn);         // their "row above" slot
     const uint32_t send_dn_mb = map_rank(smem_u32(&mbar[0][0]), rank_dn);
+    const uint32_t mb_edge = smem_u32(&mbar_edge), mb_halo = smem_u32(&mbar[0][0]);
     bool dead = false;
-    const float2 *Q = hi + lrow0 * N + lane * 2;
-    const int off = x1_0 % CL;
 
     if (threadIdx.x == 0) {
         for (int q = 0; q < 2; ++q)
             for (int sd = 0; sd < 2; ++sd) mbar_init(smem_u32(&mbar[q][sd]), 1);
+        mbar_init(mb_edge, my_warps > 0 ? my_warps : 1);
         mbar_init(smem_u32(&mbar_never), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -285,109 +263,188 @@ __global__ void __launch_bounds__(32 * W, MINB) taylor_fused_rows_kernel(const _
         cluster_barrier();
         return r;
     };
-    // the whole step loop, for this warp's (constant) diagonal offset
-    auto main_loop = [&](auto off_tag) {
-        constexpr int OFF = decltype(off_tag)::value;
+    // edge rows of the warp and of its neighbours, by parity (with one CTA the
+    // slab's edges are each other's neighbours)
+    const bool push_up = C > 1 && top, push_dn = C > 1 && bottom;
+    float4 *edge_own = edge + warp * 2 * RQ + lane;
+    const float4 *above = push_up ? halo + lane : edge + ((top ? my_warps : warp) - 1) * 2 * RQ + RQ + lane;
+    const float4 *below = push_dn ? halo + RQ + lane : edge + (bottom ? 0 : warp + 1) * 2 * RQ + lane;
+    const int above_stride = push_up ? 2 * RQ : 2 * W * RQ, below_stride = push_dn ? 2 * RQ : 2 * W * RQ;
+    // dt U for the lane's column that lies d = -2, 0, 2 or 4 beyond the row's
+    // index in the warp, where that column is on the diagonal x1 = x2
+    pair_t dU[4];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        const float v = x1_0 - x2_0 == 2 * d - 2 ? a.dtU : 0.f;
+        dU[d] = pack2(v, v);
+    }
+    const float2 *rcw = rowc + lrow0;
+    {
         // the stage counter runs on across realizations: the halo slots and
         // their mbarrier phases continue without a reset, and a neighbour can
         // never be more than one stage ahead
         unsigned tc = 0;
+        // the warp's first and last rows to its neighbours: shared memory, and
+        // from the slab's edges the neighbour CTAs (each edge warp arms the
+        // barrier it will wait on itself, whose previous phase it has seen)
+        auto publish = [&](const pair_t (&first)[CL], const pair_t (&last)[CL]) {
+            const int par = tc & 1;
+            ulonglong2 *eb = reinterpret_cast<ulonglong2 *>(edge_own + par * (2 * W * RQ));
+#pragma unroll
+            for (int k = 0; k < CL; k += 2) {
+                eb[k * 16] = make_ulonglong2(first[k], first[k + 1]);
+                eb[RQ + k * 16] = make_ulonglong2(last[k], last[k + 1]);
+            }
+            if (push_up) {
+                if (lane == 0) mbar_expect_tx(mb_halo + par * 16, RQ * 16);
+#pragma unroll
+                for (int k = 0; k < CL; k += 2)
+                    st_async16(send_up + par * (2 * RQ * 16) + k * 256, first[k], first[k + 1], send_up_mb + par * 16);
+            }
+            if (push_dn) {
+                if (lane == 0) mbar_expect_tx(mb_halo + par * 16 + 8, RQ * 16);
+#pragma unroll
+                for (int k = 0; k < CL; k += 2)
+                    st_async16(send_dn + par * (2 * RQ * 16) + k * 256, last[k], last[k + 1], send_dn_mb + par * 16);
+            }
+            __syncwarp();
+            mbar_arrive_lane0(mb_edge, lane);
+        };
+        auto wait_edges = [&]() {
+            if (!dead) dead = !mbar_wait_bounded(mb_edge, tc & 1, a.wait_limit_ns, a.status);
+            if (push_up || push_dn) {
+                const int par = tc & 1;
+                const uint32_t phase = (tc >> 1) & 1;
+                if (push_up && !dead) dead = !mbar_wait_bounded(mb_halo + par * 16, phase, a.wait_limit_ns, a.status);
+                if (push_dn && !dead) dead = !mbar_wait_bounded(mb_halo + par * 16 + 8, phase, a.wait_limit_ns, a.status);
+            }
+        };
+        auto load_row = [&](pair_t (&v)[CL], const float4 *src) {
+#pragma unroll
+            for (int k = 0; k < CL; k += 2) {
+                const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(src + k * 16);
+                v[k] = f.x;
+                v[k + 1] = f.y;
+            }
+        };
+        // the row above the warp's first and below its last row
+        auto load_above = [&](pair_t (&v)[CL]) { load_row(v, above + (tc & 1) * above_stride); };
+        auto load_below = [&](pair_t (&v)[CL]) { load_row(v, below + (tc & 1) * below_stride); };
+#define CTQW_ROW(i, up, c, dn) \
+    stencil_row<CL, i>(ec, nJc, rcw[i], rcw[(i) + 1], up, c, dn, dU, from_left, from_right, y)
+        // one middle stage: the edge rows in place, the inner rows from one register set to the other
+#define CTQW_MID(I1, I2, O1, O2)                    \
+    {                                               \
+        pair_t y[CL], nb[CL];                       \
+        publish(P[0], P[3]);                        \
+        CTQW_ROW(1, P[0], I1, I2);                  \
+        horner_row<CL>(O1, Q[1], y, inv_j);         \
+        CTQW_ROW(2, I1, I2, P[3]);                  \
+        horner_row<CL>(O2, Q[2], y, inv_j);         \
+        wait_edges();                               \
+        load_above(nb);                             \
+        CTQW_ROW(0, nb, P[0], I1);                  \
+        horner_row<CL>(P[0], Q[0], y, inv_j);       \
+        load_below(nb);                             \
+        CTQW_ROW(3, I2, P[3], nb);                  \
+        horner_row<CL>(P[3], Q[3], y, inv_j);       \
+        ++tc;                                       \
+    }
+        // psi(t+dt) = psi + A w_2, the rounding error carried in lo
+        auto update = [&](int i, const pair_t (&y)[CL]) {
+#pragma unroll
+            for (int k = 0; k < CL; k += 2) {
+                const float2 y0 = unpack2(y[k]), y1 = unpack2(y[k + 1]);
+                float2 h0 = unpack2(Q[i][k]), h1 = unpack2(Q[i][k + 1]);
+                const float2 s0 = make_float2(y0.y, -y0.x), s1 = make_float2(y1.y, -y1.x);
+                if (a.compensated) {
+                    float4 *lp = los + (lrow0 + i) * RQ + k * 16 + lane;
+                    const float4 l4 = *lp;
+                    float2 l0 = make_float2(l4.x, l4.y), l1 = make_float2(l4.z, l4.w);
+                    compensated_add2(h0, l0, s0);
+                    compensated_add2(h1, l1, s1);
+                    *lp = make_float4(l0.x, l0.y, l1.x, l1.y);
+                } else {
+                    h0 = make_float2(h0.x + s0.x, h0.y + s0.y);
+                    h1 = make_float2(h1.x + s1.x, h1.y + s1.y);
+                }
+                Q[i][k] = pack2(h0.x, h0.y);
+                Q[i][k + 1] = pack2(h1.x, h1.y);
+            }
+        };
         // realizations are handed out one at a time, so a cluster that runs
         // faster takes more of them
         for (int r = grab(); r < a.r0 + a.R_run; r = grab()) {
             __syncthreads();
             load_realization(r);
+            __syncthreads();
+            if (!active) continue;
             for (long long step = 0; step < n_steps; ++step) {
-                auto run_stage = [&](const int j, auto mode_tag) {
-                    constexpr int MODE = decltype(mode_tag)::value;
-                    const int parity = tc & 1;
-                    const uint32_t phase = (tc >> 1) & 1;
-                    // publish: this warp's first and last rows (shared memory; the slab
-                    // edge rows also into the neighbour CTAs)
-                    float2 *eb = edge + parity * (W * 2 * N) + warp * (2 * N) + lane * 2;
-    #pragma unroll
-                    for (int k = 0; k < CL; k += 2) {
-                        const float4 t = make_float4(L.P[0][k].x, L.P[0][k].y, L.P[0][k + 1].x, L.P[0][k + 1].y);
-                        const float4 b = make_float4(L.P[RL - 1][k].x, L.P[RL - 1][k].y, L.P[RL - 1][k + 1].x,
-                                                     L.P[RL - 1][k + 1].y);
-                        *reinterpret_cast<float4 *>(eb + k * 32) = t;
-                        *reinterpret_cast<float4 *>(eb + N + k * 32) = b;
-                        if (warp == 0) st_async16(send_up + parity * (2 * N * 8) + k * 256, t, send_up_mb + parity * 16);
-                        if (warp == W - 1) st_async16(send_dn + parity * (2 * N * 8) + k * 256, b, send_dn_mb + parity * 16);
-                    }
-                    __syncthreads();
-                    mbar_expect_tx2_if(smem_u32(&mbar[parity][0]), smem_u32(&mbar[parity][1]), N * 8,
-                                       threadIdx.x == 0);
-                    // the rows above and below this warp's block
-                    const float2 *usrc, *dsrc;
-                    if (warp > 0) {
-                        usrc = edge + parity * (W * 2 * N) + (warp - 1) * (2 * N) + N + lane * 2;
-                    } else {
-                        if (!dead) dead = !mbar_wait_bounded(smem_u32(&mbar[parity][0]), phase, a.wait_limit_ns, a.status);
-                        usrc = halo + parity * (2 * N) + lane * 2;
-                    }
-                    if (warp < W - 1) {
-                        dsrc = edge + parity * (W * 2 * N) + (warp + 1) * (2 * N) + lane * 2;
-                    } else {
-                        if (!dead) dead = !mbar_wait_bounded(smem_u32(&mbar[parity][1]), phase, a.wait_limit_ns, a.status);
-                        dsrc = halo + parity * (2 * N) + N + lane * 2;
-                    }
-                    stage<MODE, CL, RL, N, OFF>(L, rowc + lrow0, usrc, dsrc, Q, lane, x1_0, a.dtU, a.inv_j[j]);
+                if (K > 1) {
+                    // the first stage: w_K from psi, which stays in place
+                    const float inv_j = a.inv_j[K];
+                    pair_t y[CL], nb[CL];
+                    publish(Q[0], Q[3]);
+                    CTQW_ROW(1, Q[0], Q[1], Q[2]);
+                    horner_row<CL>(P[1], Q[1], y, inv_j);
+                    CTQW_ROW(2, Q[1], Q[2], Q[3]);
+                    horner_row<CL>(P[2], Q[2], y, inv_j);
+                    wait_edges();
+                    load_above(nb);
+                    CTQW_ROW(0, nb, Q[0], Q[1]);
+                    horner_row<CL>(P[0], Q[0], y, inv_j);
+                    load_below(nb);
+                    CTQW_ROW(3, Q[2], Q[3], nb);
+                    horner_row<CL>(P[3], Q[3], y, inv_j);
                     ++tc;
-                };
-                for (int j = K; j >= 2; --j) run_stage(j, std::integral_constant<int, kHorner>());
-                run_stage(1, std::integral_constant<int, kFinal>());
-                // psi(t+dt) = psi + A w_2 (in P); rounding error carried in lo
-        #pragma unroll
-                for (int i = 0; i < RL; ++i) {
-        #pragma unroll
-                    for (int k = 0; k < CL; k += 2) {
-                        float4 *hp = reinterpret_cast<float4 *>(hi + (lrow0 + i) * N + lane * 2 + k * 32);
-                        float4 *lp = reinterpret_cast<float4 *>(los + (lrow0 + i) * N + lane * 2 + k * 32);
-                        float4 h4 = *hp;
-                        if (a.compensated) {
-                            float4 l4 = *lp;
-                            float2 h0 = make_float2(h4.x, h4.y), h1 = make_float2(h4.z, h4.w);
-                            float2 l0 = make_float2(l4.x, l4.y), l1 = make_float2(l4.z, l4.w);
-                            compensated_add2(h0, l0, L.P[i][k]);
-                            compensated_add2(h1, l1, L.P[i][k + 1]);
-                            h4 = make_float4(h0.x, h0.y, h1.x, h1.y);
-                            *lp = make_float4(l0.x, l0.y, l1.x, l1.y);
-                        } else {
-                            h4.x += L.P[i][k].x;
-                            h4.y += L.P[i][k].y;
-                            h4.z += L.P[i][k + 1].x;
-                            h4.w += L.P[i][k + 1].y;
-                        }
-                        *hp = h4;
-                        L.P[i][k] = make_float2(h4.x, h4.y);
-                        L.P[i][k + 1] = make_float2(h4.z, h4.w);
-                    }
-                }
-                // a snapshot step: the new state (P) to its slot, row-major like psi
-                if (a.snap_every > 0 && step + 1 < n_steps && (step + 1) % a.snap_every == 0) {
-                    float2 *gs = a.snap + ((step + 1) / a.snap_every - 1) * a.snap_stride + a.tab.st_off[r];
-        #pragma unroll
+                } else {
+#pragma unroll
                     for (int i = 0; i < RL; ++i) {
-        #pragma unroll
-                        for (int k = 0; k < CL; k += 2)
-                            *reinterpret_cast<float4 *>(gs + (size_t)(x1_0 + i) * N + x2_0 + k) =
-                                make_float4(L.P[i][k].x, L.P[i][k].y, L.P[i][k + 1].x, L.P[i][k + 1].y);
+#pragma unroll
+                        for (int k = 0; k < CL; ++k) P[i][k] = Q[i][k];
                     }
                 }
+                int j = K - 1;
+#pragma unroll 1
+                while (j >= 2) {
+                    float inv_j = a.inv_j[j];
+                    CTQW_MID(P[1], P[2], T[0], T[1]);
+                    if (--j < 2) {
+#pragma unroll
+                        for (int k = 0; k < CL; ++k) {
+                            P[1][k] = T[0][k];
+                            P[2][k] = T[1][k];
+                        }
+                        break;
+                    }
+                    inv_j = a.inv_j[j];
+                    CTQW_MID(T[0], T[1], P[1], P[2]);
+                    --j;
+                }
+                {
+                    pair_t y[CL], nb[CL];
+                    publish(P[0], P[3]);
+                    CTQW_ROW(1, P[0], P[1], P[2]);
+                    update(1, y);
+                    CTQW_ROW(2, P[1], P[2], P[3]);
+                    update(2, y);
+                    wait_edges();
+                    load_above(nb);
+                    CTQW_ROW(0, nb, P[0], P[1]);
+                    update(0, y);
+                    load_below(nb);
+                    CTQW_ROW(3, P[2], P[3], nb);
+                    update(3, y);
+                    ++tc;
+                }
+                // a snapshot step: the new state to its slot, row-major like psi
+                if (a.snap_every > 0 && step + 1 < n_steps && (step + 1) % a.snap_every == 0)
+                    store_rows(a.snap + ((step + 1) / a.snap_every - 1) * a.snap_stride, r, false);
             }
-            store_realization(r);
+            store_rows(a.psi, r, true);
         }
-    };
-    // the first row's offset modulo CL: a multiple of gcd(RL, CL); only those are compiled
-    constexpr int GD = RL % CL == 0 ? CL : (CL % RL == 0 ? RL : (RL % 2 == 0 && CL % 2 == 0 ? 2 : 1));
-    static_assert(CL == 2 || CL == 4 || CL == 6 || CL == 8, "diagonal offsets enumerated for CL <= 8");
-    switch (off) {
-        case 0: main_loop(std::integral_constant<int, 0>()); break;
-        case 2: if constexpr (CL > 2 && 2 % GD == 0) main_loop(std::integral_constant<int, 2 % CL>()); break;
-        case 4: if constexpr (CL > 4 && 4 % GD == 0) main_loop(std::integral_constant<int, 4 % CL>()); break;
-        case 6: if constexpr (CL > 6 && 6 % GD == 0) main_loop(std::integral_constant<int, 6 % CL>()); break;
-        default: break;
+#undef CTQW_MID
+#undef CTQW_ROW
     }
     cluster_barrier();   // no CTA leaves while a neighbour may still push into it
 }
@@ -395,58 +452,55 @@ __global__ void __launch_bounds__(32 * W, MINB) taylor_fused_rows_kernel(const _
 using RowsKernel = void (*)(RowsArgs);
 
 struct RowsShape {
-    int C, threads;
+    int C, W, threads;
     size_t smem;
     RowsKernel kern;
 };
 
-template <int CL, int RL, int W, int MINB>
-RowsShape rows_shape() {
-    constexpr int N = 32 * CL, SR = RL * W;
-    RowsShape f;
-    f.C = N / SR;
-    f.threads = 32 * W;
-    f.smem = sizeof(float2) * ((size_t)SR * N + (size_t)2 * 2 * N + (size_t)2 * W * 2 * N) +
-             sizeof(float4) * (size_t)(SR + 1) + sizeof(float2) * (size_t)SR * N;
-    f.kern = taylor_fused_rows_kernel<CL, RL, W, MINB>;
-    return f;
-}
-
 constexpr int kRowsShapes = 3;
 
-bool rows_shape_for(int N, int idx, RowsShape &f) {
-    RowsShape opts[kRowsShapes];
-    switch (N) {
-        case 64: opts[0] = rows_shape<2, 8, 8, 2>(); opts[1] = rows_shape<2, 4, 8, 2>(); opts[2] = rows_shape<2, 8, 4, 3>(); break;
-        case 128: opts[0] = rows_shape<4, 8, 4, 2>(); opts[1] = rows_shape<4, 4, 8, 2>(); opts[2] = rows_shape<4, 4, 4, 3>(); break;
-        case 192: opts[0] = rows_shape<6, 4, 8, 1>(); opts[1] = rows_shape<6, 4, 4, 3>(); opts[2] = rows_shape<6, 4, 4, 2>(); break;
-        case 256: opts[0] = rows_shape<8, 4, 4, 2>(); opts[1] = rows_shape<8, 4, 8, 1>(); opts[2] = rows_shape<8, 4, 4, 3>(); break;
-        default: return false;
+// Columns per lane for the lattice: the fewest that cover it, and on a ring
+// divide it (0: none does).
+int rows_columns(int N, int periodic) {
+    for (int CL = 2; CL <= 8; CL += 2)
+        if (N <= 32 * CL && (!periodic || (N % CL == 0 && N % 4 == 0))) return CL;
+    return 0;
+}
+
+// Most warps a CTA: what one SM's registers hold (128 a thread for 16, 255
+// for 8), so smaller CTAs share an SM.
+int rows_max_warps(int CL) { return CL <= 4 ? 16 : 8; }
+
+// The kernel for the lattice with at most maxw warps a CTA, evened out over
+// the CTAs of the cluster.
+bool rows_shape_for(int N, int periodic, int maxw, RowsShape &f) {
+    const int CL = rows_columns(N, periodic);
+    if (CL == 0 || maxw < 1) return false;
+    switch (CL) {
+        case 2: f.kern = taylor_fused_rows_kernel<2, 16>; break;
+        case 4: f.kern = taylor_fused_rows_kernel<4, 16>; break;
+        case 6: f.kern = taylor_fused_rows_kernel<6, 8>; break;
+        default: f.kern = taylor_fused_rows_kernel<8, 8>; break;
     }
-    if (idx < 0 || idx >= kRowsShapes) return false;
-    f = opts[idx];
+    const int units = (N + 3) / 4;
+    f.C = (units + maxw - 1) / maxw;
+    if (f.C > 16) return false;
+    f.W = (units + f.C - 1) / f.C;
+    f.C = (units + f.W - 1) / f.W;
+    f.threads = 32 * f.W;
+    f.smem = sizeof(float4) * 16 * CL * (size_t)(4 + 4 * f.W + 4 * f.W) + sizeof(float2) * (size_t)(4 * f.W + 1);
     return true;
 }
 
-}  // namespace
-
-bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype) {
-    RowsShape f;
-    return dtype == CTQW_C64 && h->m == 2 && h->uniform && rows_shape_for(h->Nmax, 0, f);
-}
-
-namespace {
-
+// The kernels are shared by layouts of different sizes: the limit is always
+// the device's, so that calls for two handles cannot undo each other's.
 int set_rows_attributes(const RowsShape &f) {
-    CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)f.smem));
-    if (f.C > 8)
-        CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern,
-                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
+    CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return CTQW_OK;
 }
 
-int rows_clusters(const RowsShape &f, int *clusters) {
+int rows_residency(const RowsShape &f, int *clusters, int *per_sm) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)f.C);
     cfg.blockDim = dim3((unsigned)f.threads);
@@ -459,29 +513,77 @@ int rows_clusters(const RowsShape &f, int *clusters) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     CTQW_CUDA_TRY(cudaOccupancyMaxActiveClusters(clusters, (const void *)f.kern, &cfg));
+    CTQW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, (const void *)f.kern, f.threads, f.smem));
     return CTQW_OK;
+}
+
+// Layout `shape` of the handle: 0 the planned one, 1 at most half and 2 three
+// quarters of the most warps a CTA.
+bool rows_shape_of(const ctqw_hamiltonian *h, int shape, RowsShape &f) {
+    if (shape < 0 || shape >= kRowsShapes) return false;
+    const int most = rows_max_warps(rows_columns(h->Nmax, h->periodic));
+    return rows_shape_for(h->Nmax, h->periodic, shape == 0 ? h->rows_W : (shape == 1 ? most / 2 : most * 3 / 4), f);
 }
 
 }  // namespace
 
-// Tiled-to-fused throughput ratio per SM, measured on two bosons at N = 256,
-// K = 16: register tiles 4.43e11 site-updates/s on 152 SMs, the full-row
-// clusters 8.74e11 on the 112 that hold them.
+bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype) {
+    RowsShape f;
+    return dtype == CTQW_C64 && h->m == 2 && h->uniform && rows_shape_for(h->Nmax, h->periodic, 16, f);
+}
+
+// With many realizations the largest CTAs win by a little (fewest rows cross
+// between SMs: N = 128, R = 4096: 1.33e12 site-updates/s against 1.28e12 with
+// 8 warps).  With few, a realization spread over more SMs takes its stages
+// faster.  A stage measured a + b w microseconds with w warps on the SM:
+// (a, b) = (0.33, 0.011), (0.40, 0.034), (0.41, 0.035), (0.54, 0.042) for 2,
+// 4, 6, 8 columns a lane (N = 128, R = 1: 0.94, 0.65, 0.56 with 16, 8, 4
+// warps a CTA; N = 256: 0.88, 0.71 with 8, 4).  So: the time of the full
+// rounds of resident clusters plus the last one, which has its SMs to itself
+// as far as they go.
+int plan_fused_rows(ctqw_hamiltonian *h) {
+    if (!fused_rows_supported(h, CTQW_C64)) return CTQW_OK;
+    static const double a_of[5] = {0, 0.33, 0.40, 0.41, 0.54}, b_of[5] = {0, 0.011, 0.034, 0.035, 0.042};
+    const int CL = rows_columns(h->Nmax, h->periodic);
+    const double a = a_of[CL / 2], b = b_of[CL / 2];
+    double best = 0.0;
+    for (int maxw = rows_max_warps(CL); maxw >= rows_max_warps(CL) / 4; maxw /= 2) {
+        RowsShape f;
+        if (!rows_shape_for(h->Nmax, h->periodic, maxw, f)) continue;
+        CTQW_TRY(set_rows_attributes(f));
+        int clusters = 0, per_sm = 0;
+        CTQW_TRY(rows_residency(f, &clusters, &per_sm));
+        if (clusters < 1 || per_sm < 1) continue;
+        const int rounds = h->R / clusters, rest = h->R % clusters;
+        const int alone = std::max(1, clusters / per_sm);   // clusters that find SMs of their own
+        double t = rounds * (a + b * f.W * per_sm);
+        if (rest) t += a + b * f.W * std::min(per_sm, (rest + alone - 1) / alone);
+        if (best == 0.0 || t < 0.97 * best) {
+            best = t;
+            h->rows_W = f.W;
+            h->rows_C = f.C;
+            h->rows_clusters = clusters;
+            h->rows_per_sm = per_sm;
+        }
+    }
+    return CTQW_OK;
+}
+
+// Tiled-to-fused throughput ratio per SM on two bosons at N = 256, K = 16
+// (register tiles 4.43e11 site-updates/s on 152 SMs, the full-row clusters
+// 1.11e12 on the 120 that hold them: 0.32); 1024 realizations, 50 steps took
+// 48.4 ms with 0.32 and 47.8 ms with 0.37.
 static constexpr double kTiledPerSmRatio = 0.37;
 
 int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) {
     *R_tiled = 0;
-    RowsShape f;
-    if (!fused_rows_supported(h, CTQW_C64) || !rows_shape_for(h->Nmax, shape, f) ||
-        !tiled_supported(h, CTQW_C64, tiled_default_shape(h, K)) || h->group_N.size() != 1)
+    if (shape != 0 || h->rows_clusters < 1 || h->group_N.size() != 1 ||
+        !tiled_supported(h, CTQW_C64, tiled_default_shape(h, K)))
         return CTQW_OK;
-    CTQW_TRY(set_rows_attributes(f));
-    int clusters = 0, per_sm = 0, n_sm = 0;
-    CTQW_TRY(rows_clusters(f, &clusters));
-    CTQW_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void *)f.kern, f.threads, f.smem));
+    const int clusters = h->rows_clusters, per_sm = h->rows_per_sm;
+    int n_sm = 0;
     CTQW_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device));
-    if (clusters < 1 || per_sm < 1) return CTQW_OK;
-    const int used = std::min(n_sm, (clusters * f.C + per_sm - 1) / per_sm);
+    const int used = std::min(n_sm, (clusters * h->rows_C + per_sm - 1) / per_sm);
     const int idle = n_sm - used;
     if (idle * 16 < n_sm) return CTQW_OK;   // under 1/16 of the SMs idle: not worth a second stream
     // both parts end together when each one's share of the realizations
@@ -497,7 +599,7 @@ int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, voi
                              int snap_every, double dt, int K, int64_t n_steps, int compensated,
                              int shape, int test_timeout, int r0, int R_run, cudaStream_t s) {
     RowsShape f;
-    if (!rows_shape_for(h->Nmax, shape, f)) {
+    if (!rows_shape_of(h, shape, f)) {
         ctqw_set_error("fused path: unsupported size N=%d or shape %d", h->Nmax, shape);
         return CTQW_EUNSUPPORTED;
     }
@@ -521,6 +623,10 @@ int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, voi
     a.snap_stride = h->total_amp;
     a.dt = dt;
     a.dtU = (float)(dt * h->U);
+    a.N = h->Nmax;
+    a.W = f.W;
+    // even rows, and states that start on 16 bytes (N^2 amplitudes each)
+    a.vec = h->Nmax % 2 == 0 && (((uintptr_t)psi | (uintptr_t)lo | (uintptr_t)snap) & 15) == 0;
     a.K = K;
     a.n_steps = n_steps;
     a.compensated = compensated;
@@ -545,8 +651,8 @@ int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, voi
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int clusters = 0;
-    CTQW_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, (const void *)f.kern, &cfg));
+    int clusters = h->rows_clusters, per_sm = 0;
+    if (shape != 0) CTQW_TRY(rows_residency(f, &clusters, &per_sm));
     if (clusters < 1) {
         ctqw_set_error("fused path: no cluster of %d CTAs x %d threads fits", f.C, f.threads);
         return CTQW_EUNSUPPORTED;

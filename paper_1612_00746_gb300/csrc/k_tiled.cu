@@ -835,6 +835,8 @@ int tiled_depth(int shape) {
 // The 96 x 64 regions (depth 7 and 8 only) run at 0.94 of the rate a region
 // point and are taken where they save more than that: N = 1024 5.44e11,
 // N = 512 4.99e11 against 5.03e11.
+// Where every tile finds an SM of its own, launches are all that counts: the
+// 64 x 64 regions at the even split of the fewest launches.
 int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
     static const int by_depth[9] = {4, 10, 5, 9, 3, 8, 7, 6, 4};   // 64 x 64 regions
     constexpr double kTileFixed = 1180.0, kRowStage = 27.0, kTallRate = 0.94;
@@ -856,15 +858,26 @@ int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
             best_cost = cost;
         }
     };
+    const int few = (K + 7) / 8, even8 = (K + few - 1) / few;
+    {
+        TiledShape f;
+        int n_sm = 152;
+        tiled_shape_for(by_depth[even8], f);
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device);
+        int64_t tiles = 0;
+        for (size_t g = 0; g < h->group_N.size(); ++g)
+            tiles += (int64_t)h->group_count[g] * ((h->group_N[g] + f.TMAX - 1) / f.TMAX) *
+                     ((h->group_N[g] + f.TMAX2 - 1) / f.TMAX2);
+        if (tiles <= n_sm) return by_depth[even8];
+    }
     for (int d = 8; d >= 1; --d) {
         // only depths that split the stages evenly: another one does the same
         // launches on smaller tiles
         const int launches = (K + d - 1) / d;
         if ((K + launches - 1) / launches == d) consider(by_depth[d]);
     }
-    const int launches = (K + 7) / 8, even = (K + launches - 1) / launches;
-    if (even == 8) consider(13);
-    if (even == 7) consider(14);
+    if (even8 == 8) consider(13);
+    if (even8 == 7) consider(14);
     return best;
 }
 
