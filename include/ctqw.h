@@ -288,9 +288,12 @@ int ctqw_fused_split(const ctqw_hamiltonian *h, int32_t K, uint32_t flags, int32
  * to its right (never the absent wrap bond of an open chain).
  * The call first restores the parameters as built, so equal arguments give
  * equal results; afterwards the handle holds the parameters after the last
- * update (ctqw_get_params).  Paths: two particles in CTQW_C64 on the
- * temporally blocked tiles, everything else (or CTQW_FLAG_PLAIN) one launch
- * per term; both need 3 states of workspace (ctqw_workspace_size with
+ * update (ctqw_get_params).  Paths: two particles in CTQW_C64 on the fused
+ * cluster kernel where ctqw_propagate_taylor uses it (the clusters redraw
+ * their realization's parameters after every step, a launch per sampling
+ * interval), else on the temporally blocked tiles; everything else (or
+ * CTQW_FLAG_PLAIN) one launch per term; all need 3 states of workspace
+ * (ctqw_workspace_size with
  * CTQW_FLAG_PLAIN).  Outputs as ctqw_propagate_taylor; energies use H of
  * the sampled step.  Errors: as ctqw_propagate_taylor, EINVAL for p_switch
  * outside [0, 1] or a short workspace.  Asynchronous.

@@ -9,6 +9,7 @@
 #include <map>
 
 #include "ctqw_internal.cuh"
+#include "switching.cuh"
 
 namespace {
 
@@ -837,6 +838,27 @@ static int propagate_switching_impl(const ctqw_hamiltonian *h, int32_t dtype, vo
     sw.on = true;
     sw.seed = seed;
     sw.p = p_switch;
+    if (!(flags & CTQW_FLAG_PLAIN) && fused_rows_supported(h, dtype)) {
+        // the clusters redraw the parameters themselves after every step; a
+        // launch per sampling interval, since a sample uses H of its step
+        CTQW_TRY(zero_outputs(h, n_samples(n_steps, obs_every), P_mean_dev, norm_dev, energy_dev, s));
+        void *lo = workspace_dev;
+        CTQW_CUDA_TRY(cudaMemsetAsync(lo, 0, (size_t)h->total_amp * sizeof(float2), s));
+        const SwitchLaw law = switch_law(h, seed, p_switch);
+        for (int64_t s0 = 0;;) {
+            if (obs_every > 0 && s0 % obs_every == 0) {
+                const int64_t q = s0 / obs_every;
+                CTQW_TRY(launch_observables(h, dtype, psi_dev, P_mean_dev ? P_mean_dev + q * h->p_width : nullptr, nullptr,
+                                            norm_dev ? norm_dev + q * h->R : nullptr,
+                                            energy_dev ? energy_dev + q * h->R : nullptr, s));
+            }
+            if (s0 == n_steps) return CTQW_OK;
+            const int64_t chunk = obs_every > 0 ? std::min<int64_t>(n_steps - s0, obs_every) : n_steps;
+            CTQW_TRY(launch_taylor_fused_rows_switching(h, psi_dev, lo, dt, K, s0, chunk,
+                                                        (flags & CTQW_FLAG_NO_COMPENSATION) ? 0 : 1, law, s));
+            s0 += chunk;
+        }
+    }
     const int tshape = tiled_default_shape(h, K);
     if (!(flags & CTQW_FLAG_PLAIN) && tiled_supported(h, dtype, tshape))
         return propagate_tiled(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,

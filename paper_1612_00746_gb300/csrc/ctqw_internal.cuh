@@ -158,6 +158,8 @@ int launch_build_params(const ctqw_hamiltonian *h, const double *u_eps_d, const 
 // J of every realization redrawn with probability p (Philox4x64-10, key
 // (seed, 0), counter (step, r, i, 0)); restore_params puts back the
 // parameters as built.
+struct SwitchLaw;
+SwitchLaw switch_law(const ctqw_hamiltonian *h, uint64_t seed, double p);
 int launch_switch_params(const ctqw_hamiltonian *h, uint64_t seed, uint64_t step, double p,
                          cudaStream_t s);
 int restore_params(const ctqw_hamiltonian *h, cudaStream_t s);
@@ -262,6 +264,12 @@ int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled);
 int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap,
                              int snap_every, double dt, int K, int64_t n_steps, int compensated,
                              int shape, int test_timeout, int r0, int R_run, cudaStream_t s);
+// The same with switching noise: the Hamiltonian update of `law` after every
+// step (step0 is the first step's number), in the kernel; the handle holds the
+// parameters after the last one.  All realizations.
+int launch_taylor_fused_rows_switching(const ctqw_hamiltonian *h, void *psi, void *lo, double dt, int K,
+                                       int64_t step0, int64_t n_steps, int compensated, const SwitchLaw &law,
+                                       cudaStream_t s);
 
 // Fused row-wavefront Taylor propagation (m = 2, c64, open chains): every
 // Taylor term of a step on chip, psi streamed once per step; lo: the carried

@@ -61,6 +61,7 @@
 
 #include "ctqw_internal.cuh"
 #include "fused_common.cuh"
+#include "switching.cuh"
 
 namespace {
 
@@ -89,6 +90,12 @@ struct RowsArgs {
     int test_timeout;
     int r0, R_run;          // realizations r0 .. r0 + R_run - 1, handed out one at a time
     int *work;              // ticket counter of the hand-out, zero at the launch
+    // switching noise: the law, the number of the first step, and the
+    // parameters to leave the updated values in
+    SwitchLaw law;
+    unsigned long long step0;
+    double *eps_out, *J_out;
+    float *eps32_out, *J32_out;
     float inv_j[kMaxK + 1];
 };
 
@@ -129,7 +136,12 @@ __device__ __forceinline__ void horner_row(pair_t (&out)[CL], const pair_t (&Q)[
 }
 
 // CL columns per lane (N <= 32 CL), 4 rows a warp, up to MAXW warps a CTA.
-template <int CL, int MAXW>
+// SWITCH: the Hamiltonian update of switching noise after every step.  Every
+// CTA keeps the realization's parameters in shared memory and redraws all N
+// sites (the draws depend on nothing but the counter), so nothing is
+// exchanged for it.  256 realizations of N = 256, 50 steps of K = 16: 29.2 ms
+// on the tiles with an update launch a step, 18.3 ms here.
+template <int CL, int MAXW, bool SWITCH>
 __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const __grid_constant__ RowsArgs a) {
     constexpr int RL = 4;
     constexpr int RQ = 16 * CL;       // float4 (column pairs) a row in shared memory, lane-major
@@ -141,6 +153,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
     float4 *edge = halo + 2 * 2 * RQ;                       // [2 parity][W][2: first, last][RQ]
     float4 *los = edge + 2 * W * 2 * RQ;                    // [SR][RQ] carried error
     float2 *rowc = reinterpret_cast<float2 *>(los + SR * RQ);   // [SR + 1] (dt eps, -dt J of the bond above)
+    double *par = reinterpret_cast<double *>(rowc + SR + 2);    // SWITCH: [2][N] eps, J
     __shared__ __align__(8) unsigned long long mbar[2][2];      // halo rows: [parity][above, below]
     __shared__ __align__(8) unsigned long long mbar_edge;       // the CTA's warps have published a stage
     __shared__ __align__(8) unsigned long long mbar_never;
@@ -159,11 +172,9 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
     const int from_left = lane == 0 ? lanes - 1 : lane - 1, from_right = lane + 1 >= lanes ? 0 : lane + 1;
 
     pair_t P[RL][CL], Q[RL][CL], T[2][CL], ec[CL], nJc[CL + 1];
-    // coefficients and state of realization r (every warp reads rowc, so the
-    // caller orders this behind the previous realization's last stage)
-    auto load_realization = [&](const int r) {
-        const int64_t po = a.tab.par_off[r];
-        const double *eps = a.eps + po, *J = a.J + po;
+    // this warp's and lane's coefficients from the parameters (every warp
+    // reads rowc, so the caller orders this behind the last stage that did)
+    auto coefficients = [&](const double *eps, const double *J) {
         const double dt = a.dt;
         for (int q = threadIdx.x; q <= SR; q += blockDim.x) {
             const int x1 = rank * SR + q;
@@ -182,6 +193,20 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
             const int x = x2_0 + k;
             const float v = x2_0 < N && x <= N ? (float)(-dt * J[x == 0 ? N - 1 : x - 1]) : 0.f;
             nJc[k] = pack2(v, v);
+        }
+    };
+    // coefficients and state of realization r
+    auto load_realization = [&](const int r) {
+        const int64_t po = a.tab.par_off[r];
+        if (SWITCH) {
+            for (int i = threadIdx.x; i < N; i += blockDim.x) {
+                par[i] = a.eps[po + i];
+                par[N + i] = a.J[po + i];
+            }
+            __syncthreads();
+            coefficients(par, par + N);
+        } else {
+            coefficients(a.eps + po, a.J + po);
         }
         const int64_t base = a.tab.st_off[r];
 #pragma unroll
@@ -437,11 +462,31 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
                     update(3, y);
                     ++tc;
                 }
+                if (SWITCH) {
+                    // the Hamiltonian update: the warps with rows have read the
+                    // coefficients of this step when they get here
+                    const int threads = 32 * my_warps;
+                    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+                    for (int i = threadIdx.x; i < N; i += threads)
+                        (void)switch_site(a.law, a.step0 + step, r, i, N, par[i], par[N + i]);
+                    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+                    coefficients(par, par + N);
+                    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+                }
                 // a snapshot step: the new state to its slot, row-major like psi
                 if (a.snap_every > 0 && step + 1 < n_steps && (step + 1) % a.snap_every == 0)
                     store_rows(a.snap + ((step + 1) / a.snap_every - 1) * a.snap_stride, r, false);
             }
             store_rows(a.psi, r, true);
+            if (SWITCH && rank == 0) {
+                const int64_t po = a.tab.par_off[r];
+                for (int i = threadIdx.x; i < N; i += 32 * my_warps) {
+                    a.eps_out[po + i] = par[i];
+                    a.J_out[po + i] = par[N + i];
+                    a.eps32_out[po + i] = (float)par[i];
+                    a.J32_out[po + i] = (float)par[N + i];
+                }
+            }
         }
 #undef CTQW_MID
 #undef CTQW_ROW
@@ -454,7 +499,7 @@ using RowsKernel = void (*)(RowsArgs);
 struct RowsShape {
     int C, W, threads;
     size_t smem;
-    RowsKernel kern;
+    RowsKernel kern, kern_switch;
 };
 
 constexpr int kRowsShapes = 3;
@@ -477,10 +522,10 @@ bool rows_shape_for(int N, int periodic, int maxw, RowsShape &f) {
     const int CL = rows_columns(N, periodic);
     if (CL == 0 || maxw < 1) return false;
     switch (CL) {
-        case 2: f.kern = taylor_fused_rows_kernel<2, 16>; break;
-        case 4: f.kern = taylor_fused_rows_kernel<4, 16>; break;
-        case 6: f.kern = taylor_fused_rows_kernel<6, 8>; break;
-        default: f.kern = taylor_fused_rows_kernel<8, 8>; break;
+        case 2: f.kern = taylor_fused_rows_kernel<2, 16, false>; f.kern_switch = taylor_fused_rows_kernel<2, 16, true>; break;
+        case 4: f.kern = taylor_fused_rows_kernel<4, 16, false>; f.kern_switch = taylor_fused_rows_kernel<4, 16, true>; break;
+        case 6: f.kern = taylor_fused_rows_kernel<6, 8, false>; f.kern_switch = taylor_fused_rows_kernel<6, 8, true>; break;
+        default: f.kern = taylor_fused_rows_kernel<8, 8, false>; f.kern_switch = taylor_fused_rows_kernel<8, 8, true>; break;
     }
     const int units = (N + 3) / 4;
     f.C = (units + maxw - 1) / maxw;
@@ -488,15 +533,15 @@ bool rows_shape_for(int N, int periodic, int maxw, RowsShape &f) {
     f.W = (units + f.C - 1) / f.C;
     f.C = (units + f.W - 1) / f.W;
     f.threads = 32 * f.W;
-    f.smem = sizeof(float4) * 16 * CL * (size_t)(4 + 4 * f.W + 4 * f.W) + sizeof(float2) * (size_t)(4 * f.W + 1);
+    f.smem = sizeof(float4) * 16 * CL * (size_t)(4 + 4 * f.W + 4 * f.W) + sizeof(float2) * (size_t)(4 * f.W + 2);
     return true;
 }
 
 // The kernels are shared by layouts of different sizes: the limit is always
 // the device's, so that calls for two handles cannot undo each other's.
-int set_rows_attributes(const RowsShape &f) {
-    CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
-    CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+int set_rows_attributes(RowsKernel kern) {
+    CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - 1024));
+    CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     return CTQW_OK;
 }
 
@@ -550,7 +595,7 @@ int plan_fused_rows(ctqw_hamiltonian *h) {
     for (int maxw = rows_max_warps(CL); maxw >= rows_max_warps(CL) / 4; maxw /= 2) {
         RowsShape f;
         if (!rows_shape_for(h->Nmax, h->periodic, maxw, f)) continue;
-        CTQW_TRY(set_rows_attributes(f));
+        CTQW_TRY(set_rows_attributes(f.kern));
         int clusters = 0, per_sm = 0;
         CTQW_TRY(rows_residency(f, &clusters, &per_sm));
         if (clusters < 1 || per_sm < 1) continue;
@@ -595,9 +640,9 @@ int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) 
     return CTQW_OK;
 }
 
-int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap,
-                             int snap_every, double dt, int K, int64_t n_steps, int compensated,
-                             int shape, int test_timeout, int r0, int R_run, cudaStream_t s) {
+static int launch_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap, int snap_every, double dt, int K,
+                       int64_t n_steps, int compensated, int shape, int test_timeout, int r0, int R_run,
+                       const SwitchLaw *law, int64_t step0, cudaStream_t s) {
     RowsShape f;
     if (!rows_shape_of(h, shape, f)) {
         ctqw_set_error("fused path: unsupported size N=%d or shape %d", h->Nmax, shape);
@@ -636,9 +681,19 @@ int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, voi
     a.r0 = r0;
     a.R_run = R_run;
     a.work = work_counter(h);
+    a.step0 = (unsigned long long)step0;
+    if (law) {
+        a.law = *law;
+        a.eps_out = h->eps64;
+        a.J_out = h->J64;
+        a.eps32_out = h->eps32;
+        a.J32_out = h->J32;
+        f.kern = f.kern_switch;
+        f.smem += sizeof(double) * 2 * (size_t)h->Nmax;
+    }
     a.inv_j[0] = 0.f;
     for (int j = 1; j <= kMaxK; ++j) a.inv_j[j] = (float)(1.0 / j);
-    CTQW_TRY(set_rows_attributes(f));
+    CTQW_TRY(set_rows_attributes(f.kern));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)f.C);
     cfg.blockDim = dim3((unsigned)f.threads);
@@ -652,7 +707,7 @@ int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, voi
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int clusters = h->rows_clusters, per_sm = 0;
-    if (shape != 0) CTQW_TRY(rows_residency(f, &clusters, &per_sm));
+    if (shape != 0 || law) CTQW_TRY(rows_residency(f, &clusters, &per_sm));
     if (clusters < 1) {
         ctqw_set_error("fused path: no cluster of %d CTAs x %d threads fits", f.C, f.threads);
         return CTQW_EUNSUPPORTED;
@@ -662,4 +717,17 @@ int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, voi
     CTQW_CUDA_TRY(cudaMemsetAsync(a.work, 0, sizeof(int), s));
     CTQW_CUDA_TRY(cudaLaunchKernelEx(&cfg, f.kern, a));
     return CTQW_OK;
+}
+
+int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap, int snap_every, double dt,
+                             int K, int64_t n_steps, int compensated, int shape, int test_timeout, int r0,
+                             int R_run, cudaStream_t s) {
+    return launch_rows(h, psi, lo, snap, snap_every, dt, K, n_steps, compensated, shape, test_timeout, r0, R_run, nullptr,
+                       0, s);
+}
+
+int launch_taylor_fused_rows_switching(const ctqw_hamiltonian *h, void *psi, void *lo, double dt, int K,
+                                       int64_t step0, int64_t n_steps, int compensated, const SwitchLaw &law,
+                                       cudaStream_t s) {
+    return launch_rows(h, psi, lo, nullptr, 0, dt, K, n_steps, compensated, 0, 0, 0, h->R, &law, step0, s);
 }

@@ -87,3 +87,24 @@ def test_new_sizes_still_need_a_workspace(ctqw):
         ctqw.ctqw_propagate_taylor(h, psi, w.dtype, w.dt, 8, 1)
     assert e.value.status == ctqw.CTQW_EINVAL
     h.close()
+
+
+@pytest.mark.parametrize("N,R,periodic", [(30, 5, False), (64, 3, True), (100, 90, True), (130, 3, False), (256, 20, False)])
+@pytest.mark.parametrize("every", [0, 1, 4])
+def test_switching_in_the_kernel(ctqw, N, R, periodic, every):
+    # the same law and draws as the per-term path, whose updates are launches of their own
+    w = cw.get("bosons_n256_u2").with_(N=N, R=R, K=6, n_steps=9, periodic=periodic, sites=(N // 2 - 1, N // 2))
+    got = {}
+    for flags in (0, ctqw.FLAG_PLAIN):
+        h = ctqw.build_for_workload(w)
+        psi = h.new_state(w.dtype)
+        ctqw.ctqw_init_state(h, psi, ctqw.initial_sites(w, h), w.dtype)
+        P, nr, en = ctqw._outputs(h, h.n_obs(w.n_steps, every), True, True, True, "cuda")
+        ctqw.ctqw_propagate_taylor_switching(h, psi, w.dtype, w.dt, w.K, w.n_steps, every, P, nr, en, 11, 0.2, flags)
+        ctqw.ctqw_check_status(h)
+        got[flags] = [psi.cpu().numpy()] + [t.cpu().numpy() for t in (P, nr, en) if t is not None] + list(h.params())
+        h.close()
+    a, b = got[0], got[ctqw.FLAG_PLAIN]
+    assert np.array_equal(a[-1], b[-1]) and np.array_equal(a[-2], b[-2])   # parameters: the same bits
+    for x, y in zip(a[:-2], b[:-2]):
+        assert np.max(np.abs(x - y)) <= 12 * 5e-6
