@@ -178,16 +178,17 @@ constexpr int kObsWarps = 8;
 constexpr int kObsRows = 8;   // rows a warp takes at once (one multi-value reduction)
 
 // P(x), norm and energy of one sample; see the file comment.  Block
-// (blockIdx.x, r - r0) owns rows_per_block rows of realization r; warp w takes
-// groups of kObsRows consecutive rows (group w, w + 8, ...), lane l column
-// c0 + l of each 32-column tile.  <psi|H|psi> = sum_s V(s)|psi(s)|^2 -
+// (blockIdx.x, r - r0, blockIdx.z) owns rows_per_block rows and cols_per_block
+// (a multiple of 32) columns of realization r; warp w of the block's up to kObsWarps takes groups of kObsRows consecutive rows (group
+// w, w + warps, ...), lane l column c0 + l of each 32-column tile.  <psi|H|psi> = sum_s V(s)|psi(s)|^2 -
 // 2 sum_bonds J Re(conj(psi(s)) psi(s')), every bond taken once, by the
 // amplitude before it along its direction.  Dynamic shared memory:
 // rows_per_block accumulators.
-template <typename T, int M>
+// WHOLE: blocks of kObsWarps warps over all columns (the usual case).
+template <typename T, int M, bool WHOLE>
 __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
     RealTable tab, const T *__restrict__ eps, const T *__restrict__ J,
-    const cplx_t<T> *__restrict__ psi, int rows_per_block, double *P_mean, double *norm,
+    const cplx_t<T> *__restrict__ psi, int rows_per_block, int cols_per_block, double *P_mean, double *norm,
     double *energy, int r0) {
     using S = ObsSum<T>;
     using A = typename S::A;
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
     const int row0 = blockIdx.x * rows_per_block;
     if (row0 >= n_rows) return;
     const int nr = min(rows_per_block, n_rows - row0);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = WHOLE ? kObsWarps : blockDim.x >> 5;
     for (int i = threadIdx.x; i < nr; i += blockDim.x) rowacc[i] = A(0);
     if (threadIdx.x == 0) red_bad = 0u;
     __syncthreads();
@@ -215,7 +216,9 @@ __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
     const bool want_e = energy != nullptr;
     A en = A(0);
     unsigned bad = 0u;
-    for (int c0 = 0; c0 < N; c0 += 32) {
+    const int c_first = WHOLE ? 0 : blockIdx.z * cols_per_block, c_last = WHOLE ? N : min(N, c_first + cols_per_block);
+    if (c_first >= N) return;
+    for (int c0 = c_first; c0 < c_last; c0 += 32) {
         const int x = c0 + lane;
         const bool valid = x < N;
         const int xv = valid ? x : 0;
@@ -223,7 +226,7 @@ __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
         const bool load_right = lane == 31 || x + 1 >= N;
         const T ex = ep[xv], jx = valid ? jp[xv] : T(0);
         A col = A(0);
-        for (int q0 = warp * kObsRows; q0 < nr; q0 += kObsWarps * kObsRows) {
+        for (int q0 = warp * kObsRows; q0 < nr; q0 += warps * kObsRows) {
             A rp[kObsRows];
 #pragma unroll
             for (int u = 0; u < kObsRows; ++u) {
@@ -254,8 +257,14 @@ __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
 #pragma unroll
                             for (int l = j + 1; l < M - 1; ++l) pairs += (xs[j] == xs[l]);
                         }
-                        v += U * T(pairs);
-                        T e = p * v - T(2) * jx * (c.x * right.x + c.y * right.y);
+                        if (sizeof(T) == 4 || pairs) v += U * T(pairs);
+                        // FP64: the bonds' sum doubled once (its pipe is the bound)
+                        T bonds = T(0);
+                        T e = T(0);
+                        if (sizeof(T) == 4)
+                            e = p * v - T(2) * jx * (c.x * right.x + c.y * right.y);
+                        else
+                            bonds = jx * (c.x * right.x + c.y * right.y);
                         // bonds along the row coordinates: the amplitude one step further along x_j
                         int64_t stride = N;
 #pragma unroll
@@ -263,9 +272,13 @@ __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
                             const int xj = xs[j];
                             const int xjn = xj + 1 == N ? 0 : xj + 1;
                             const cplx_t<T> d = a[(int64_t)x + rb + (int64_t)(xjn - xj) * stride];
-                            e -= T(2) * jp[xj] * (c.x * d.x + c.y * d.y);
+                            if (sizeof(T) == 4)
+                                e -= T(2) * jp[xj] * (c.x * d.x + c.y * d.y);
+                            else
+                                bonds += jp[xj] * (c.x * d.x + c.y * d.y);
                             stride *= N;
                         }
+                        if (sizeof(T) == 8) e = p * v - T(2) * bonds;
                         en += S::e(e, bad);
                     }
                 }
@@ -280,7 +293,8 @@ __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
         if (warp == 0) {
             A t = colred[0][lane];
 #pragma unroll
-            for (int w = 1; w < kObsWarps; ++w) t += colred[w][lane];
+            for (int w = 1; w < kObsWarps; ++w)
+                if (w < warps) t += colred[w][lane];
             bad |= S::over(t);
             if (valid && Pg) atomicAdd(Pg + x, S::dp(t) * scale);
         }
@@ -313,7 +327,7 @@ __global__ void __launch_bounds__(32 * kObsWarps) occupation_kernel(
     __syncthreads();
     if (threadIdx.x == 0) {
         A tn = red[0][0], te = red[0][1];
-        for (int w = 1; w < kObsWarps; ++w) {
+        for (int w = 1; w < warps; ++w) {
             tn += red[w][0];
             te += red[w][1];
         }
@@ -388,23 +402,39 @@ int launch_observables_range(const ctqw_hamiltonian *h, int dtype, const void *p
         return CTQW_EINVAL;
     }
     RealTable t = real_table(h);
-    // rows per block: about one wave of 8 blocks per SM over the realizations
+    // about one wave of 8 blocks per SM over the realizations: first fewer
+    // rows a block, down to the 64 of 8 warps; where few realizations leave SMs
+    // without a block even so, fewer columns, then fewer warps.  (Blocks that
+    // share columns or rows also share the addresses of their atomics: 16
+    // realizations of N = 256 in FP64 took 98 us a sample in 64 whole-width
+    // blocks, 82 us in 512 of one warp, 45 us split by columns.)
     const int64_t rows_max = h->m == 2 ? (int64_t)h->Nmax : (int64_t)h->Nmax * h->Nmax;
     const int64_t target = 152 * 8;
     const int64_t per_r = std::max<int64_t>(1, (target + R_run - 1) / R_run);
     int64_t rpb = (rows_max + per_r - 1) / per_r;
-    // a whole number of 8-row groups for every warp, at most 4096 rows
     constexpr int64_t unit = kObsWarps * kObsRows;
     rpb = std::min<int64_t>(4096, std::max<int64_t>(unit, (rpb + unit - 1) / unit * unit));
-    const dim3 grid((unsigned)((rows_max + rpb - 1) / rpb), (unsigned)R_run);
+    int warps = kObsWarps;
+    const int width = (h->Nmax + 31) / 32 * 32;
+    int cols = width;
+    auto blocks = [&]() { return (rows_max + rpb - 1) / rpb * R_run * ((width + cols - 1) / cols); };
+    while (blocks() < 304 && cols > 32) cols = (cols / 2 + 31) / 32 * 32;
+    while (blocks() < 152 && warps > 1 && rpb == (int64_t)warps * kObsRows) {
+        warps /= 2;
+        rpb /= 2;
+    }
+    const dim3 grid((unsigned)((rows_max + rpb - 1) / rpb), (unsigned)R_run, (unsigned)((width + cols - 1) / cols));
+    const bool whole = warps == kObsWarps && cols == width;
     const size_t smem = (size_t)rpb * 8;
     if (dtype == CTQW_C64) {
-        auto k = h->m == 2 ? occupation_kernel<float, 2> : occupation_kernel<float, 3>;
-        k<<<grid, 32 * kObsWarps, smem, s>>>(t, h->eps32, h->J32, (const float2 *)psi, (int)rpb, P_mean,
+        auto k = h->m == 2 ? (whole ? occupation_kernel<float, 2, true> : occupation_kernel<float, 2, false>)
+                           : (whole ? occupation_kernel<float, 3, true> : occupation_kernel<float, 3, false>);
+        k<<<grid, 32 * warps, smem, s>>>(t, h->eps32, h->J32, (const float2 *)psi, (int)rpb, cols, P_mean,
                                              norm, energy, r0);
     } else {
-        auto k = h->m == 2 ? occupation_kernel<double, 2> : occupation_kernel<double, 3>;
-        k<<<grid, 32 * kObsWarps, smem, s>>>(t, h->eps64, h->J64, (const double2 *)psi, (int)rpb, P_mean,
+        auto k = h->m == 2 ? (whole ? occupation_kernel<double, 2, true> : occupation_kernel<double, 2, false>)
+                           : (whole ? occupation_kernel<double, 3, true> : occupation_kernel<double, 3, false>);
+        k<<<grid, 32 * warps, smem, s>>>(t, h->eps64, h->J64, (const double2 *)psi, (int)rpb, cols, P_mean,
                                              norm, energy, r0);
     }
     CTQW_CUDA_TRY(cudaGetLastError());
