@@ -811,6 +811,21 @@ static int propagate_taylor_impl(const ctqw_hamiltonian *h, int32_t dtype, void 
                                    energy_dev, comp, shape - 4, test, s);
     }
 
+    if (const int ctas = dtype == CTQW_C128 && !(flags & CTQW_FLAG_PLAIN) && n_steps > 0 ? resident_f64_ctas(h) : 0) {
+        // small FP64 states: a launch per sampling interval
+        for (int64_t s0 = 0;;) {
+            if (obs_every > 0 && s0 % obs_every == 0) {
+                const int64_t q = s0 / obs_every;
+                CTQW_TRY(launch_observables(h, dtype, psi_dev, P_mean_dev ? P_mean_dev + q * h->p_width : nullptr, nullptr,
+                                            norm_dev ? norm_dev + q * h->R : nullptr,
+                                            energy_dev ? energy_dev + q * h->R : nullptr, s));
+            }
+            if (s0 == n_steps) return CTQW_OK;
+            const int64_t chunk = obs_every > 0 ? std::min<int64_t>(n_steps - s0, obs_every) : n_steps;
+            CTQW_TRY(launch_resident_f64(h, ctas, psi_dev, dt, K, chunk, s));
+            s0 += chunk;
+        }
+    }
     return propagate_per_term(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,
                               energy_dev, workspace_dev, s, SwitchSpec{});
 }

@@ -176,6 +176,13 @@ int launch_init_state(const ctqw_hamiltonian *h, const int32_t *sites_d, int dty
 int launch_horner_f64(const ctqw_hamiltonian *h, const void *in, const void *psi, void *out, double coef,
                       cudaStream_t s);
 
+// FP64 propagation of small states resident on chip (k_resident64.cu): most
+// CTAs of a realization's cluster, 0 where one launch per term is the better
+// way (or the only one); n_steps steps in place.
+int resident_f64_ctas(const ctqw_hamiltonian *h);
+int launch_resident_f64(const ctqw_hamiltonian *h, int C_max, void *psi, double dt, int K, int64_t n_steps,
+                        cudaStream_t s);
+
 // FP32 per-term path in Horner form: out = psi + coef (-i) H in;
 // final: psi (+lo, carried rounding error) += -i dt H w2.
 int launch_horner_stage(const ctqw_hamiltonian *h, const void *in, const void *psi, void *out,

@@ -87,3 +87,24 @@ def test_ragged_and_rk4(ctqw, N, R):
     w = cw.get("ragged_n128_1024").with_(R=R, ragged_sizes=(N, N + 7, 2 * N), n_steps=3, dtype=cw.C128, sites=(-1, 0))
     _compare(ctqw, w, ctqw.TAYLOR)
     _compare(ctqw, w, ctqw.RK4)
+
+
+@pytest.mark.parametrize("N,R", [(2, 1), (3, 2), (7, 5), (16, 1), (17, 3), (31, 4), (32, 70), (48, 9), (64, 8), (65, 2), (100, 1),
+                                 (128, 1)])
+@pytest.mark.parametrize("K,periodic", [(1, True), (5, False), (12, True)])
+def test_resident_states(ctqw, N, R, K, periodic):
+    # the sizes that stay on chip: slabs of one row, uneven last slabs, one
+    # to eight amplitudes a thread; with samples (a launch per interval)
+    w = cw.get("bosons_n256_u2").with_(N=N, R=R, periodic=periodic, K=K, n_steps=3, dtype=cw.C128)
+    _compare(ctqw, w, ctqw.TAYLOR)
+    h = ctqw.build_for_workload(w)
+    out = []
+    for flags in (0, ctqw.FLAG_PLAIN):
+        psi = torch.randn(2 * h.total_amplitudes, dtype=torch.float64, device="cuda",
+                          generator=torch.Generator("cuda").manual_seed(1)).view(torch.complex128) / N
+        P, nr, en = ctqw._outputs(h, h.n_obs(5, 2), True, True, True, "cuda")
+        ctqw.ctqw_propagate_taylor(h, psi, w.dtype, w.dt, K, 5, 2, P, nr, en, flags, h.workspace(w.dtype))
+        out.append([t.cpu().numpy() for t in (psi, P, nr, en)])
+    h.close()
+    for a, b in zip(*out):   # sums of up to N^2 products of order 1 / N^2
+        assert np.max(np.abs(a - b)) <= 1e-12
