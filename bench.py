@@ -220,14 +220,15 @@ def propagation_path(w, dtype, flags, switching=False):
     shape = (flags >> 8) & 0xF
     if flags & ctqw.FLAG_PLAIN:
         return "plain"
+    on_clusters = (dtype == ctqw.C64 and w.m == 2 and w.ragged_sizes is None and w.N <= 256
+                   and (not w.periodic or w.N % 4 == 0))
     if switching:
-        return "tiled" if dtype == ctqw.C64 and w.m == 2 else "plain"
+        return "rows" if on_clusters else "tiled" if dtype == ctqw.C64 and w.m == 2 else "plain"
     if shape == ctqw.SHAPE_WAVEFRONT:
         return "wavefront"
     if shape >= 9:
         return "tiled"
-    uniform = w.ragged_sizes is None
-    if dtype == ctqw.C64 and w.m == 2 and uniform and w.N in (64, 128, 192, 256):
+    if on_clusters:
         return "rows" if shape < 4 else "banded"
     if dtype == ctqw.C64 and w.m == 2 and shape == 0:
         return "tiled"   # the library's default for the other two-particle FP32 handles
@@ -241,8 +242,9 @@ def roofline_of(w, dtype, flags, units, kernel_ms, peaks, traffic, switching=Fal
     8m+4 algorithmic flops per site-update against the SMs x 128 lanes x 2
     flop x 2070 MHz.  The FP32 per-term kernels stream the state through HBM:
     per site-update ((K-1) 24 + 40)/K bytes (Horner stages and the
-    compensated final stage), against the measured copy bandwidth.  The FP64
-    per-term kernels move 64 bytes per site-update but are bound by the FP64
+    compensated final stage), against the measured copy bandwidth; three
+    particles take two stages a launch and are bound by the FP32 pipe.  The FP64
+    per-term kernels move 48 bytes per site-update but are bound by the FP64
     pipe (2 DFMA per SM per cycle).
     """
     from paper_1612_00746_gb300 import ctqw
@@ -272,6 +274,18 @@ def roofline_of(w, dtype, flags, units, kernel_ms, peaks, traffic, switching=Fal
                               "hbm_gbs_achieved": units * 48.0 / sec / 1e9, "bytes_per_site_update": 48.0,
                               "peak_basis": f"{SM_COUNT} SMs x 2 DFMA x 2 flop x 2070 MHz (FP64, derived)",
                               "timing": "the whole propagate call (observables kernels included)"}, "fp64")
+    if w.m == 3 and not flags & ctqw.FLAG_PLAIN:
+        # two stages a launch: 12 bytes a site-update, bound by instructions
+        flops_per_unit = 8 * w.m + 4
+        achieved = units * flops_per_unit / sec / 1e12
+        peak = alu_peak()
+        bpu = ((w.K - 2) * 12.0 + 40.0) / w.K
+        return with_measured({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+                              "frac": achieved / peak, "traffic": None, "kernel": "horner3_pair_kernel",
+                              "kernel_ms": kernel_ms, "flops_per_site_update": flops_per_unit,
+                              "hbm_gbs_achieved": units * bpu / sec / 1e9, "bytes_per_site_update": bpu,
+                              "peak_basis": f"{SM_COUNT} SMs x 128 FP32 FMA lanes x 2 flop x 2070 MHz (derived)",
+                              "timing": "the whole propagate call (observables kernels included)"}, "fp32")
     bpu = ((w.K - 1) * 24.0 + 40.0) / w.K
     kernel = "horner_stage_kernel + horner_final_kernel"
     gbs = units * bpu / sec / 1e9

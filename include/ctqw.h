@@ -233,7 +233,9 @@ int ctqw_autotune_order(const ctqw_hamiltonian *h, int32_t dtype, double dt, int
  * of a cluster point to point, see ctqw_check_status); other m = 2 handles
  * in CTQW_C64 (N > 256, ragged sizes, other rings) run the temporally blocked
  * tiled kernel with the iterate in registers, at the tile and depth that
- * cost the fewest instructions; everything
+ * cost the fewest instructions; m = 3 handles in CTQW_C64 (5 <= N <= 256)
+ * run two Taylor terms per launch; m = 2 handles in CTQW_C128 small enough
+ * for it keep their states on chip; everything
  * else, or CTQW_FLAG_PLAIN, runs one launch per Taylor term.  Every path
  * needs the workspace of ctqw_workspace_size (3 states).  The fused path
  * keeps the carried error in the first state and stores the state at

@@ -103,8 +103,18 @@ int taylor_step_plain(const ctqw_hamiltonian *h, int dtype, const void *in, void
     }
     const void *w = in;
     void *dst = phiA;
+    const bool pairs = dtype == CTQW_C64 && horner3_pair_supported(h);
     for (int j = K; j >= 1; --j) {
         void *o = (j == 1) ? out : dst;
+        if (pairs && (j & 1) == 0) {   // stages j and j - 1
+            o = j == 2 ? out : dst;
+            int st = launch_horner3_pair(h, w, in, o, nullptr, dt / j, dt / (j - 1), s);
+            if (st != CTQW_OK) return st;
+            --j;
+            w = o;
+            dst = (dst == phiA) ? phiB : phiA;
+            continue;
+        }
         int st = dtype == CTQW_C64 ? launch_horner_stage(h, w, in, o, dt / j, s)
                                    : launch_horner_f64(h, w, in, o, dt / j, s);
         if (st != CTQW_OK) return st;
@@ -593,6 +603,46 @@ static int propagate_per_term(const ctqw_hamiltonian *h, int32_t dtype, void *ps
     return CTQW_OK;
 }
 
+// Three particles in c64 with two stages per launch (an odd order starts with
+// a single one).  The new state cannot overwrite the one that other blocks
+// still read, so it rotates through psi and the two iterate buffers; outputs
+// already zeroed and the workspace (3 states) checked by the caller.
+static int propagate_pairs(const ctqw_hamiltonian *h, void *psi_dev, double dt, int32_t K, int64_t n_steps,
+                           int32_t obs_every, double *P_mean_dev, double *norm_dev, double *energy_dev,
+                           void *workspace_dev, cudaStream_t s, const SwitchSpec &sw) {
+    const size_t sb = (size_t)h->total_amp * sizeof(float2);
+    char *ws = (char *)workspace_dev;
+    void *bufs[3] = {psi_dev, ws, ws + sb}, *lo = ws + 2 * sb;
+    CTQW_CUDA_TRY(cudaMemsetAsync(lo, 0, sb, s));
+    int cur = 0;
+    int64_t obs = 0;
+    for (int64_t step = 0; step <= n_steps; ++step) {
+        if (obs_every > 0 && step % obs_every == 0) {
+            CTQW_TRY(launch_observables(h, CTQW_C64, bufs[cur], P_mean_dev ? P_mean_dev + obs * h->p_width : nullptr,
+                                        nullptr, norm_dev ? norm_dev + obs * h->R : nullptr,
+                                        energy_dev ? energy_dev + obs * h->R : nullptr, s));
+            ++obs;
+        }
+        if (step == n_steps) break;
+        const int o1 = (cur + 1) % 3, o2 = (cur + 2) % 3;
+        int in = cur, out = o1, j = K;
+        if (j & 1) {
+            CTQW_TRY(launch_horner_stage(h, bufs[in], bufs[cur], bufs[out], dt / j, s));
+            in = out;
+            --j;
+        }
+        for (; j >= 2; j -= 2) {
+            out = in == o1 ? o2 : o1;
+            CTQW_TRY(launch_horner3_pair(h, bufs[in], bufs[cur], bufs[out], j == 2 ? lo : nullptr, dt / j, dt / (j - 1), s));
+            in = out;
+        }
+        cur = out;
+        if (sw.on) CTQW_TRY(launch_switch_params(h, sw.seed, (uint64_t)step, sw.p, s));
+    }
+    if (cur != 0) CTQW_CUDA_TRY(cudaMemcpyAsync(psi_dev, bufs[cur], sb, cudaMemcpyDeviceToDevice, s));
+    return CTQW_OK;
+}
+
 // The step loop of the temporally blocked tiled kernels (c64) over
 // realizations r0 .. r0 + R_run - 1: ceil(K / D) launches per step.  The
 // state rotates through bufs[0] (psi) and the iterate buffers bufs[1],
@@ -826,6 +876,9 @@ static int propagate_taylor_impl(const ctqw_hamiltonian *h, int32_t dtype, void 
             s0 += chunk;
         }
     }
+    if (dtype == CTQW_C64 && K > 1 && !(flags & CTQW_FLAG_PLAIN) && horner3_pair_supported(h))
+        return propagate_pairs(h, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev, energy_dev, workspace_dev, s,
+                               SwitchSpec{});
     return propagate_per_term(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,
                               energy_dev, workspace_dev, s, SwitchSpec{});
 }
@@ -879,6 +932,9 @@ static int propagate_switching_impl(const ctqw_hamiltonian *h, int32_t dtype, vo
         return propagate_tiled(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,
                                energy_dev, flags, tshape, workspace_dev, workspace_bytes, s, sw);
     CTQW_TRY(zero_outputs(h, n_samples(n_steps, obs_every), P_mean_dev, norm_dev, energy_dev, s));
+    if (dtype == CTQW_C64 && K > 1 && !(flags & CTQW_FLAG_PLAIN) && horner3_pair_supported(h))
+        return propagate_pairs(h, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev, energy_dev, workspace_dev, s,
+                               sw);
     return propagate_per_term(h, dtype, psi_dev, dt, K, n_steps, obs_every, P_mean_dev, norm_dev,
                               energy_dev, workspace_dev, s, sw);
 }

@@ -190,6 +190,13 @@ int launch_horner_stage(const ctqw_hamiltonian *h, const void *in, const void *p
 int launch_horner_final(const ctqw_hamiltonian *h, const void *w2, void *psi, void *lo, double dt,
                         cudaStream_t s);
 
+// Two FP32 Horner stages per launch, three particles (k_horner3.cu): out =
+// psi + c2 (-i) H (psi + c1 (-i) H in); with lo the second one adds its
+// increment compensated.  out is none of the inputs.
+bool horner3_pair_supported(const ctqw_hamiltonian *h);
+int launch_horner3_pair(const ctqw_hamiltonian *h, const void *in, const void *psi, void *out, void *lo, double c1,
+                        double c2, cudaStream_t s);
+
 // RK4 stage (a4): k = -i H in; next = psi + a k (if next); acc (= psi if first) += b k.
 int launch_rk4_stage(const ctqw_hamiltonian *h, int dtype, const void *in, void *next,
                      const void *psi, void *acc, double a, double b, int first, cudaStream_t s);
