@@ -993,7 +993,16 @@ def run_lattice(args):
     value = units / (ms / 1000.0)
     drift = float((nr[-1] - 1.0).abs().max().item()) if n_obs else None
     peaks = measured_peaks()
-    if w.dtype == cw.C64:
+    if w.dtype == cw.C64 and w.m == 2 and g.N <= 324 and 2 * g.E <= 4 * g.N:
+        # iterates on chip, bound by shared memory; against the FP32 pipe
+        flops = 4.0 * w.m * 2 * g.E / g.N + 4
+        ach = units * flops / (ms / 1000.0) / 1e12
+        peak = alu_peak()
+        roof = {"bound": "alu", "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
+                "traffic": None, "kernel": "graph_resident_kernel", "kernel_ms": ms, "flops_per_site_update": flops,
+                "peak_basis": f"{SM_COUNT} SMs x 128 FP32 FMA lanes x 2 flop x 2070 MHz (derived)",
+                "timing": "the whole propagate call (observables kernels included)"}
+    elif w.dtype == cw.C64:
         bpu = ((w.K - 1) * 24.0 + 40.0) / w.K
         gbs = units * bpu / (ms / 1000.0) / 1e9
         peak = peaks.get("hbm_gbs")

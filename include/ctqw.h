@@ -564,7 +564,9 @@ int ctqw_graph_workspace_size(const ctqw_graph *g, int32_t dtype, size_t *bytes)
 
 /*
  * Advance every realization by n_steps order-K Taylor steps (Sec. 2.3,
- * Algorithm 3), one launch per term over all realizations.  CTQW_C128 runs
+ * Algorithm 3), one launch per term over all realizations; m = 2 in CTQW_C64
+ * on graphs whose two iterates fit on chip (a few hundred nodes of at most 8
+ * links), where that is faster, one launch per sampling interval.  CTQW_C128 runs
  * the terms in the order of Algorithm 3; CTQW_C64 the same polynomial in
  * Horner form with the state update compensated (the carried rounding
  * error lives in the third workspace state), as the chain's per-term path.

@@ -167,6 +167,7 @@ int ctqw_graph_build(const ctqw_graph_desc *d, void *stream, ctqw_graph **out) {
         ctqw_set_error("graph parameter build failed");
         st = CTQW_ECUDA;
     }
+    if (st == CTQW_OK) st = plan_graph_resident(g, row_ptr.data(), col.data(), *std::max_element(deg.begin(), deg.end()));
     if (u_eps_d) cudaFree(u_eps_d);
     if (u_J_d) cudaFree(u_J_d);
     if (st != CTQW_OK) {
@@ -257,6 +258,26 @@ int ctqw_graph_propagate_taylor(const ctqw_graph *g, int32_t dtype, void *psi_de
     char *ws = (char *)workspace_dev;
     CTQW_TRY(zero_graph_outputs(g, g_samples(n_steps, obs_every), P_mean_dev, norm_dev, energy_dev, s));
     const int chunk = graph_chunk(g);
+    if (dtype == CTQW_C64 && g->res_CL > 0) {
+        // all steps between two samples in one launch, on states in [r][s] order
+        void *psi_t = ws, *lo = ws + sb;
+        if (n_steps > 0) CTQW_CUDA_TRY(cudaMemsetAsync(lo, 0, sb, s));
+        for (int rb = 0; rb < g->R; rb += chunk) {
+            const int re = std::min(g->R, rb + chunk);
+            if (n_steps > 0) CTQW_TRY(launch_graph_to_rows(g, rb, re, psi_dev, psi_t, s));
+            int64_t obs = 0;
+            for (int64_t step = 0;;) {
+                if (obs_every > 0 && step % obs_every == 0)
+                    CTQW_TRY(sample(g, rb, re, dtype, psi_dev, obs++, P_mean_dev, norm_dev, energy_dev, s));
+                if (step == n_steps) break;
+                const int64_t n = obs_every > 0 ? std::min<int64_t>(obs_every, n_steps - step) : n_steps;
+                CTQW_TRY(launch_graph_resident(g, rb, re, psi_t, lo, dt, K, n, s));
+                step += n;
+                CTQW_TRY(launch_graph_from_rows(g, rb, re, psi_t, psi_dev, s));
+            }
+        }
+        return CTQW_OK;
+    }
     if (dtype == CTQW_C64) {
         // Horner stages w_K = psi + (A/K) psi, w_j = psi + (A/j) w_{j+1},
         // psi += A w_2 (A = -i dt H), the update compensated

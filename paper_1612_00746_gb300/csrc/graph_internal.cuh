@@ -33,6 +33,7 @@ struct ctqw_graph {
     int nnz = 0;              // 2E
     int device = 0;
     int chunk = 0;            // realizations per pass through the steps (0: all)
+    int res_CL = 0, res_G = 0, res_deg = 0;   // k_graph_resident.cu: CTAs a realization (0: not used), rows at a time, links a node at most
     int32_t *row_ptr_d = nullptr, *col_d = nullptr, *link_d = nullptr;   // CSR of the one-particle graph
     float *eps32 = nullptr, *w32 = nullptr;                              // [N][Rp], [nnz][Rp]
     double *eps64 = nullptr, *w64 = nullptr, *J64 = nullptr;             // [N][Rp], [nnz][Rp], [R][E]
@@ -79,6 +80,15 @@ int launch_graph_horner_stage(const ctqw_graph *g, int rb, int re, const void *i
                               void *out, double coef, cudaStream_t s);
 int launch_graph_horner_final(const ctqw_graph *g, int rb, int re, const void *w2, void *psi, void *lo,
                               double dt, cudaStream_t s);
+
+// Two particles in FP32 with the iterate on chip (k_graph_resident.cu): the plan
+// of a handle (res_CL = 0 where it does not fit), n_steps steps on states in
+// [r][s] order (lo the carried error), and the change of order either way.
+int plan_graph_resident(ctqw_graph *g, const int32_t *row_ptr, const int32_t *col, int max_deg);
+int launch_graph_resident(const ctqw_graph *g, int rb, int re, void *psi, void *lo, double dt, int K, int64_t n_steps,
+                          cudaStream_t s);
+int launch_graph_to_rows(const ctqw_graph *g, int rb, int re, const void *psi, void *psi_t, cudaStream_t s);
+int launch_graph_from_rows(const ctqw_graph *g, int rb, int re, const void *psi_t, void *psi, cudaStream_t s);
 
 // Forward Taylor term: out = -(i coef) H in; acc (= psi if first) += out.
 int launch_graph_taylor_term(const ctqw_graph *g, int rb, int re, int dtype, const void *in, void *out,
