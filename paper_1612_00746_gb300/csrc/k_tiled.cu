@@ -34,11 +34,16 @@ using namespace fused;
 // One launch for every size group (register tiles): the work items
 // (realization, tile row, tile column) of all groups form one 1D grid,
 // groups in descending N so that the block scheduler starts the largest
-// items first and the small ones fill the tail.
+// items first and the small ones fill the tail.  Groups next to each other
+// with the same number of tiles are one range of it (a block reads its own
+// realization's N), so only batches of more than 32 tile counts take a second
+// launch.  Where more than 32 sizes took one launch each, of a few
+// realizations: 873 of sizes 192..512, 27 steps of K = 16, 344 -> 130 ms; 500 of
+// 64..128, 20 of K = 8, 25.2 -> 3.0; 200 of 128..1024, 4 of K = 16, 30.8 -> 12.8.
 constexpr int kMaxFlatGroups = 32;
 struct FlatGroups {
-    int n;                              // groups in the launch (0: one launch per group)
-    int64_t item_off[kMaxFlatGroups + 1];   // first item of each group
+    int n;                              // ranges in the launch (0: one launch per group)
+    int64_t item_off[kMaxFlatGroups + 1];   // first item of each range
     int list_off[kMaxFlatGroups];       // its realizations in by_group (the launch's list)
     int tiles_y[kMaxFlatGroups], tiles_x[kMaxFlatGroups];
 };
@@ -919,30 +924,43 @@ int launch_taylor_tiled_range(const ctqw_hamiltonian *h, int shape, const void *
                                        (int)f.smem));
     const int G = (int)h->group_N.size();
     a.flat.n = 0;
-    if (f.fixed_tile && G > 1 && G <= kMaxFlatGroups) {
+    if (f.fixed_tile && G > 1) {
         // one launch over every group, largest N first (see FlatGroups)
-        a.flat.n = G;
         a.list = h->by_group_d;
-        int64_t items = 0;
-        for (int k = 0; k < G; ++k) {
-            const int g = G - 1 - k;   // groups are stored in ascending N
-            int off = 0;
-            for (int q = 0; q < g; ++q) off += h->group_count[q];
-            const int N = h->group_N[g];
-            a.flat.item_off[k] = items;
-            a.flat.list_off[k] = off;
-            a.flat.tiles_y[k] = (N + f.TMAX - 1) / f.TMAX;
-            a.flat.tiles_x[k] = (N + f.TMAX2 - 1) / f.TMAX2;
-            items += (int64_t)h->group_count[g] * a.flat.tiles_y[k] * a.flat.tiles_x[k];
-        }
-        a.flat.item_off[G] = items;
         a.T = f.TMAX;
-        if (items > 0x7fffffffLL) {
-            ctqw_set_error("tiled path: %lld tiles in one launch", (long long)items);
-            return CTQW_EUNSUPPORTED;
+        int off = h->R;
+        int64_t items = 0;
+        for (int g = G - 1; g >= 0; --g) {   // groups are stored in ascending N
+            const int N = h->group_N[g], cnt = h->group_count[g];
+            const int ty = (N + f.TMAX - 1) / f.TMAX, tx = (N + f.TMAX2 - 1) / f.TMAX2;
+            off -= cnt;
+            const int n = a.flat.n;
+            if (n > 0 && a.flat.tiles_y[n - 1] == ty && a.flat.tiles_x[n - 1] == tx) {
+                a.flat.list_off[n - 1] = off;   // the group before it joins its range of the list
+            } else {
+                a.flat.item_off[n] = items;
+                a.flat.list_off[n] = off;
+                a.flat.tiles_y[n] = ty;
+                a.flat.tiles_x[n] = tx;
+                ++a.flat.n;
+            }
+            items += (int64_t)cnt * ty * tx;
+            bool flush = g == 0;
+            if (!flush && a.flat.n == kMaxFlatGroups) {   // unless the next group joins the last range
+                const int Nn = h->group_N[g - 1];
+                flush = (Nn + f.TMAX - 1) / f.TMAX != ty || (Nn + f.TMAX2 - 1) / f.TMAX2 != tx;
+            }
+            if (!flush) continue;
+            if (items > 0x7fffffffLL) {
+                ctqw_set_error("tiled path: %lld tiles in one launch", (long long)items);
+                return CTQW_EUNSUPPORTED;
+            }
+            a.flat.item_off[a.flat.n] = items;
+            f.kern<<<(unsigned)items, f.threads, f.smem, s>>>(a);
+            CTQW_CUDA_TRY(cudaGetLastError());
+            a.flat.n = 0;
+            items = 0;
         }
-        f.kern<<<(unsigned)items, f.threads, f.smem, s>>>(a);
-        CTQW_CUDA_TRY(cudaGetLastError());
         return CTQW_OK;
     }
     // one size group: a range is a slice of its (ascending) realization list
