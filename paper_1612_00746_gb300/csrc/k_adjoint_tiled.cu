@@ -56,6 +56,7 @@ struct ChainArgs {
     int n_stages;                     // stencil stages of the launch
     int init;                         // mu chain: the initial iterate is (i^K / K!) lambda
     int final;                        // mu chain: the last stage is level -1 (lambda_n)
+    int aligned16;                    // every buffer starts on a 16-byte boundary
 };
 
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
@@ -81,20 +82,25 @@ __device__ __forceinline__ float warp_sum32_f(float (&v)[32], int lane) {
 }
 
 // MU = false: the phi chain; MU = true: the mu chain, storing every level's
-// tile for adj_contract_kernel.
+// tile for adj_contract_kernel.  The halo along x2 is D rounded up to a whole
+// pair of columns, so that a lane's pair starts on 16 bytes wherever N is even:
+// N = 512, 64 realizations, K = 14 (D = 7): one phi chain 527 -> 457 us, one mu
+// chain 719 -> 625 us, with 8-byte row coefficients (a broadcast of 16 bytes is
+// four passes of the shared-memory pipe, which bounds these kernels beside the
+// instructions).
 template <int D, int W, bool MU>
 __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_constant__ ChainArgs a) {
-    constexpr int RS = 8 * W, T = RS - 2 * D, T2 = 64 - 2 * D, RL = 8;
+    constexpr int RS = 8 * W, DC = (D + 1) & ~1, T = RS - 2 * D, T2 = 64 - 2 * DC, RL = 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *Q = reinterpret_cast<float4 *>(smem_raw);            // mu chain: [RS][32] lambda, (row, lane) -> 2 columns
     float4 *edge = Q + (MU ? RS * 32 : 0);                        // [2 parity][W warps][2][32]
     float4 *zero = edge + 2 * W * 2 * 32;                         // [32] a row of zeros
-    float4 *rowc = zero + 32;                                     // [RS + 1] (dt eps, dt eps, -dt J_up, -dt J_up)
+    float2 *rowc = reinterpret_cast<float2 *>(zero + 32);         // [RS + 1] (dt eps, -dt J of the bond above)
     int *x_row = reinterpret_cast<int *>(rowc + RS + 1);          // [RS]
 
     const int r = a.list[blockIdx.z];
     const int N = a.tab.N[r];
-    const int x1_0 = (int)blockIdx.y * T - D, x2_0 = (int)blockIdx.x * T2 - D;
+    const int x1_0 = (int)blockIdx.y * T - D, x2_0 = (int)blockIdx.x * T2 - DC;
     const int64_t base = a.tab.st_off[r];
     const int64_t po = a.tab.par_off[r];
     const float dt = a.dt;
@@ -106,7 +112,7 @@ __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_const
         if (i < RS) x_row[i] = X1;
         const float e = i < RS ? dt * a.eps[po + X1] : 0.f;
         const float j = -dt * a.J[po + (X1 + N - 1) % N];
-        rowc[i] = make_float4(e, e, j, j);
+        rowc[i] = make_float2(e, j);
     }
     if (threadIdx.x < 32) zero[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
     int X2[2];
@@ -125,23 +131,52 @@ __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_const
     }
     __syncthreads();
 
+    // pairs of columns are 16 bytes apart and never straddle the wrap
+    const bool vec = a.aligned16 && ((N | (int)(base & 1)) & 1) == 0;
     // the tile's points among this lane's: rows D .. D + T - 1 and columns
-    // D .. D + T2 - 1 of the region that lie inside the lattice
+    // DC .. DC + T2 - 1 of the region that lie inside the lattice
     bool col_in[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int ck = 2 * lane + k;
-        col_in[k] = ck >= D && ck < D + T2 && x2_0 + ck < N;
+        col_in[k] = ck >= DC && ck < DC + T2 && x2_0 + ck < N;
     }
     auto row_in = [&](int ri) { return ri >= D && ri < D + T && x1_0 + ri < N; };
 
     float2 P[RL][2];
+    auto store = [&](float2 *dst) {   // P on the tile
+        if (vec) {
+#pragma unroll
+            for (int i = 0; i < RL; ++i) {
+                const int ri = r0 + i;
+                if (row_in(ri) && col_in[0])
+                    *reinterpret_cast<float4 *>(dst + (int64_t)x_row[ri] * N + X2[0]) =
+                        make_float4(P[i][0].x, P[i][0].y, P[i][1].x, P[i][1].y);
+            }
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < RL; ++i) {
+            const int ri = r0 + i;
+            if (!row_in(ri)) continue;
+            const int64_t grow = (int64_t)x_row[ri] * N;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (col_in[k]) dst[grow + X2[k]] = P[i][k];
+        }
+    };
     if (MU) {
         // lambda of the region into shared memory
         const float2 *gq = a.q + base;
         const uint32_t sQ = smem_u32(Q);
         for (int i = warp; i < RS; i += W) {
             const int64_t grow = (int64_t)x_row[i] * N;
+            if (vec) {
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sQ + (uint32_t)((i * 32 + lane) * 16)),
+                             "l"(gq + grow + X2[0])
+                             : "memory");
+                continue;
+            }
 #pragma unroll
             for (int k = 0; k < 2; ++k)
                 asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sQ + (uint32_t)((i * 32 + lane) * 16 + 8 * k)),
@@ -153,9 +188,15 @@ __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_const
         const float2 *win = a.in + base;
 #pragma unroll
         for (int i = 0; i < RL; ++i) {
-            const int64_t grow = (int64_t)x_row[r0 + i] * N;
-            P[i][0] = win[grow + X2[0]];
-            P[i][1] = win[grow + X2[1]];
+            const float2 *g = win + (int64_t)x_row[r0 + i] * N;
+            if (vec) {
+                const float4 v = *reinterpret_cast<const float4 *>(g + X2[0]);
+                P[i][0] = make_float2(v.x, v.y);
+                P[i][1] = make_float2(v.z, v.w);
+            } else {
+                P[i][0] = g[X2[0]];
+                P[i][1] = g[X2[1]];
+            }
         }
     }
     if (MU) {
@@ -171,17 +212,7 @@ __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_const
             P[i][0] = cmulf(co, make_float2(q.x, q.y));
             P[i][1] = cmulf(co, make_float2(q.z, q.w));
         }
-        // the first level's tile
-        float2 *dst = a.mlev[a.a_in] + base;
-#pragma unroll
-        for (int i = 0; i < RL; ++i) {
-            const int ri = r0 + i;
-            if (!row_in(ri)) continue;
-            const int64_t grow = (int64_t)x_row[ri] * N;
-#pragma unroll
-            for (int k = 0; k < 2; ++k)
-                if (col_in[k]) dst[grow + X2[k]] = P[i][k];
-        }
+        store(a.mlev[a.a_in] + base);   // the first level's tile
     }
 
     const float2 dU = make_float2(a.dtU, a.dtU);
@@ -198,7 +229,7 @@ __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_const
         const float4 u4 = warp > 0 ? edge[(par * W + warp - 1) * 2 * 32 + 32 + lane] : zero[lane];
         const float4 d4 = warp < W - 1 ? edge[(par * W + warp + 1) * 2 * 32 + lane] : zero[lane];
         float2 prev[2] = {make_float2(u4.x, u4.y), make_float2(u4.z, u4.w)};
-        float4 rc = rowc[r0];
+        float2 rc = rowc[r0];
         const float2 co = MU ? a.co[lev + 1] : make_float2(0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < RL; ++i) {
@@ -206,8 +237,8 @@ __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_const
             const float2 lft = shfl2(c1, from_left), rgt = shfl2(c0, from_right);
             const float2 n0 = i < RL - 1 ? P[i + 1][0] : make_float2(d4.x, d4.y);
             const float2 n1 = i < RL - 1 ? P[i + 1][1] : make_float2(d4.z, d4.w);
-            const float4 rn = rowc[r0 + i + 1];
-            const float2 er = make_float2(rc.x, rc.y), jup = make_float2(rc.z, rc.w), jdn = make_float2(rn.z, rn.w);
+            const float2 rn = rowc[r0 + i + 1];
+            const float2 er = make_float2(rc.x, rc.x), jup = make_float2(rc.y, rc.y), jdn = make_float2(rn.y, rn.y);
             rc = rn;
             // y = Hh P: the diagonal (column and row eps), the bonds above and
             // below, left and right, and dt U where x1 = x2
@@ -240,16 +271,7 @@ __global__ void __launch_bounds__(32 * W, 3) adj_chain_kernel(const __grid_const
         const bool last = d == a.n_stages;
         if (!MU || lev >= 0 || (a.final && last)) {
             // the phi level, lambda_n, or the stored mu level, on the tile
-            float2 *dst = !MU ? a.lev[lev] + base : (lev < 0 ? a.out + base : a.mlev[lev] + base);
-#pragma unroll
-            for (int i = 0; i < RL; ++i) {
-                const int ri = r0 + i;
-                if (!row_in(ri)) continue;
-                const int64_t grow = (int64_t)x_row[ri] * N;
-#pragma unroll
-                for (int k = 0; k < 2; ++k)
-                    if (col_in[k]) dst[grow + X2[k]] = P[i][k];
-            }
+            store(!MU ? a.lev[lev] + base : (lev < 0 ? a.out + base : a.mlev[lev] + base));
         }
     }
 }
@@ -430,13 +452,20 @@ ChainShape chain_shape() {
     ChainShape s;
     s.D = D;
     s.T = RS - 2 * D;
-    s.T2 = 64 - 2 * D;
+    s.T2 = 64 - 2 * ((D + 1) & ~1);
     s.threads = 32 * W;
     s.phi = adj_chain_kernel<D, W, false>;
     s.mu = adj_chain_kernel<D, W, true>;
-    s.smem_phi = sizeof(float4) * (2 * W * 2 * 32 + 32 + RS + 1) + sizeof(int) * RS;
+    s.smem_phi = sizeof(float4) * (2 * W * 2 * 32 + 32) + sizeof(float2) * (RS + 1) + sizeof(int) * RS;
     s.smem_mu = s.smem_phi + sizeof(float4) * RS * 32;
     return s;
+}
+
+// Whether every buffer of the launch starts on a 16-byte boundary.
+bool chain_aligned16(const ChainArgs &a) {
+    uintptr_t all = (uintptr_t)a.in | (uintptr_t)a.q | (uintptr_t)a.out;
+    for (int i = 0; i < kMaxLevels; ++i) all |= (uintptr_t)a.lev[i] | (uintptr_t)a.mlev[i];
+    return (all & 15) == 0;
 }
 
 // Depth for K levels: the fewest launches at depth <= 8, the levels split
@@ -473,6 +502,7 @@ ChainArgs chain_args(const ctqw_hamiltonian *h, double dt) {
     a.n_stages = 0;
     a.init = 0;
     a.final = 0;
+    a.aligned16 = 0;
     return a;
 }
 
@@ -505,6 +535,7 @@ int launch_adjoint_phi_chain(const ctqw_hamiltonian *h, int K, double dt, void *
         a.in = (const float2 *)levels[a0];
         a.a_in = a0;
         a.n_stages = n;
+        a.aligned16 = chain_aligned16(a);
         int off = 0;
         for (size_t g = 0; g < h->group_N.size(); ++g) {
             const int N = h->group_N[g], cnt = h->group_count[g];
@@ -540,6 +571,7 @@ int launch_adjoint_mu_chain(const ctqw_hamiltonian *h, int K, double dt, const v
         a.n_stages = n;
         a.init = init ? 1 : 0;
         a.final = final ? 1 : 0;
+        a.aligned16 = chain_aligned16(a);
         int off = 0;
         for (size_t g = 0; g < h->group_N.size(); ++g) {
             const int N = h->group_N[g], cnt = h->group_count[g];

@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(256) taylor_tiled_kernel(const __grid_constant
 }
 
 // The same D stages with the iterate in registers: the region is 8W rows x
-// 64 columns (tile (8W - 2D) x (64 - 2D)), every warp holds 8 region rows
+// 64 columns (tile (8W - 2D) x (64 - 2 DC), DC = D or D + 1), every warp holds 8 region rows
 // and every lane the two adjacent columns 2l, 2l+1 of them.  Neighbours along x2 are in the lane or
 // one 64-bit shuffle away; along x1 in registers except the warp's first
 // and last rows, which pass through shared memory once per stage (one
@@ -264,10 +264,17 @@ __global__ void __launch_bounds__(256) taylor_tiled_kernel(const __grid_constant
 // error words read in the final stage and psi read twice, 79.9 ms with both
 // fetched at the start, 74.2 ms with the 8-byte coefficients and the regions
 // that tiled_default_shape picks.
+//
+// The halo along x2 is D rounded up to a whole pair of columns, so a lane's
+// pair starts on 16 bytes at odd depths too (even N): one 16-byte copy where
+// there were two of 8.  10 steps: 64 x N = 512, K = 14 (D = 7) 5.97 -> 5.07 ms,
+// K = 10 (D = 5) 4.44 -> 3.67; 16 x N = 1000, K = 7 2.80 -> 2.35; odd N, which
+// has 8-byte copies either way, 64 x N = 301, K = 14 2.48 -> 2.53.
 template <int D, int W>
 struct RegTile {
     static constexpr int RS = 8 * W, RL = 8;              // region rows, rows a warp
-    static constexpr int T = RS - 2 * D, T2 = 64 - 2 * D;   // tile rows and columns
+    static constexpr int DC = (D + 1) & ~1;               // halo along x2: whole pairs of columns
+    static constexpr int T = RS - 2 * D, T2 = 64 - 2 * DC;  // tile rows and columns
     static constexpr size_t q_bytes = sizeof(float4) * RS * 32;
     static constexpr size_t lo_bytes = (sizeof(float2) * T * T2 + 15) / 16 * 16;
     static constexpr size_t edge_bytes = sizeof(float4) * 2 * W * 2 * 32;
@@ -311,7 +318,7 @@ __device__ __forceinline__ void reg_stencil_row(const float2 (&P)[8][2], int i, 
 template <int D, int W>
 __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kernel(const __grid_constant__ TiledArgs a) {
     using Tile = RegTile<D, W>;
-    constexpr int RS = Tile::RS, T = Tile::T, T2 = Tile::T2, RL = Tile::RL;
+    constexpr int RS = Tile::RS, T = Tile::T, T2 = Tile::T2, RL = Tile::RL, DC = Tile::DC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *Q = reinterpret_cast<float4 *>(smem_raw);                        // [RS][32] psi, (row, lane) -> 2 columns
     float2 *los = reinterpret_cast<float2 *>(smem_raw + Tile::q_bytes);      // [T][T2] carried error of the tile
@@ -323,7 +330,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kerne
     const TileItem item = tile_item(a);
     const int r = item.r;
     const int N = a.tab.N[r];
-    const int x1_0 = item.ty * T - D, x2_0 = item.tx * T2 - D;
+    const int x1_0 = item.ty * T - D, x2_0 = item.tx * T2 - DC;
     const int64_t base = a.tab.st_off[r];
     const int64_t po = a.tab.par_off[r];
     const float dt = a.dt;
@@ -338,13 +345,13 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kerne
 #pragma unroll
     for (int k = 0; k < 2; ++k) X2[k] = wrap(x2_0 + 2 * lane + k);
     // pairs of columns are 16 bytes apart and never straddle the wrap
-    const bool vec = a.aligned16 && D % 2 == 0 && ((N | (int)(base & 1)) & 1) == 0;
+    const bool vec = a.aligned16 && ((N | (int)(base & 1)) & 1) == 0;
     // the tile's part of this lane and warp
     bool col_in[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
         const int ck = 2 * lane + k;
-        col_in[k] = ck >= D && ck < D + T2 && x2_0 + ck < N;
+        col_in[k] = ck >= DC && ck < DC + T2 && x2_0 + ck < N;
     }
     auto row_in = [&](int ri) { return ri >= D && ri < D + T && x1_0 + ri < N; };
 
@@ -352,7 +359,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kerne
     const bool carried = a.final && a.compensated;
     const uint32_t sQ = smem_u32(Q) + (uint32_t)(r0 * 32 + lane) * 16u;
     // slot of (row, column) of the tile: negative rows and columns are never touched
-    const int lo_at = (r0 - D) * T2 + 2 * lane - D;
+    const int lo_at = (r0 - D) * T2 + 2 * lane - DC;
     const uint32_t sL = smem_u32(los);
     float2 P[RL][2];
     if (vec) {
@@ -789,7 +796,8 @@ TiledShape tiled_wide_shape() {
 // regions of at most 64 x 64 (two 32-lane column passes per row); shapes
 // 3..10: the iterate in registers at depths 4, 8, 2, 7, 6, 5, 3 and 1;
 // 11, 12: registers on 64 x 128 regions at depths 8 and 4; 13, 14:
-// registers on 96 x 64 regions (12 warps) at depths 8 and 7
+// registers on 96 x 64 regions (12 warps) at depths 8 and 7 (tiles: 2D less, along
+// x2 at odd depths 2D + 2 less)
 constexpr int kTiledShapes = 15;
 
 bool tiled_shape_for(int idx, TiledShape &s) {
