@@ -13,13 +13,16 @@
 // a_lo b_hi (the dropped a_lo b_lo is ~2^-22 of it).
 //
 // Only the 128 x 128 tiles (x, x') with x / 128 <= x' / 128 are computed;
-// the rest of rho1 is their conjugate transpose.  A CTA owns one tile and a
+// the rest of rho1 is their conjugate transpose.  A tile on the diagonal has
+// the same rows on both sides: they are loaded and split once, by both halves
+// of the producers, and its Im takes Z = Ai Ar^T alone (Im = Z - Z^T), nine
+// products instead of twelve.  A CTA owns one tile and a
 // range of (realization, particle) pairs, and its warps have three roles:
 //  - warps 0-7 (producers) load 16 k at a time of the tile's 128 + 128 rows,
 //    split them into the four TF32 arrays re_hi, re_lo, im_hi, im_lo and
 //    store them into a three-stage shared-memory ring in the MMA's
 //    canonical K-major layout (8-row by 16-byte core matrices);
-//  - one thread of warp 8 issues 12 MMAs per 8 k (M = 128, N = 128, K = 8,
+//  - one thread of warp 8 issues 12 (9) MMAs per 8 k (M = 128, N = 128, K = 8,
 //    FP32 accumulate in TMEM: 128 columns for Re, 128 for Im) and commits
 //    them to the stage's mbarrier, which hands the stage back;
 //  - warps 9-12 drain: every 256 k the MMAs switch to the other of two TMEM
@@ -30,7 +33,12 @@
 //    |terms| (the adds may round toward zero): at most 256 x 2^-23 of the
 //    largest element of rho1.
 // A second kernel sums the slots of all CTAs in FP64 and fills the lower
-// triangle.  Every wait is bounded in time (status word, then the CTA stops).
+// triangle.  The producers' loads and stores bound an off-diagonal tile, so a
+// diagonal one takes less time, and the (realization, particle) pairs are
+// split over more CTAs of the one than of the other (see density_splits).  1024
+// realizations of N = 256: 1.05 ms and 0.06 ms for the sum of the slots -> 0.92
+// and 0.02 ms.  Every wait is bounded in time (status word, then the CTA stops).
+#include <algorithm>
 #include <cstdint>
 
 #include "ctqw_internal.cuh"
@@ -56,7 +64,8 @@ struct TcArgs {
     int *status;
     int N, m, pairs;         // pairs = R_g m
     int tiles;               // tiles per side, ceil(N / 128)
-    int pairs_per_split;
+    int off_ctas;            // CTAs of the tiles above the diagonal; those on it follow (-1: tile by tile)
+    int off_pairs, diag_pairs;   // pairs a CTA
     int64_t n_k;             // N^(m-1)
 };
 
@@ -165,15 +174,33 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
     __shared__ int stop;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int N = a.N, m = a.m;
-    // blockIdx.x: a tile (ty <= tx) of the upper triangle, row by row; the
-    // lower one is its conjugate transpose (rho1 is Hermitian)
-    int ty = 0, rest = blockIdx.x;
-    while (rest >= a.tiles - ty) rest -= a.tiles - ty++;
-    const int x0 = ty * kM, xp0 = (ty + rest) * kNt;
-    const int p0 = blockIdx.y * a.pairs_per_split;
-    const int p1 = min(a.pairs, p0 + a.pairs_per_split);
-    const int cta = blockIdx.y * gridDim.x + blockIdx.x;
-    float *slot = a.slots + (size_t)cta * (2 * 2 * kNt * kM);
+    // blockIdx.x: (split, tile) row by row over the upper triangle, or, where
+    // the diagonal has splits of its own, first the tiles above it, then those
+    // on it; the lower triangle is the upper one's conjugate transpose (rho1 is
+    // Hermitian)
+    int ty = 0, tx = 0, split, per = a.off_pairs;
+    if (a.off_ctas < 0) {
+        const int n_up = a.tiles * (a.tiles + 1) / 2;
+        split = (int)blockIdx.x / n_up;
+        int rest = (int)blockIdx.x - split * n_up;
+        while (rest >= a.tiles - ty) rest -= a.tiles - ty++;
+        tx = ty + rest;
+    } else if ((int)blockIdx.x >= a.off_ctas) {
+        split = ((int)blockIdx.x - a.off_ctas) / a.tiles;
+        ty = tx = (int)blockIdx.x - a.off_ctas - split * a.tiles;
+        per = a.diag_pairs;
+    } else {
+        const int n_off = a.tiles * (a.tiles - 1) / 2;
+        split = (int)blockIdx.x / n_off;
+        int rest = (int)blockIdx.x - split * n_off;
+        while (rest >= a.tiles - 1 - ty) rest -= a.tiles - 1 - ty++;
+        tx = ty + 1 + rest;
+    }
+    const bool diag = tx == ty;
+    const int x0 = ty * kM, xp0 = tx * kNt;
+    const int p0 = split * per;
+    const int p1 = min(a.pairs, p0 + per);
+    float *slot = a.slots + (size_t)blockIdx.x * (2 * 2 * kNt * kM);
 
     if (tid == 0) {
         for (int i = 0; i < kStages; ++i) {
@@ -215,15 +242,18 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
         // quarter warp writes 128 contiguous bytes of shared memory:
         //   x contiguous (S_k = N): lane = row, group q = k / 4;
         //   k contiguous (S_k = 1): lane = 8 (k / 4) + row % 8, group q = row / 8 % 4.
+        // On the diagonal both sides are the same rows: warps 0-3 stage groups
+        // 0 and 1 of them, warps 4-7 groups 2 and 3.
         const int side = warp >> 2, row0 = 32 * (warp & 3);
+        const int q0 = diag ? 2 * side : 0, to = diag ? 0 : side * 4 * kArr;
         const int xA = (side ? xp0 : x0) + row0 + lane;
         int xB[4], soffA[4], soffB[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int rowB = row0 + 8 * q + (lane & 7);
+            const int rowB = row0 + 8 * ((q0 + q) & 3) + (lane & 7);
             xB[q] = (side ? xp0 : x0) + rowB;
-            soffA[q] = side * 4 * kArr + canon(row0 + lane, 4 * q);
-            soffB[q] = side * 4 * kArr + canon(rowB, 4 * (lane >> 3));
+            soffA[q] = to + canon(row0 + lane, 4 * ((q0 + q) & 3));
+            soffB[q] = to + canon(rowB, 4 * (lane >> 3));
         }
         // The chunk the next load reads: amplitude (x, k0 + kk) of pair p sits
         // at base + x S_x + kk S_k.  With the partial trace over particle j,
@@ -271,6 +301,7 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
                 const int k4 = lane >> 3;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
+                    if (q == 2 && diag) break;
                     float4 u0 = make_float4(0.f, 0.f, 0.f, 0.f), u1 = u0;
                     if (xB[q] < N) {
                         const float4 *src = (const float4 *)(a.psi + base + (int64_t)xB[q] * S_x + 4 * k4);
@@ -283,12 +314,14 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
                     v[4 * q + 3] = make_float2(u1.z, u1.w);
                 }
             } else {
-                const float2 *src = a.psi + base + xA;
+                const float2 *src = a.psi + base + xA + 4 * q0 * S_k;
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
+                for (int q = 0; q < 4; ++q) {
+                    if (q == 2 && diag) break;
 #pragma unroll
                     for (int t = 0; t < 4; ++t)
                         v[4 * q + t] = xA < N ? __ldg(src + (int64_t)(4 * q + t) * S_k) : make_float2(0.f, 0.f);
+                }
             }
             advance();
         };
@@ -306,6 +339,7 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
             float *st = smem + s * 8 * kArr;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
+                if (q == 2 && diag) break;
                 float4 rh, rl, ih, il;
                 float *ph = &rh.x, *pl = &rl.x, *qh = &ih.x, *ql = &il.x;
 #pragma unroll
@@ -358,7 +392,7 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t d = tmem + (uint32_t)(256 * acc);
                 const float *st = smem + s * 8 * kArr;
-                const uint32_t sa = smem_u32(st), sb = smem_u32(st + 4 * kArr);
+                const uint32_t sa = smem_u32(st), sb = diag ? sa : smem_u32(st + 4 * kArr);
 #pragma unroll
                 for (int ks = 0; ks < kKc / 8; ++ks) {
                     const uint32_t koff = (uint32_t)ks * 2 * kLbo;
@@ -372,10 +406,11 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
                     mma_tf32(d, A(2), B(2), id_pos, 1u);
                     mma_tf32(d, A(2), B(3), id_pos, 1u);
                     mma_tf32(d, A(3), B(2), id_pos, 1u);
-                    // Im += Ai Br - Ar Bi
+                    // Im += Ai Br - Ar Bi (on the diagonal Ai Br, see the reduction)
                     mma_tf32(d + kNt, A(2), B(0), id_pos, first);
                     mma_tf32(d + kNt, A(2), B(1), id_pos, 1u);
                     mma_tf32(d + kNt, A(3), B(0), id_pos, 1u);
+                    if (diag) continue;
                     mma_tf32(d + kNt, A(0), B(2), id_neg, 1u);
                     mma_tf32(d + kNt, A(0), B(3), id_neg, 1u);
                     mma_tf32(d + kNt, A(1), B(2), id_neg, 1u);
@@ -420,7 +455,7 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
                     const size_t o = (size_t)(c0 - part * kNt + i) * kM + row;
-                    float h = hi[o], l = lo[o];
+                    float h = bi > 0 ? hi[o] : 0.f, l = bi > 0 ? lo[o] : 0.f;
                     two_sum_add(h, l, tv[i]);
                     hi[o] = h;
                     lo[o] = l;
@@ -438,32 +473,123 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
     if (warp == kMmaWarp) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
-// rho1(x, x') = scale * sum over the splits of (hi + lo), in FP64, read
-// from tile (x / 128, x' / 128) of the upper triangle, or conjugated from
-// its transpose below the diagonal.
-__global__ void __launch_bounds__(256) rho1_tc_reduce_kernel(const float *__restrict__ slots, int tiles, int splits,
-                                                             int N, double scale, double *__restrict__ rho) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= (int64_t)N * N) return;
-    int x = (int)(i / N), xp = (int)(i - (int64_t)x * N);
-    const bool lower = x / kM > xp / kNt;
-    if (lower) {
-        const int t = x;
-        x = xp;
-        xp = t;
+// The CTAs' slots of a tile summed over the splits: sums[tile][re, im][column]
+// [row].  Each 32 rows of a column are `share` warps' (8, or fewer for fewer
+// splits), every share-th split of a warp in two FP32 words, as the CTAs' own
+// totals, and the warps' sums in FP64.
+// (3 tiles of 50 splits: one thread walking all splits of an element in FP64,
+// the lower triangle read across the rows, 61 us; 8 warps in FP64, whose
+// conversions and adds then bound it, 44; now 12.)
+constexpr int kRedWarps = 8;
+__global__ void __launch_bounds__(32 * kRedWarps) rho1_tc_reduce_kernel(const float *__restrict__ slots, int tiles,
+                                                                        int off_splits, int diag_splits, int share,
+                                                                        double *__restrict__ sums) {
+    __shared__ double part[2][kRedWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_off = tiles * (tiles - 1) / 2, id = blockIdx.y;   // tiles above the diagonal, then those on it
+    const bool diag = id >= n_off;
+    const int w0 = warp & ~(share - 1);   // the first of this warp's share
+    const size_t o = ((size_t)blockIdx.x * (kRedWarps / share) + warp / share) * 32 + lane, plane = (size_t)kNt * kM;
+    int splits = off_splits, step = n_off, first = id;
+    if (diag_splits == 0) {   // the same splits for all, tile by tile over the upper triangle
+        step = n_off + tiles;
+        int ty = 0, rest = diag ? 0 : id;
+        if (diag) ty = id - n_off;
+        while (!diag && rest >= tiles - 1 - ty) rest -= tiles - 1 - ty++;
+        first = ty * tiles - ty * (ty - 1) / 2 + (diag ? 0 : 1 + rest);
+    } else if (diag) {
+        splits = diag_splits;
+        step = tiles;
+        first = n_off * off_splits + id - n_off;
     }
-    const int ty = x / kM, tx = xp / kNt, row = x - ty * kM, col = xp - tx * kNt;
-    const int n_up = tiles * (tiles + 1) / 2;
-    const int id = ty * tiles - ty * (ty - 1) / 2 + (tx - ty);
+    const float *slot0 = slots + (size_t)first * (4 * plane);
+    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+#pragma unroll 4
+    for (int s = warp - w0; s < splits; s += share) {
+        const float *slot = slot0 + (size_t)s * step * (4 * plane);
+        two_sum_add(rh, rl, slot[o]);
+        two_sum_add(ih, il, slot[plane + o]);
+        rl = __fadd_rn(rl, slot[2 * plane + o]);
+        il = __fadd_rn(il, slot[3 * plane + o]);
+    }
+    part[0][warp][lane] = (double)rh + (double)rl;
+    part[1][warp][lane] = (double)ih + (double)il;
+    __syncthreads();
+    if (warp != w0) return;
     double re = 0.0, im = 0.0;
-    for (int s = 0; s < splits; ++s) {
-        const float *slot = slots + (size_t)(s * n_up + id) * (2 * 2 * kNt * kM);
-        const size_t o = (size_t)col * kM + row;
-        re += (double)slot[o] + (double)slot[2 * kNt * kM + o];
-        im += (double)slot[kNt * kM + o] + (double)slot[3 * kNt * kM + o];
+    for (int w = w0; w < w0 + share; ++w) {
+        re += part[0][w][lane];
+        im += part[1][w][lane];
     }
-    rho[2 * i] += scale * re;
-    rho[2 * i + 1] += scale * (lower ? -im : im);
+    sums[(size_t)(2 * id) * plane + o] = re;
+    sums[(size_t)(2 * id + 1) * plane + o] = im;
+}
+
+// rho1(x, x') += scale * the tile's sum; on the diagonal Im = Z - Z^T, and
+// below it the conjugate of the transposed tile.  Block: 32 x 32 of a tile,
+// turned in shared memory so that reads and writes both run along rows.
+__global__ void __launch_bounds__(256) rho1_tc_spread_kernel(const double *__restrict__ sums, int tiles, int N,
+                                                             double scale, double *__restrict__ rho) {
+    __shared__ double re[32][33], im[32][33], zt[32][33];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n_off = tiles * (tiles - 1) / 2, id = blockIdx.y;
+    const bool diag = id >= n_off;
+    int ty = 0, tx = 0;
+    if (diag) {
+        ty = tx = id - n_off;
+    } else {
+        int rest = id;
+        while (rest >= tiles - 1 - ty) rest -= tiles - 1 - ty++;
+        tx = ty + 1 + rest;
+    }
+    const int r0 = 32 * (blockIdx.x % (kM / 32)), c0 = 32 * (blockIdx.x / (kM / 32));
+    const size_t plane = (size_t)kNt * kM;
+    const double *t = sums + (size_t)(2 * id) * plane;
+    for (int k = warp; k < 32; k += 8) {
+        re[k][lane] = t[(size_t)(c0 + k) * kM + r0 + lane];
+        im[k][lane] = t[plane + (size_t)(c0 + k) * kM + r0 + lane];
+        if (diag) zt[k][lane] = t[plane + (size_t)(r0 + k) * kM + c0 + lane];
+    }
+    __syncthreads();
+    const int x0 = ty * kM + r0, xp0 = tx * kNt + c0;
+    for (int k = warp; k < 32; k += 8) {
+        if (x0 + k < N && xp0 + lane < N) {
+            const int64_t i = (int64_t)(x0 + k) * N + xp0 + lane;
+            rho[2 * i] += scale * re[lane][k];
+            rho[2 * i + 1] += scale * (im[lane][k] - (diag ? zt[k][lane] : 0.0));
+        }
+        if (!diag && xp0 + k < N && x0 + lane < N) {
+            const int64_t i = (int64_t)(xp0 + k) * N + x0 + lane;
+            rho[2 * i] += scale * re[k][lane];
+            rho[2 * i + 1] += scale * -im[k][lane];
+        }
+    }
+}
+
+// How many CTAs share the pairs of an off-diagonal tile and of a diagonal one:
+// one wave of CTAs of the least longest time, a diagonal tile counting
+// kDiagCost, if that is 5% below as many for every tile (which reads the same
+// states at the same time).  Alone a diagonal tile takes 0.78 of its former time (N = 128, 2048
+// realizations: 368 -> 285 us); beside the others 0.7 gave the better splits (N =
+// 256: 64 + 2 x 44 CTAs 918 us, 60 + 2 x 46 972, 3 x 50 before 1050).
+constexpr double kDiagCost = 0.7;
+
+void density_splits(int sms, int tiles, int pairs, int &off, int &diag) {
+    const int n_off = tiles * (tiles - 1) / 2;
+    auto each = [pairs](int splits) { return (pairs + splits - 1) / splits; };
+    off = diag = std::max(1, std::min(pairs, sms / (n_off + tiles)));
+    double best = 0.95 * each(off);
+    for (int so = 1; n_off > 0 && so <= std::min(pairs, sms / n_off); ++so) {
+        int sd = std::min(pairs, (sms - n_off * so) / tiles);
+        if (sd < 1) break;
+        const double t = std::max((double)each(so), kDiagCost * each(sd));
+        while (sd > 1 && kDiagCost * each(sd - 1) <= t) --sd;
+        if (t < best) {
+            best = t;
+            off = so;
+            diag = sd;
+        }
+    }
 }
 
 }  // namespace
@@ -489,17 +615,18 @@ int launch_one_body_density_tc(const ctqw_hamiltonian *h, const void *psi, doubl
         for (int j = 1; j < h->m; ++j) n_k *= N;
         const int tiles = (N + kM - 1) / kM, n_up = tiles * (tiles + 1) / 2;
         const int pairs = cnt * h->m;
-        int splits = std::max(1, sms / n_up);
-        splits = std::min(splits, pairs);
-        const int pps = (pairs + splits - 1) / splits;
-        splits = (pairs + pps - 1) / pps;
-        const size_t slot_floats = (size_t)n_up * splits * (2 * 2 * kNt * kM);
+        const int n_off = n_up - tiles;
+        int so = 1, sd = 1;
+        density_splits(sms, tiles, pairs, so, sd);
+        const int po = (pairs + so - 1) / so, pd = (pairs + sd - 1) / sd;
+        so = (pairs + po - 1) / po;
+        sd = (pairs + pd - 1) / pd;
+        const int ctas = n_off * so + tiles * sd;
+        const size_t slot_floats = (size_t)(ctas + n_up) * (2 * 2 * kNt * kM);   // and the tiles' FP64 sums
         float *slots = nullptr;
         CTQW_CUDA_TRY(ctqw_malloc_async((void **)&slots, slot_floats * sizeof(float), s));
         int st = CTQW_OK;
-        const cudaError_t em = cudaMemsetAsync(slots, 0, slot_floats * sizeof(float), s);
-        if (em != cudaSuccess) st = ctqw_cuda_fail(em, "memset of the rho1 slots");
-        if (st == CTQW_OK) {
+        {
             TcArgs a;
             a.tab = real_table(h);
             a.list = h->by_group_d + off;
@@ -509,17 +636,23 @@ int launch_one_body_density_tc(const ctqw_hamiltonian *h, const void *psi, doubl
             a.N = N;
             a.m = h->m;
             a.pairs = pairs;
-            a.pairs_per_split = pps;
+            a.off_ctas = so == sd ? -1 : n_off * so;
+            a.off_pairs = po;
+            a.diag_pairs = pd;
             a.n_k = n_k;
             a.tiles = tiles;
-            rho1_tc_kernel<<<dim3((unsigned)n_up, (unsigned)splits), kThreads, smem, s>>>(a);
+            rho1_tc_kernel<<<(unsigned)ctas, kThreads, smem, s>>>(a);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) st = ctqw_cuda_fail(e, "rho1 tensor-core launch");
         }
         if (st == CTQW_OK) {
-            const int64_t n = (int64_t)N * N;
-            rho1_tc_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
-                slots, tiles, splits, N, 1.0 / ((double)cnt * h->m), rho + 2 * h->joint_off[g]);
+            double *sums = (double *)(slots + (size_t)ctas * (2 * 2 * kNt * kM));
+            int share = 1;
+            while (share < kRedWarps && 2 * share <= std::max(so, sd)) share *= 2;
+            rho1_tc_reduce_kernel<<<dim3(kNt * kM / 32 / (kRedWarps / share), (unsigned)n_up), 32 * kRedWarps, 0, s>>>(
+                slots, tiles, so, so == sd ? 0 : sd, share, sums);
+            rho1_tc_spread_kernel<<<dim3((kM / 32) * (kNt / 32), (unsigned)n_up), 256, 0, s>>>(
+                sums, tiles, N, 1.0 / ((double)cnt * h->m), rho + 2 * h->joint_off[g]);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) st = ctqw_cuda_fail(e, "rho1 reduction launch");
         }
