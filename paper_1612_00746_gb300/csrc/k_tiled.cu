@@ -268,12 +268,12 @@ __global__ void __launch_bounds__(256) taylor_tiled_kernel(const __grid_constant
 // The halo along x2 is D rounded up to a whole pair of columns, so a lane's
 // pair starts on 16 bytes at odd depths too (even N): one 16-byte copy where
 // there were two of 8.  10 steps: 64 x N = 512, K = 14 (D = 7) 5.97 -> 5.07 ms,
-// K = 10 (D = 5) 4.44 -> 3.67; 16 x N = 1000, K = 7 2.80 -> 2.35; odd N, which
-// has 8-byte copies either way, 64 x N = 301, K = 14 2.48 -> 2.53.
-template <int D, int W>
+// K = 10 (D = 5) 4.44 -> 3.67; 16 x N = 1000, K = 7 2.80 -> 2.35.  FLUSH keeps a
+// halo of D columns at odd depths (settle_columns).
+template <int D, int W, bool FLUSH>
 struct RegTile {
     static constexpr int RS = 8 * W, RL = 8;              // region rows, rows a warp
-    static constexpr int DC = (D + 1) & ~1;               // halo along x2: whole pairs of columns
+    static constexpr int DC = FLUSH ? D : (D + 1) & ~1;   // halo along x2: whole pairs of columns
     static constexpr int T = RS - 2 * D, T2 = 64 - 2 * DC;  // tile rows and columns
     static constexpr size_t q_bytes = sizeof(float4) * RS * 32;
     static constexpr size_t lo_bytes = (sizeof(float2) * T * T2 + 15) / 16 * 16;
@@ -315,9 +315,9 @@ __device__ __forceinline__ void reg_stencil_row(const float2 (&P)[8][2], int i, 
     }
 }
 
-template <int D, int W>
+template <int D, int W, bool FLUSH>
 __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kernel(const __grid_constant__ TiledArgs a) {
-    using Tile = RegTile<D, W>;
+    using Tile = RegTile<D, W, FLUSH>;
     constexpr int RS = Tile::RS, T = Tile::T, T2 = Tile::T2, RL = Tile::RL, DC = Tile::DC;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *Q = reinterpret_cast<float4 *>(smem_raw);                        // [RS][32] psi, (row, lane) -> 2 columns
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(32 * W, W == 8 ? 3 : 2) taylor_tiled_reg_kerne
 #pragma unroll
     for (int k = 0; k < 2; ++k) X2[k] = wrap(x2_0 + 2 * lane + k);
     // pairs of columns are 16 bytes apart and never straddle the wrap
-    const bool vec = a.aligned16 && ((N | (int)(base & 1)) & 1) == 0;
+    const bool vec = a.aligned16 && DC % 2 == 0 && ((N | (int)(base & 1)) & 1) == 0;
     // the tile's part of this lane and warp
     bool col_in[2];
 #pragma unroll
@@ -750,6 +750,10 @@ struct TiledShape {
     bool fixed_tile;   // the register kernels: tile TMAX (rows) x TMAX2 (columns) exactly
     int TMAX2;
     int threads = 256;
+    // odd depths: the same with a halo of D columns (see settle_columns)
+    TiledKernel kern_flush = nullptr;
+    size_t smem_flush = 0;
+    int T2_flush = 0;
 };
 
 template <int TMAX, int D>
@@ -768,15 +772,20 @@ TiledShape tiled_shape() {
 
 template <int D, int W = 8>
 TiledShape tiled_reg_shape() {
-    using Tile = RegTile<D, W>;
+    using Tile = RegTile<D, W, false>;
     TiledShape s;
     s.TMAX = Tile::T;
     s.TMAX2 = Tile::T2;
     s.D = D;
-    s.kern = taylor_tiled_reg_kernel<D, W>;
+    s.kern = taylor_tiled_reg_kernel<D, W, false>;
     s.smem = Tile::smem;
     s.fixed_tile = true;
     s.threads = 32 * W;
+    if (D % 2) {
+        s.kern_flush = taylor_tiled_reg_kernel<D, W, true>;
+        s.T2_flush = RegTile<D, W, true>::T2;
+        s.smem_flush = RegTile<D, W, true>::smem;
+    }
     return s;
 }
 
@@ -823,6 +832,30 @@ bool tiled_shape_for(int idx, TiledShape &s) {
 
 }  // namespace
 
+// At an odd depth the halo of whole column pairs costs two columns of the tile
+// and saves half the copies of lattices of even N.  Odd N has no aligned pairs
+// to copy, so there (every size odd) the tiles keep the two columns; and so
+// they do where that needs fewer tiles by more than the 15% that the copies
+// are worth (K = 14, 64 x N = 512: 5.97 against 5.07 ms).  7 x N = 771, K = 19, 37
+// steps: 8.96 ms with pairs, 7.86 without.  Returns the cost against a tile of pairs.
+static double settle_columns(const ctqw_hamiltonian *h, TiledShape &f) {
+    if (!f.kern_flush) return 1.0;
+    double pairs = 0.0, flush = 0.0;
+    bool all_odd = true;
+    for (size_t g = 0; g < h->group_N.size(); ++g) {
+        const int N = h->group_N[g];
+        const double rows = (double)h->group_count[g] * ((N + f.TMAX - 1) / f.TMAX);
+        pairs += rows * ((N + f.TMAX2 - 1) / f.TMAX2);
+        flush += rows * ((N + f.T2_flush - 1) / f.T2_flush);
+        all_odd = all_odd && N % 2 == 1;
+    }
+    if (!all_odd && 1.15 * flush >= pairs) return 1.0;
+    f.kern = f.kern_flush;
+    f.smem = f.smem_flush;
+    f.TMAX2 = f.T2_flush;
+    return all_odd ? 1.0 : 1.15;
+}
+
 int tiled_shape_count() { return kTiledShapes; }
 
 bool tiled_supported(const ctqw_hamiltonian *h, int dtype, int shape) {
@@ -858,13 +891,14 @@ int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
     auto consider = [&](int shape) {
         TiledShape f;
         if (!tiled_shape_for(shape, f)) return;
+        const double rate = settle_columns(h, f);
         double tiles = 0.0;
         for (size_t g = 0; g < h->group_N.size(); ++g) {
             const int N = h->group_N[g];
             tiles += (double)h->group_count[g] * ((N + f.TMAX - 1) / f.TMAX) * ((N + f.TMAX2 - 1) / f.TMAX2);
         }
         const int launches = (K + f.D - 1) / f.D;
-        double cost = tiles * (f.threads / 256.0) * (launches * kTileFixed + 8.0 * kRowStage * K);
+        double cost = rate * tiles * (f.threads / 256.0) * (launches * kTileFixed + 8.0 * kRowStage * K);
         if (f.threads > 256) cost /= kTallRate;
         if (best_cost == 0.0 || cost < best_cost) {
             best = shape;
@@ -876,6 +910,7 @@ int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
         TiledShape f;
         int n_sm = 152;
         tiled_shape_for(by_depth[even8], f);
+        settle_columns(h, f);
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device);
         int64_t tiles = 0;
         for (size_t g = 0; g < h->group_N.size(); ++g)
@@ -909,6 +944,7 @@ int launch_taylor_tiled_range(const ctqw_hamiltonian *h, int shape, const void *
         ctqw_set_error("tiled path: unknown shape %d", shape);
         return CTQW_EUNSUPPORTED;
     }
+    settle_columns(h, f);
     if (n_stages < 1 || n_stages > f.D || (final && j0 != n_stages)) {
         ctqw_set_error("tiled path: %d stages from j0=%d with depth %d", n_stages, j0, f.D);
         return CTQW_EINVAL;
