@@ -268,7 +268,7 @@ int ctqw_propagate_taylor(const ctqw_hamiltonian *h, int32_t dtype, void *psi_de
  * one GPC, so the SMs left over in each GPC hold no cluster; the tiles get
  * the share of realizations that their throughput on those SMs can finish
  * in the time the clusters take for the rest (whole rounds of the resident
- * clusters).  0 when fewer than 1/16 of the SMs are left over, when the
+ * clusters), if that is sooner than the clusters alone.  0 when fewer than 1/16 of the SMs are left over, when the
  * handle has no fused path, with CTQW_FLAG_ONE_STREAM, CTQW_FLAG_PLAIN or
  * CTQW_FLAG_RENORMALIZE, or with a shape flag.  Queries the device's
  * occupancy; launches nothing.  Errors: CTQW_EINVAL for a null handle or

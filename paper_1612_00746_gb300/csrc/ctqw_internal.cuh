@@ -47,6 +47,7 @@ struct ctqw_hamiltonian {
     // the cluster kernel's layout for this handle (plan_fused_rows, at the
     // build): warps a CTA, CTAs a cluster, resident clusters, CTAs an SM
     int rows_W = 0, rows_C = 0, rows_clusters = 0, rows_per_sm = 0;
+    double rows_stage_us = 0.0;   // a stage of a resident round, by the plan's model
     int density_method = 0;         // one-body density: 0 tensor cores where supported, 1 CUDA cores
     // second stream of the fused path (the realizations on the SMs that hold
     // no cluster) and the events that fork it from and join it to the caller's

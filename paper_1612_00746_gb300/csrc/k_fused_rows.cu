@@ -609,6 +609,7 @@ int plan_fused_rows(ctqw_hamiltonian *h) {
             h->rows_C = f.C;
             h->rows_clusters = clusters;
             h->rows_per_sm = per_sm;
+            h->rows_stage_us = a + b * f.W * per_sm;
         }
     }
     return CTQW_OK;
@@ -616,9 +617,9 @@ int plan_fused_rows(ctqw_hamiltonian *h) {
 
 // Tiled-to-fused throughput ratio per SM on two bosons at N = 256, K = 16
 // (register tiles 4.43e11 site-updates/s on 152 SMs, the full-row clusters
-// 1.11e12 on the 120 that hold them: 0.32); 1024 realizations, 50 steps took
-// 48.4 ms with 0.32 and 47.8 ms with 0.37.
-static constexpr double kTiledPerSmRatio = 0.37;
+// 1.11e12 on the 120 that hold them: 0.32).  1024 realizations, 50 steps: 62
+// rounds of clusters 47.8 ms, 63 48.4; 0.39 gives 62.
+static constexpr double kTiledPerSmRatio = 0.39;
 
 int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) {
     *R_tiled = 0;
@@ -631,11 +632,25 @@ int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) 
     const int used = std::min(n_sm, (clusters * h->rows_C + per_sm - 1) / per_sm);
     const int idle = n_sm - used;
     if (idle * 16 < n_sm) return CTQW_OK;   // under 1/16 of the SMs idle: not worth a second stream
-    // both parts end together when each one's share of the realizations
-    // matches its share of the throughput; the fused part gets whole rounds
-    const double share = used / (used + kTiledPerSmRatio * idle);
-    const int rounds = std::max(1, (int)std::lround(h->R * share / clusters));
-    const int R_f = std::min(h->R, rounds * clusters);
+    // the rounds of resident clusters with the least time of the longer part,
+    // a stage: so many rounds, against the tiles' throughput on the SMs left over
+    // and what a launch takes however few tiles it has (17 us for 8 stages: 1 of
+    // 24 x N = 192 on the tiles made 20 steps of K = 16 0.70 ms instead of 0.41).
+    // A share by throughput alone also gave: 77 x N = 192 1.27 ms, now 0.85; 20 x
+    // N = 256 0.96, now 0.53; 40 x N = 160 1.15, now 0.53.
+    constexpr double kTiledStageUs = 2.2;
+    const double tiled_us = h->rows_stage_us * used / (clusters * kTiledPerSmRatio * idle);   // a realization
+    const int most = (h->R + clusters - 1) / clusters;
+    int R_f = h->R;
+    double best = most * h->rows_stage_us;
+    for (int rounds = std::max(1, most / 2); rounds < most; ++rounds) {
+        const double t = std::max(rounds * h->rows_stage_us,
+                                  std::max(kTiledStageUs, (h->R - rounds * clusters) * tiled_us));
+        if (t < best) {
+            best = t;
+            R_f = rounds * clusters;
+        }
+    }
     *R_tiled = h->R - R_f;
     return CTQW_OK;
 }
