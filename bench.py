@@ -395,8 +395,7 @@ def ragged_leg(args, dev, stream):
     roof["timing"] = "the whole propagate call (tile launches and the reductions of 101 samples)"
     launches8 = -(-K // 8)
     depth = -(-K // launches8)
-    groups_per_launch = 1 if len(h.group_sizes) <= 32 else len(h.group_sizes)   # all groups in one launch
-    launches = 1 + w.n_steps * (-(-K // depth)) * groups_per_launch + n_obs + 1
+    launches = 1 + w.n_steps * (-(-K // depth)) + n_obs + 1   # all groups in one launch
     out = {"workload": w.name, "value": units / (ms / 1000.0), "unit": UNIT, "ms": ms,
            "R": w.R, "sizes": "N in {128, 192, ..., 1024} per realization (15 groups)",
            "K": K, "K_range": [8, 20], "n_steps": w.n_steps, "obs_every": w.obs_every,
@@ -474,15 +473,17 @@ def run_ours(args):
         n_seg = -(-w.n_steps // w.obs_every) if w.obs_every else 1
         launches_per_step = 1 + n_obs + n_seg * len(h.group_sizes)
     elif path == "plain":
-        # init_state + K stage launches per step + one observables kernel per sample
-        launches_per_step = 1 + w.n_steps * w.K + n_obs
+        # init_state + K stage launches per step (three particles in FP32: two
+        # stages a launch) + one observables kernel per sample
+        pairs = w.m == 3 and dtype == ctqw.C64 and not args.flags & ctqw.FLAG_PLAIN
+        launches_per_step = 1 + w.n_steps * (-(-w.K // 2) if pairs else w.K) + n_obs
     elif path == "tiled":
         # ceil(K / D) launches per step and size group, observables, init
         launches8 = -(-w.K // 8)
         depth = {0: -(-w.K // launches8), 9: 4, 10: 8, 11: 8, 12: 4, 13: 8, 14: 2, 15: 7}[(args.flags >> 8) & 0xF]
         # register tiles run every size group in one launch (the shared-memory shapes one per group)
         shared_mem_shape = ((args.flags >> 8) & 0xF) == 9
-        per_launch_groups = len(h.group_sizes) if shared_mem_shape or len(h.group_sizes) > 32 else 1
+        per_launch_groups = len(h.group_sizes) if shared_mem_shape else 1
         launches_per_step = 1 + w.n_steps * (-(-w.K // depth)) * per_launch_groups + n_obs
     else:
         # init_state + one fused launch per S + 1 sampling intervals + one
@@ -496,7 +497,7 @@ def run_ours(args):
         tile_depth = -(-w.K // -(-w.K // 8))   # the stages split evenly over ceil(K / 8) launches
         launches_per_step += w.n_steps * -(-w.K // tile_depth) + n_obs
     if args.switch is not None:
-        launches_per_step += 1 + w.n_steps   # parameter restore + one update per step
+        launches_per_step += 1 + (0 if path == "rows" else w.n_steps)   # parameter restore, one update per step
     launches_per_step += 1   # the norm check of the sampled norms
 
     prop_events = []
@@ -852,11 +853,11 @@ def rho1_line(args):
     The tensor-core kernel computes the 128 x 128 tiles of the upper
     triangle only (the rest is their conjugate transpose) and forms every
     real product from three TF32 piece products: per size group it runs
-    n_up 128^2 K 24 flops on the TF32 tensor pipe (n_up = T (T + 1) / 2
-    tiles, T = ceil(N / 128), K = R_g m N^(m-1)), whose peak is the measured
-    BF16 GEMM rate times the nominal TF32/BF16 ratio (1.1 / 2.25 PFLOP/s).
-    The call's time (slot clearing, the tensor-core kernel, the FP64 sum of
-    the slots) is the denominator, so the kernel's own rate is higher by
+    128^2 K (24 T (T - 1) / 2 + 18 T) flops on the TF32 tensor pipe (a tile on
+    the diagonal takes half of Im; T = ceil(N / 128), K = R_g m N^(m-1)), whose
+    peak is the measured BF16 GEMM rate times the nominal TF32/BF16 ratio (1.1
+    / 2.25 PFLOP/s).  The call's time (the tensor-core kernel, the sum of the
+    slots) is the denominator, so the kernel's own rate is higher by
     the share the launch list gives it.
     """
     import numpy as np
@@ -884,7 +885,7 @@ def rho1_line(args):
     for N_g in np.unique(sizes):
         T = (int(N_g) + 127) // 128
         K_g = float(np.sum(sizes == N_g)) * w.m * float(N_g) ** (w.m - 1)
-        tensor_flops += T * (T + 1) / 2 * 128.0 ** 2 * K_g * 24.0
+        tensor_flops += (T * (T - 1) / 2 * 24.0 + T * 18.0) * 128.0 ** 2 * K_g
     peaks = measured_peaks()
 
     def timed(method):
@@ -993,7 +994,10 @@ def run_lattice(args):
     value = units / (ms / 1000.0)
     drift = float((nr[-1] - 1.0).abs().max().item()) if n_obs else None
     peaks = measured_peaks()
-    if w.dtype == cw.C64 and w.m == 2 and g.N <= 324 and 2 * g.E <= 4 * g.N:
+    on_chip = w.dtype == cw.C64 and w.m == 2 and g.N <= 324 and 2 * g.E <= 4 * g.N
+    # on chip: one launch and a transpose per sampling interval, one transpose at the start
+    launches = w.n_steps * w.K if not on_chip else 1 + 2 * (-(-w.n_steps // w.obs_every) if w.obs_every else 1)
+    if on_chip:
         # iterates on chip, bound by shared memory; against the FP32 pipe
         flops = 4.0 * w.m * 2 * g.E / g.N + 4
         ach = units * flops / (ms / 1000.0) / 1e12
@@ -1029,7 +1033,7 @@ def run_lattice(args):
                    "n_steps": w.n_steps, "obs_every": w.obs_every,
                    "l2": "states larger than L2" if g.total_amplitudes * 8 > 129e6 else "L2-resident"},
         "roofline": roof, "norm_drift": drift, "clocks": clk,
-        "gpu_launches": int(args.steps * (w.n_steps * w.K + n_obs + 1)),
+        "gpu_launches": int(args.steps * (launches + n_obs + 1)),
     }
     print(json.dumps(line), flush=True)
     g.close()
