@@ -402,7 +402,10 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
         for (int r = grab(); r < a.r0 + a.R_run; r = grab()) {
             __syncthreads();
             load_realization(r);
-            __syncthreads();
+            if (SWITCH)
+                cluster_barrier();   // every CTA has read the parameters that CTA 0 overwrites when it is done
+            else
+                __syncthreads();
             if (!active) continue;
             for (long long step = 0; step < n_steps; ++step) {
                 if (K > 1) {
