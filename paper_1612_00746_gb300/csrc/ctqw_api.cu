@@ -296,7 +296,7 @@ int ctqw_build_hamiltonian(const ctqw_lattice_desc *d, void *stream, ctqw_hamilt
         ctqw_malloc(&h->J32, sizeof(float) * h->total_par) != cudaSuccess ||
         ctqw_malloc(&h->eps64, pb) != cudaSuccess || ctqw_malloc(&h->J64, pb) != cudaSuccess ||
         ctqw_malloc(&u_eps_d, pb) != cudaSuccess || ctqw_malloc(&u_J_d, pb) != cudaSuccess ||
-        ctqw_malloc((void **)&h->status_d, 32) != cudaSuccess ||
+        ctqw_malloc((void **)&h->status_d, 16) != cudaSuccess ||
         ctqw_malloc((void **)&h->renorm_d, sizeof(double) * h->R) != cudaSuccess ||
         ctqw_malloc((void **)&h->sites_d, sizeof(int32_t) * h->R * h->m) != cudaSuccess) {
         ctqw_set_error("cudaMalloc of the parameter arrays failed");

@@ -40,7 +40,7 @@ struct ctqw_hamiltonian {
     // status word (16 bytes): int flags at [0] (bit 0: a bounded wait gave
     // up, bit 1: the norm check failed), at byte 8 the 64-bit key of the
     // first norm failure, (realization << 40) | (sample << 8) | reason
-    int *status_d = nullptr;        // 32 bytes: the status word, then at int [4] the fused kernel's ticket counter
+    int *status_d = nullptr;
     double *renorm_d = nullptr;     // [R] norms of the per-step renormalization
     int32_t *sites_d = nullptr;     // [R][m] initial sites (ctqw_init_state)
     double norm_drift_tol = 0.0;    // norm check: |norm - norm at step 0| above this fails (0: finiteness only)
@@ -69,8 +69,6 @@ struct RealTable {
     int periodic;
     double U;
 };
-
-inline int *work_counter(const ctqw_hamiltonian *h) { return h->status_d + 4; }
 
 inline RealTable real_table(const ctqw_hamiltonian *h) {
     RealTable t;
@@ -264,9 +262,9 @@ int launch_group_sum(const ctqw_hamiltonian *h, const double *grad, double *out,
 // rounding error in and out; when snap is not null the state after every
 // snap_every-th step before the last is stored to slot q = step/snap_every - 1
 // of snap (consecutive states, the layout of psi).  The launch covers
-// realizations r0 .. r0 + R_run - 1 with one cluster per resident slot; the
-// clusters take the realizations one at a time from the handle's ticket
-// counter (work_counter), which the launch zeroes on its stream.
+// realizations r0 .. r0 + R_run - 1, dealt out in turn to one cluster per
+// resident slot; it keeps nothing in the handle, so calls on several streams
+// do not meet.
 bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype);
 // Picks the split of a lattice over warps, CTAs and the cluster for the
 // handle's N and R (rows_* of the handle); a no-op where the kernel does not apply.

@@ -4,8 +4,13 @@
 // One thread-block cluster owns one realization at a time for all steps of
 // the launch (the order-K Taylor polynomial of Algorithm 3, Sec. 2.3, applied
 // n_steps times).  The grid holds only as many clusters as are resident at
-// once, and each takes realization after realization from a ticket counter,
-// so the SMs a cluster holds stay its own until the launch ends.
+// once, and cluster q of n takes the realizations q, q + n, q + 2 n, ..., so the
+// SMs a cluster holds stay its own until the launch ends.  (A counter in the
+// handle, from which a cluster took its next realization, was shared by calls
+// that overlap on one handle: they stepped each other's realizations twice or
+// not at all.  All take the same time, so the counter gained nothing: 1024
+// realizations of N = 256, 50 steps: 47.93 ms with it, 47.91 without; 1000 rings
+// of N = 100, 100 steps: 21.75 and 21.83; one of N = 64, 10 steps: 75.8 and 73.5 us.)
 // The N x N tile is split into row slabs, one per CTA; every warp owns RL
 // whole rows and each lane CL adjacent columns of them (N <= 32 CL), so a warp
 // covers full rows: neighbours along x2 are in the lane's registers or one
@@ -42,7 +47,7 @@
 // barrier a stage (K = 16, site-updates/s, one stream): N = 64 1.17e12 ->
 // 1.23e12, N = 128 1.27e12 -> 1.33e12, N = 192 1.01e12 -> 1.23e12, N = 256
 // 9.1e11 -> 1.11e12; N = 100, on the register tiles before, 4.4e11 -> 7.6e11;
-// one realization of N = 64, 10 steps: 129 us -> 76 us.
+// one realization of N = 64, 10 steps: 129 us -> 74 us.
 //
 // Control flow: the stages of a step are a first one (from psi), middle ones
 // in pairs and a final one, with no per-stage dispatch.  A row tests the few
@@ -88,8 +93,7 @@ struct RowsArgs {
     int *status;
     unsigned long long wait_limit_ns;
     int test_timeout;
-    int r0, R_run;          // realizations r0 .. r0 + R_run - 1, handed out one at a time
-    int *work;              // ticket counter of the hand-out, zero at the launch
+    int r0, R_run;          // realizations r0 .. r0 + R_run - 1
     // switching noise: the law, the number of the first step, and the
     // parameters to leave the updated values in
     SwitchLaw law;
@@ -157,7 +161,6 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
     __shared__ __align__(8) unsigned long long mbar[2][2];      // halo rows: [parity][above, below]
     __shared__ __align__(8) unsigned long long mbar_edge;       // the CTA's warps have published a stage
     __shared__ __align__(8) unsigned long long mbar_never;
-    __shared__ int next_r;
 
     const int rank = (int)cluster_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -279,15 +282,6 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
 
     const long long n_steps = a.n_steps;
     const int K = a.K;
-    // the next realization of this cluster: CTA 0 takes a ticket, the others
-    // read it from CTA 0's shared memory between two cluster barriers
-    auto grab = [&]() -> int {
-        if (rank == 0 && threadIdx.x == 0) next_r = a.r0 + atomicAdd(a.work, 1);
-        cluster_barrier();
-        const int r = ld_shared_cluster_s32(map_rank(smem_u32(&next_r), 0));
-        cluster_barrier();
-        return r;
-    };
     // edge rows of the warp and of its neighbours, by parity (with one CTA the
     // slab's edges are each other's neighbours)
     const bool push_up = C > 1 && top, push_dn = C > 1 && bottom;
@@ -397,10 +391,9 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
                 Q[i][k + 1] = pack2(h1.x, h1.y);
             }
         };
-        // realizations are handed out one at a time, so a cluster that runs
-        // faster takes more of them
-        for (int r = grab(); r < a.r0 + a.R_run; r = grab()) {
-            __syncthreads();
+        const int r_end = a.r0 + a.R_run, clusters = (int)gridDim.x / C;
+        for (int r = a.r0 + (int)blockIdx.x / C; r < r_end; r += clusters) {
+            cluster_barrier();   // every warp is done with the last one's shared memory
             load_realization(r);
             if (SWITCH)
                 cluster_barrier();   // every CTA has read the parameters that CTA 0 overwrites when it is done
@@ -698,7 +691,6 @@ static int launch_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *sna
     a.wait_limit_ns = 2000000000ull;
     a.r0 = r0;
     a.R_run = R_run;
-    a.work = work_counter(h);
     a.step0 = (unsigned long long)step0;
     if (law) {
         a.law = *law;
@@ -730,9 +722,8 @@ static int launch_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *sna
         ctqw_set_error("fused path: no cluster of %d CTAs x %d threads fits", f.C, f.threads);
         return CTQW_EUNSUPPORTED;
     }
-    // one cluster per resident slot, each taking realizations until none is left
+    // one cluster per resident slot
     cfg.gridDim = dim3((unsigned)(std::min(R_run, clusters) * f.C));
-    CTQW_CUDA_TRY(cudaMemsetAsync(a.work, 0, sizeof(int), s));
     CTQW_CUDA_TRY(cudaLaunchKernelEx(&cfg, f.kern, a));
     return CTQW_OK;
 }

@@ -1,0 +1,58 @@
+"""Two calls on one handle at the same time, each with its own state, workspace
+and stream: the states they end in have the same bits as when the calls run
+one after the other.  Sizes with one CTA a realization and with clusters, with
+fewer and with more realizations than run at once."""
+import numpy as np
+import pytest
+
+import ctqw_workloads as cw
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctqw():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1612_00746_gb300 import build, ctqw as c
+
+    build.build()
+    c.load()
+    return c
+
+
+def _calls(ctqw, h, w, n):
+    """n states of different contents and n workspaces, and a call on each."""
+    rng = np.random.default_rng(w.N)
+    v = rng.standard_normal((n, h.total_amplitudes)) + 1j * rng.standard_normal((n, h.total_amplitudes))
+    psis = [torch.from_numpy((x / np.linalg.norm(x) * np.sqrt(w.R)).astype(np.complex64)).cuda() for x in v]
+    spaces = [torch.empty(3 * 8 * h.total_amplitudes, dtype=torch.uint8, device="cuda") for _ in range(n)]
+
+    def call(i, stream, steps, flags=0):
+        ctqw.ctqw_propagate_taylor(h, psis[i], cw.C64, w.dt, w.K, steps, 0, None, None, None, flags, spaces[i], stream)
+
+    return psis, call
+
+
+@pytest.mark.parametrize("N,R", [(64, 40), (64, 700), (100, 60), (100, 400), (200, 20), (256, 7), (256, 40)])
+def test_two_streams(ctqw, N, R):
+    w = cw.get("bosons_n256_u2").with_(N=N, R=R, sites=(N // 2 - 1, N // 2))
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    steps = (60, 37)
+    out = []
+    for overlap in (False, True):
+        h = ctqw.build_for_workload(w)
+        psis, call = _calls(ctqw, h, w, 2)
+        torch.cuda.synchronize()
+        for i in range(2):
+            for part in range(3):   # several launches a stream
+                call(i, streams[i], steps[i])
+            if not overlap:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        ctqw.ctqw_check_status(h)
+        out.append([p.cpu().numpy() for p in psis])
+        h.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
