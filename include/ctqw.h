@@ -247,7 +247,10 @@ int ctqw_autotune_order(const ctqw_hamiltonian *h, int32_t dtype, double dt, int
  * realizations on the register tiles, on a second stream of the handle that
  * it forks from and joins back to `stream` (so the call stays ordered on
  * `stream`, also under graph capture): those tiles fill the SMs that no
- * cluster can hold.  Overlapping calls on one handle share that stream.  The
+ * cluster can hold.  The calls of one handle share that stream: they may
+ * overlap, on streams and from threads of their own, but their parts on it run
+ * one after the other, and a call made while that stream belongs to another
+ * call's unfinished graph capture runs on `stream` alone.  The
  * per-term path evaluates the polynomial of Algorithm 3 in Horner form
  * (w_j = Psi + (-i dt / j) H w_{j+1}, j = K..2, Psi(t+dt) = Psi - i dt H w_2):
  * the same sum with fewer operations and roundings than term by term.  In

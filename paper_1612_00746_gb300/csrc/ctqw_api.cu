@@ -715,6 +715,19 @@ static int propagate_tiled(const ctqw_hamiltonian *h, int32_t dtype, void *psi_d
                        sw, 0, h->R, s);
 }
 
+// Whether the handle's second stream can follow s now: not while it is part of
+// a graph capture (of another call, until that capture ends) that s is not in.
+static int side_can_follow(const ctqw_hamiltonian *h, cudaStream_t s, bool *can) {
+    cudaStreamCaptureStatus side_status, s_status;
+    unsigned long long side_id = 0, s_id = 0;
+    CTQW_CUDA_TRY(cudaStreamGetCaptureInfo(h->side, &side_status, &side_id));
+    *can = side_status == cudaStreamCaptureStatusNone;
+    if (*can) return CTQW_OK;
+    CTQW_CUDA_TRY(cudaStreamGetCaptureInfo(s, &s_status, &s_id));
+    *can = s_status == cudaStreamCaptureStatusActive && s_id == side_id;
+    return CTQW_OK;
+}
+
 // The full-row fused kernel in chunks: the workspace holds the carried
 // rounding error (one state) and S >= 0 snapshot slots.  A launch runs from a
 // sample point over up to S + 1 sampling intervals, storing the state at the
@@ -728,7 +741,10 @@ static int propagate_tiled(const ctqw_hamiltonian *h, int32_t dtype, void *psi_d
 // register tiles on the handle's side stream, forked from and joined to the
 // caller's stream: the tiles use slots 1 and 2 of their own realizations as
 // iterate buffers, the clusters' snapshots only touch theirs, and both add
-// into the same zeroed P_mean rows.
+// into the same zeroed P_mean rows.  Calls on one handle from several threads
+// take the side stream and its events in turn, each until its tiles are
+// enqueued and joined: another call's fork in between would move the events,
+// or draw this call's tiles into that call's graph capture.
 static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double dt, int32_t K,
                                 int64_t n_steps, int32_t obs_every, double *P_mean_dev,
                                 double *norm_dev, double *energy_dev, uint32_t flags, int shape,
@@ -753,8 +769,15 @@ static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double
     int st = CTQW_OK;
     if (cudaMemsetAsync(lo, 0, sb, s) != cudaSuccess) st = ctqw_cuda_fail(cudaGetLastError(), "memset");
     int R_t = 0;
+    std::unique_lock<std::mutex> side_held(h->side_lock, std::defer_lock);
     if (st == CTQW_OK && h->side && slots >= 2 && shape == 0 && !(flags & CTQW_FLAG_ONE_STREAM))
         st = fused_rows_split(h, shape, K, &R_t);
+    if (st == CTQW_OK && R_t > 0) {
+        bool can = false;
+        side_held.lock();
+        st = side_can_follow(h, s, &can);
+        if (!can) R_t = 0;
+    }
     const int R_f = h->R - R_t;
     cudaStream_t side = s;
     if (st == CTQW_OK && R_t > 0) {

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -50,7 +51,9 @@ struct ctqw_hamiltonian {
     double rows_stage_us = 0.0;   // a stage of a resident round, by the plan's model
     int density_method = 0;         // one-body density: 0 tensor cores where supported, 1 CUDA cores
     // second stream of the fused path (the realizations on the SMs that hold
-    // no cluster) and the events that fork it from and join it to the caller's
+    // no cluster) and the events that fork it from and join it to the caller's;
+    // a call holds the lock from the fork to the join
+    mutable std::mutex side_lock;
     cudaStream_t side = nullptr;
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
 };

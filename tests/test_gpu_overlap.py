@@ -2,6 +2,8 @@
 and stream: the states they end in have the same bits as when the calls run
 one after the other.  Sizes with one CTA a realization and with clusters, with
 fewer and with more realizations than run at once."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -56,3 +58,64 @@ def test_two_streams(ctqw, N, R):
         h.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("N,R", [(256, 150), (192, 77)])
+def test_two_threads_and_the_second_stream(ctqw, N, R):
+    # realizations on the handle's second stream, which the calls of both threads fork and join
+    w = cw.get("bosons_n256_u2").with_(N=N, R=R, sites=(N // 2 - 1, N // 2))
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    out = []
+    for overlap in (False, True):
+        h = ctqw.build_for_workload(w)
+        assert ctqw.ctqw_fused_split(h, w.K) > 0 or N < 256
+        psis, call = _calls(ctqw, h, w, 2)
+        torch.cuda.synchronize()
+
+        def work(i):
+            for part in range(20):
+                call(i, streams[i], 2 + i)
+
+        threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+        for t in threads:
+            t.start()
+            if not overlap:
+                t.join()
+                torch.cuda.synchronize()
+        for t in threads:
+            t.join()
+        torch.cuda.synchronize()
+        ctqw.ctqw_check_status(h)
+        out.append([p.cpu().numpy() for p in psis])
+        h.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+def test_a_call_beside_another_calls_capture(ctqw):
+    w = cw.get("bosons_n256_u2").with_(R=150)
+    h = ctqw.build_for_workload(w)
+    assert ctqw.ctqw_fused_split(h, w.K) > 0
+    psis, call = _calls(ctqw, h, w, 2)
+    start = [p.clone() for p in psis]
+    call(0, None, 3)
+    call(0, None, 3)
+    call(1, None, 3, ctqw.FLAG_ONE_STREAM)
+    torch.cuda.synchronize()
+    expect = [p.cpu().numpy() for p in psis]
+    for p, q in zip(psis, start):
+        p.copy_(q)
+    captured, other = torch.cuda.Stream(), torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=captured, capture_error_mode="relaxed"):
+        call(0, captured, 3)
+        call(1, other, 3)   # at once, and not into the graph
+        call(0, captured, 3)
+    other.synchronize()
+    assert np.array_equal(psis[1].cpu().numpy(), expect[1])
+    assert torch.equal(psis[0], start[0])
+    graph.replay()
+    torch.cuda.synchronize()
+    ctqw.ctqw_check_status(h)
+    assert np.array_equal(psis[0].cpu().numpy(), expect[0])
+    h.close()
