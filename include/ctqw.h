@@ -491,6 +491,13 @@ int ctqw_check_status(const ctqw_hamiltonian *h, void *stream);
  */
 int ctqw_inject_alloc_failure(int32_t after);
 
+/*
+ * Failure injection for tests: the handle as its build leaves it on a device
+ * that holds no cluster of the fused kernel (its calls then run as those of
+ * sizes the fused kernel does not take).  Errors: EINVAL for a null handle.
+ */
+int ctqw_inject_no_clusters(ctqw_hamiltonian *h);
+
 /* ------------------------------------------------------------------------
  * q-dimensional lattices and general graphs (Sec. 2: a q-dimensional lattice
  * of N = prod_i N_i nodes, or a general graph where each node has its own

@@ -347,8 +347,8 @@ int ctqw_build_hamiltonian(const ctqw_lattice_desc *d, void *stream, ctqw_hamilt
     if (cudaMemcpyAsync(h->eps64_0, h->eps64, pb, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(h->J64_0, h->J64, pb, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
         return fail(CTQW_ECUDA);
+    if ((st = plan_fused_rows(h))) return fail(st);
     if (fused_rows_supported(h, CTQW_C64)) {
-        if ((st = plan_fused_rows(h))) return fail(st);
         // the fused path's second stream, at the lowest priority so that the
         // clusters go first when both have work waiting
         int least = 0, greatest = 0;
@@ -857,7 +857,8 @@ static int propagate_taylor_impl(const ctqw_hamiltonian *h, int32_t dtype, void 
     // the cluster kernel takes every uniform N it can lay out; the tuning
     // shapes and a missing workspace only go with the sizes of the banded kernel
     const bool tuned_size = fused_taylor_supported(h, dtype);
-    const bool fused = !(flags & CTQW_FLAG_PLAIN) && fused_rows_supported(h, dtype) && (tuned_size || shape == 0);
+    const bool fused = !(flags & CTQW_FLAG_PLAIN) && (shape >= 4 || fused_rows_supported(h, dtype)) &&
+                       (tuned_size || shape == 0);
     // two particles in FP32 that the cluster-resident kernel cannot hold
     // (N > 256, ragged sizes, some rings): the temporally blocked tiled kernel
     // with the iterate in registers, at the region and depth of least cost
@@ -929,7 +930,7 @@ static int propagate_switching_impl(const ctqw_hamiltonian *h, int32_t dtype, vo
     sw.on = true;
     sw.seed = seed;
     sw.p = p_switch;
-    if (!(flags & CTQW_FLAG_PLAIN) && fused_rows_supported(h, dtype)) {
+    if (!(flags & CTQW_FLAG_PLAIN) && fused_rows_switching_supported(h, dtype)) {
         // the clusters redraw the parameters themselves after every step; a
         // launch per sampling interval, since a sample uses H of its step
         CTQW_TRY(zero_outputs(h, n_samples(n_steps, obs_every), P_mean_dev, norm_dev, energy_dev, s));
@@ -1118,6 +1119,12 @@ int ctqw_set_norm_check(ctqw_hamiltonian *h, double drift_tol) {
 int ctqw_inject_alloc_failure(int32_t after) {
     if (after < -1) { ctqw_set_error("after must be >= -1 (got %d)", after); return CTQW_EINVAL; }
     g_alloc_fail_after.store(after);
+    return CTQW_OK;
+}
+
+int ctqw_inject_no_clusters(ctqw_hamiltonian *h) {
+    if (!h) { ctqw_set_error("null handle"); return CTQW_EINVAL; }
+    h->rows_W = h->rows_C = h->rows_clusters = h->rows_switch_clusters = h->rows_per_sm = 0;
     return CTQW_OK;
 }
 

@@ -46,8 +46,10 @@ struct ctqw_hamiltonian {
     int32_t *sites_d = nullptr;     // [R][m] initial sites (ctqw_init_state)
     double norm_drift_tol = 0.0;    // norm check: |norm - norm at step 0| above this fails (0: finiteness only)
     // the cluster kernel's layout for this handle (plan_fused_rows, at the
-    // build): warps a CTA, CTAs a cluster, resident clusters, CTAs an SM
-    int rows_W = 0, rows_C = 0, rows_clusters = 0, rows_per_sm = 0;
+    // build): warps a CTA, CTAs a cluster, resident clusters (of the kernel with
+    // switching noise: rows_switch_clusters; 0: the device holds none, the
+    // kernel is not used), CTAs an SM
+    int rows_W = 0, rows_C = 0, rows_clusters = 0, rows_switch_clusters = 0, rows_per_sm = 0;
     double rows_stage_us = 0.0;   // a stage of a resident round, by the plan's model
     int density_method = 0;         // one-body density: 0 tensor cores where supported, 1 CUDA cores
     // second stream of the fused path (the realizations on the SMs that hold
@@ -269,8 +271,10 @@ int launch_group_sum(const ctqw_hamiltonian *h, const double *grad, double *out,
 // resident slot; it keeps nothing in the handle, so calls on several streams
 // do not meet.
 bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype);
+bool fused_rows_switching_supported(const ctqw_hamiltonian *h, int dtype);
 // Picks the split of a lattice over warps, CTAs and the cluster for the
-// handle's N and R (rows_* of the handle); a no-op where the kernel does not apply.
+// handle's N and R (rows_* of the handle); a no-op where the kernel does not
+// apply.  The handle supports the kernel once it has found a resident cluster.
 int plan_fused_rows(ctqw_hamiltonian *h);
 // How many realizations (the last ones) to run on the register tiles on the
 // handle's side stream while the clusters run the rest: the SMs that hold no

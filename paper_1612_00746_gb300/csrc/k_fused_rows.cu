@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
 using RowsKernel = void (*)(RowsArgs);
 
 struct RowsShape {
-    int C, W, threads;
+    int N, C, W, threads;
     size_t smem;
     RowsKernel kern, kern_switch;
 };
@@ -523,6 +523,7 @@ bool rows_shape_for(int N, int periodic, int maxw, RowsShape &f) {
         case 6: f.kern = taylor_fused_rows_kernel<6, 8, false>; f.kern_switch = taylor_fused_rows_kernel<6, 8, true>; break;
         default: f.kern = taylor_fused_rows_kernel<8, 8, false>; f.kern_switch = taylor_fused_rows_kernel<8, 8, true>; break;
     }
+    f.N = N;
     const int units = (N + 3) / 4;
     f.C = (units + maxw - 1) / maxw;
     if (f.C > 16) return false;
@@ -531,6 +532,12 @@ bool rows_shape_for(int N, int periodic, int maxw, RowsShape &f) {
     f.threads = 32 * f.W;
     f.smem = sizeof(float4) * 16 * CL * (size_t)(4 + 4 * f.W + 4 * f.W) + sizeof(float2) * (size_t)(4 * f.W + 2);
     return true;
+}
+
+// The same layout with switching noise: room for the parameters.
+void with_switching(RowsShape &f) {
+    f.kern = f.kern_switch;
+    f.smem += sizeof(double) * 2 * (size_t)f.N;
 }
 
 // The kernels are shared by layouts of different sizes: the limit is always
@@ -568,9 +575,10 @@ bool rows_shape_of(const ctqw_hamiltonian *h, int shape, RowsShape &f) {
 
 }  // namespace
 
-bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype) {
-    RowsShape f;
-    return dtype == CTQW_C64 && h->m == 2 && h->uniform && rows_shape_for(h->Nmax, h->periodic, 16, f);
+bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype) { return dtype == CTQW_C64 && h->rows_clusters > 0; }
+
+bool fused_rows_switching_supported(const ctqw_hamiltonian *h, int dtype) {
+    return dtype == CTQW_C64 && h->rows_switch_clusters > 0;
 }
 
 // With many realizations the largest CTAs win by a little (fewest rows cross
@@ -583,7 +591,8 @@ bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype) {
 // rounds of resident clusters plus the last one, which has its SMs to itself
 // as far as they go.
 int plan_fused_rows(ctqw_hamiltonian *h) {
-    if (!fused_rows_supported(h, CTQW_C64)) return CTQW_OK;
+    RowsShape planned;
+    if (h->m != 2 || !h->uniform || !rows_shape_for(h->Nmax, h->periodic, 16, planned)) return CTQW_OK;
     static const double a_of[5] = {0, 0.33, 0.40, 0.41, 0.54}, b_of[5] = {0, 0.011, 0.034, 0.035, 0.042};
     const int CL = rows_columns(h->Nmax, h->periodic);
     const double a = a_of[CL / 2], b = b_of[CL / 2];
@@ -601,12 +610,19 @@ int plan_fused_rows(ctqw_hamiltonian *h) {
         if (rest) t += a + b * f.W * std::min(per_sm, (rest + alone - 1) / alone);
         if (best == 0.0 || t < 0.97 * best) {
             best = t;
+            planned = f;
             h->rows_W = f.W;
             h->rows_C = f.C;
             h->rows_clusters = clusters;
             h->rows_per_sm = per_sm;
             h->rows_stage_us = a + b * f.W * per_sm;
         }
+    }
+    if (h->rows_clusters > 0) {
+        with_switching(planned);
+        int per_sm = 0;
+        CTQW_TRY(set_rows_attributes(planned.kern));
+        CTQW_TRY(rows_residency(planned, &h->rows_switch_clusters, &per_sm));
     }
     return CTQW_OK;
 }
@@ -698,8 +714,7 @@ static int launch_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *sna
         a.J_out = h->J64;
         a.eps32_out = h->eps32;
         a.J32_out = h->J32;
-        f.kern = f.kern_switch;
-        f.smem += sizeof(double) * 2 * (size_t)h->Nmax;
+        with_switching(f);
     }
     a.inv_j[0] = 0.f;
     for (int j = 1; j <= kMaxK; ++j) a.inv_j[j] = (float)(1.0 / j);
@@ -716,8 +731,8 @@ static int launch_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *sna
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int clusters = h->rows_clusters, per_sm = 0;
-    if (shape != 0 || law) CTQW_TRY(rows_residency(f, &clusters, &per_sm));
+    int clusters = law ? h->rows_switch_clusters : h->rows_clusters, per_sm = 0;
+    if (shape != 0) CTQW_TRY(rows_residency(f, &clusters, &per_sm));
     if (clusters < 1) {
         ctqw_set_error("fused path: no cluster of %d CTAs x %d threads fits", f.C, f.threads);
         return CTQW_EUNSUPPORTED;

@@ -56,6 +56,7 @@ EXPORTED = (
     "ctqw_graph_state_size", "ctqw_graph_init_state", "ctqw_graph_workspace_size",
     "ctqw_graph_propagate_taylor", "ctqw_graph_propagate_rk4", "ctqw_graph_observables",
     "ctqw_graph_set_chunk", "ctqw_set_norm_check", "ctqw_inject_alloc_failure",
+    "ctqw_inject_no_clusters",
     "ctqw_set_density_method", "ctqw_fused_split",
 )
 
@@ -121,6 +122,7 @@ def load(path: Optional[str] = None) -> ctypes.CDLL:
         "ctqw_check_status": [vp, vp],
         "ctqw_set_norm_check": [vp, dbl],
         "ctqw_inject_alloc_failure": [i32],
+        "ctqw_inject_no_clusters": [vp],
         "ctqw_set_density_method": [vp, i32],
         "ctqw_fused_split": [vp, i32, u32, ctypes.POINTER(i32)],
         "ctqw_adjoint_workspace_size": [vp, i32, i32, i64, i32, ctypes.POINTER(sz)],
@@ -489,6 +491,10 @@ def ctqw_set_density_method(h: Hamiltonian, method: int) -> None:
 
 def ctqw_inject_alloc_failure(after: int) -> None:
     _check(load().ctqw_inject_alloc_failure(int(after)))
+
+
+def ctqw_inject_no_clusters(h: Hamiltonian) -> None:
+    _check(load().ctqw_inject_no_clusters(h.handle))
 
 
 def ctqw_fused_split(h: Hamiltonian, K: int, flags: int = 0) -> int:
