@@ -32,8 +32,13 @@
 //    block's FP32 sum in TMEM can be off by up to 256 ulp of its sum of
 //    |terms| (the adds may round toward zero): at most 256 x 2^-23 of the
 //    largest element of rho1.
-// A second kernel sums the slots of all CTAs in FP64 and fills the lower
-// triangle.  The producers' loads and stores bound an off-diagonal tile, so a
+// A second kernel sums the slots of a tile, keeping at least what FP64 would
+// (Sum3), and a third writes the tiles and their conjugates into rho1.  Against
+// an FP64 sum the diagonal tiles' Im is off by half of what it was with twelve
+// products (largest element 1, N = 128, 300 realizations: evolved bosons 9e-8 for
+// 1.8e-7, plane waves 1.4e-6 for 2.9e-6), but by more, 4e-8 for 2e-9, where every
+// realization is real up to a phase and Im vanishes; Re (4.8e-6) is the same.
+// The producers' loads and stores bound an off-diagonal tile, so a
 // diagonal one takes less time, and the (realization, particle) pairs are
 // split over more CTAs of the one than of the other (see density_splits).  1024
 // realizations of N = 256: 1.05 ms and 0.06 ms for the sum of the slots -> 0.92
@@ -136,14 +141,32 @@ __device__ __forceinline__ float tf32_round(float v) {
     return __uint_as_float(r);
 }
 
-// hi + lo + v, rounded back into (hi, lo): TwoSum, then the error into lo.
-__device__ __forceinline__ void two_sum_add(float &hi, float &lo, float v) {
+// hi + v rounded into hi; returns what the rounding left out, exactly (TwoSum).
+__device__ __forceinline__ float two_sum(float &hi, float v) {
     const float s = __fadd_rn(hi, v);
     const float bb = __fsub_rn(s, hi);
     const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(v, bb));
     hi = s;
+    return e;
+}
+
+// hi + lo + v, rounded back into (hi, lo).
+__device__ __forceinline__ void two_sum_add(float &hi, float &lo, float v) {
+    const float e = two_sum(hi, v);
     lo = __fadd_rn(lo, e);
 }
+
+// A sum in three FP32 words: v and its carried error w added.  The first two
+// additions lose nothing and only the third word is rounded, so n terms are
+// off by about n^2 2^-72 of the sum: less than one rounding of an FP64 sum.
+struct Sum3 {
+    float a = 0.f, b = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float v, float w) {
+        const float e1 = two_sum(a, v), e2 = two_sum(b, w), e3 = two_sum(b, e1);
+        c = __fadd_rn(c, __fadd_rn(e2, e3));
+    }
+    __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
 
 // 32 consecutive TMEM columns of this warp's 32 lanes.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
@@ -475,11 +498,12 @@ __global__ void __launch_bounds__(kThreads, 1) rho1_tc_kernel(const __grid_const
 
 // The CTAs' slots of a tile summed over the splits: sums[tile][re, im][column]
 // [row].  Each 32 rows of a column are `share` warps' (8, or fewer for fewer
-// splits), every share-th split of a warp in two FP32 words, as the CTAs' own
-// totals, and the warps' sums in FP64.
+// splits), every share-th split of a warp in three FP32 words (Sum3), which
+// keep more than FP64 would, and the warps' sums in FP64.
 // (3 tiles of 50 splits: one thread walking all splits of an element in FP64,
 // the lower triangle read across the rows, 61 us; 8 warps in FP64, whose
-// conversions and adds then bound it, 44; now 12.)
+// conversions and adds then bound it, 44; in two words, which dropped bits that
+// an FP64 sum keeps, 12; in three 16.)
 constexpr int kRedWarps = 8;
 __global__ void __launch_bounds__(32 * kRedWarps) rho1_tc_reduce_kernel(const float *__restrict__ slots, int tiles,
                                                                         int off_splits, int diag_splits, int share,
@@ -503,17 +527,15 @@ __global__ void __launch_bounds__(32 * kRedWarps) rho1_tc_reduce_kernel(const fl
         first = n_off * off_splits + id - n_off;
     }
     const float *slot0 = slots + (size_t)first * (4 * plane);
-    float rh = 0.f, rl = 0.f, ih = 0.f, il = 0.f;
+    Sum3 sr, si;
 #pragma unroll 4
     for (int s = warp - w0; s < splits; s += share) {
         const float *slot = slot0 + (size_t)s * step * (4 * plane);
-        two_sum_add(rh, rl, slot[o]);
-        two_sum_add(ih, il, slot[plane + o]);
-        rl = __fadd_rn(rl, slot[2 * plane + o]);
-        il = __fadd_rn(il, slot[3 * plane + o]);
+        sr.add(slot[o], slot[2 * plane + o]);
+        si.add(slot[plane + o], slot[3 * plane + o]);
     }
-    part[0][warp][lane] = (double)rh + (double)rl;
-    part[1][warp][lane] = (double)ih + (double)il;
+    part[0][warp][lane] = sr.value();
+    part[1][warp][lane] = si.value();
     __syncthreads();
     if (warp != w0) return;
     double re = 0.0, im = 0.0;
