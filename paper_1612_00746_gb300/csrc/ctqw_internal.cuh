@@ -302,7 +302,6 @@ int launch_taylor_wavefront(const ctqw_hamiltonian *h, void *psi, void *lo, doub
 // Temporally blocked Taylor stages (m = 2, c64): up to D Horner stages per
 // launch on shared-memory tiles with halos; final launches add A w_2 to psi
 // (compensated, lo in place) and write the new state to w_out.
-int tiled_shape_count();
 bool tiled_supported(const ctqw_hamiltonian *h, int dtype, int shape);
 int tiled_depth(int shape);
 int tiled_default_shape(const ctqw_hamiltonian *h, int K);   // the register tiles' region and depth for the sizes

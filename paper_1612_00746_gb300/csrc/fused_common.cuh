@@ -41,10 +41,6 @@ static __device__ __forceinline__ void mbar_init(uint32_t mb, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(count) : "memory");
 }
 
-static __device__ __forceinline__ void mbar_arrive(uint32_t mb) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mb) : "memory");
-}
-
 // One arrival per warp, from its first lane (no branch).
 static __device__ __forceinline__ void mbar_arrive_lane0(uint32_t mb, int lane) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.b32 p, %1, 0;\n\t"
@@ -146,10 +142,6 @@ static __device__ __forceinline__ pair_t horner2(pair_t psi, pair_t y, float c) 
     return pack2(fmaf(c, v.y, q.x), fmaf(-c, v.x, q.y));
 }
 
-static __device__ __forceinline__ float2 ffma2(float a, float2 b, float2 c) {
-    return __ffma2_rn(make_float2(a, a), b, c);
-}
-
 // (re, im) pair moved between lanes as one 64-bit value.
 static __device__ __forceinline__ float2 shfl2(float2 v, int src) {
     const unsigned long long u = __shfl_sync(0xffffffffu, *reinterpret_cast<unsigned long long *>(&v), src);
@@ -179,12 +171,6 @@ static __device__ __forceinline__ void compensated_add2(float2 &hi, float2 &lo, 
     const float2 h2 = __fadd2_rn(t, l);
     lo = __ffma2_rn(__ffma2_rn(t, m1, h2), m1, l);
     hi = h2;
-}
-
-static __device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
 }
 
 // Butterfly sum over the warp in FP64 (every lane gets the total).

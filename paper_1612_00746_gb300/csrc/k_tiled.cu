@@ -781,7 +781,7 @@ TiledShape tiled_reg_shape() {
     s.smem = Tile::smem;
     s.fixed_tile = true;
     s.threads = 32 * W;
-    if (D % 2) {
+    if constexpr (D % 2 == 1) {
         s.kern_flush = taylor_tiled_reg_kernel<D, W, true>;
         s.T2_flush = RegTile<D, W, true>::T2;
         s.smem_flush = RegTile<D, W, true>::smem;
@@ -802,18 +802,14 @@ TiledShape tiled_wide_shape() {
     return s;
 }
 
-// regions of at most 64 x 64 (two 32-lane column passes per row); shapes
+// 0: regions of at most 64 x 64 (two 32-lane column passes per row);
 // 3..10: the iterate in registers at depths 4, 8, 2, 7, 6, 5, 3 and 1;
-// 11, 12: registers on 64 x 128 regions at depths 8 and 4; 13, 14:
-// registers on 96 x 64 regions (12 warps) at depths 8 and 7 (tiles: 2D less, along
-// x2 at odd depths 2D + 2 less)
-constexpr int kTiledShapes = 15;
-
+// 11: registers on 64 x 128 regions at depth 8; 13, 14: registers on 96 x 64
+// regions (12 warps) at depths 8 and 7 (tiles: 2D less, along x2 at odd depths
+// 2D + 2 less)
 bool tiled_shape_for(int idx, TiledShape &s) {
     switch (idx) {
         case 0: s = tiled_shape<56, 4>(); return true;
-        case 1: s = tiled_shape<60, 2>(); return true;
-        case 2: s = tiled_shape<48, 8>(); return true;
         case 3: s = tiled_reg_shape<4>(); return true;
         case 4: s = tiled_reg_shape<8>(); return true;
         case 5: s = tiled_reg_shape<2>(); return true;
@@ -823,7 +819,6 @@ bool tiled_shape_for(int idx, TiledShape &s) {
         case 9: s = tiled_reg_shape<3>(); return true;
         case 10: s = tiled_reg_shape<1>(); return true;
         case 11: s = tiled_wide_shape<8, 4>(); return true;
-        case 12: s = tiled_wide_shape<4, 4>(); return true;
         case 13: s = tiled_reg_shape<8, 12>(); return true;
         case 14: s = tiled_reg_shape<7, 12>(); return true;
         default: return false;
@@ -855,8 +850,6 @@ static double settle_columns(const ctqw_hamiltonian *h, TiledShape &f) {
     f.TMAX2 = f.T2_flush;
     return all_odd ? 1.0 : 1.15;
 }
-
-int tiled_shape_count() { return kTiledShapes; }
 
 bool tiled_supported(const ctqw_hamiltonian *h, int dtype, int shape) {
     TiledShape s;
