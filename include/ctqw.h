@@ -240,7 +240,8 @@ int ctqw_autotune_order(const ctqw_hamiltonian *h, int32_t dtype, double dt, int
  * needs the workspace of ctqw_workspace_size (3 states).  The fused path
  * keeps the carried error in the first state and stores the state at
  * sample points into the others (S = workspace_bytes / state bytes - 1
- * slots); one launch covers S + 1 sampling intervals, so a larger
+ * slots); one launch covers S + 1 sampling intervals (S, with neither norms nor
+ * energies and less than 4 bytes behind the slots), so a larger
  * workspace means fewer launches.  Given no workspace, the fused path
  * allocates its 3 states stream-ordered (N a multiple of 64 only).  With S >= 2 and enough
  * realizations, the fused path also runs the last ctqw_fused_split

@@ -754,7 +754,7 @@ static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double
     size_t wsb = workspace_bytes;
     bool own = false;
     if (!ws) {
-        wsb = 3 * sb;
+        wsb = 3 * sb + sizeof(int);
         CTQW_CUDA_TRY(ctqw_malloc_async(&ws, wsb, s));
         own = true;
     } else if (wsb < sb) {
@@ -779,6 +779,15 @@ static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double
         if (!can) R_t = 0;
     }
     const int R_f = h->R - R_t;
+    // A launch's counter (the word its clusters take their realizations from) is
+    // in memory of this call that nothing else uses meanwhile: behind the slots;
+    // in a slot without a snapshot, at realization 0, which is never on the tiles;
+    // or, with snapshots in all of them, the norm or energy of realization 0 in
+    // the sample that follows the launch.  Where there is none of these, the last
+    // slot is left free.
+    int *const behind = wsb - (size_t)(slots + 1) * sb >= sizeof(int) ? (int *)(w + (size_t)(slots + 1) * sb) : nullptr;
+    double *const later = norm_dev ? norm_dev : energy_dev;
+    const bool counted = R_f > h->rows_clusters;
     cudaStream_t side = s;
     if (st == CTQW_OK && R_t > 0) {
         if (cudaEventRecord(h->fork_ev, s) != cudaSuccess || cudaStreamWaitEvent(h->side, h->fork_ev, 0) != cudaSuccess)
@@ -795,11 +804,23 @@ static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double
     for (int64_t s0 = 0; st == CTQW_OK;) {
         if (obs_every > 0 && s0 % obs_every == 0) st = observe(psi_dev, s0 / obs_every);
         if (st != CTQW_OK || s0 == n_steps) break;
-        const int64_t chunk = obs_every > 0 ? std::min<int64_t>(n_steps - s0, (slots + 1) * obs_every)
-                                            : n_steps - s0;
-        const int64_t inside = obs_every > 0 ? (chunk - 1) / obs_every : 0;   // snapshots of this launch
+        int64_t chunk = obs_every > 0 ? std::min<int64_t>(n_steps - s0, (slots + 1) * obs_every) : n_steps - s0;
+        int64_t inside = obs_every > 0 ? (chunk - 1) / obs_every : 0;   // snapshots of this launch
+        int *work = behind;
+        double *borrowed = nullptr;
+        if (!work && counted && slots > 0) {
+            if (inside == slots && chunk % obs_every == 0 && later) {
+                borrowed = later + ((s0 + chunk) / obs_every) * h->R;
+                work = (int *)borrowed;
+            } else {
+                if (inside == slots) chunk = inside-- * obs_every;
+                work = (int *)(w + (size_t)slots * sb);
+            }
+        }
         st = launch_taylor_fused_rows(h, psi_dev, lo, inside > 0 ? w + sb : nullptr, obs_every, dt, K,
-                                      chunk, comp, shape, test, 0, R_f, s);
+                                      chunk, comp, shape, test, 0, R_f, work, s);
+        if (borrowed && st == CTQW_OK && cudaMemsetAsync(borrowed, 0, sizeof(double), s) != cudaSuccess)
+            st = ctqw_cuda_fail(cudaGetLastError(), "memset");
         test = 0;
         for (int64_t q = 0; st == CTQW_OK && q < inside; ++q)
             st = observe(w + (size_t)(q + 1) * sb, s0 / obs_every + q + 1);
@@ -935,6 +956,7 @@ static int propagate_switching_impl(const ctqw_hamiltonian *h, int32_t dtype, vo
         // launch per sampling interval, since a sample uses H of its step
         CTQW_TRY(zero_outputs(h, n_samples(n_steps, obs_every), P_mean_dev, norm_dev, energy_dev, s));
         void *lo = workspace_dev;
+        int *work = (int *)((char *)workspace_dev + (size_t)h->total_amp * sizeof(float2));   // the second state is free
         CTQW_CUDA_TRY(cudaMemsetAsync(lo, 0, (size_t)h->total_amp * sizeof(float2), s));
         const SwitchLaw law = switch_law(h, seed, p_switch);
         for (int64_t s0 = 0;;) {
@@ -947,7 +969,7 @@ static int propagate_switching_impl(const ctqw_hamiltonian *h, int32_t dtype, vo
             if (s0 == n_steps) return CTQW_OK;
             const int64_t chunk = obs_every > 0 ? std::min<int64_t>(n_steps - s0, obs_every) : n_steps;
             CTQW_TRY(launch_taylor_fused_rows_switching(h, psi_dev, lo, dt, K, s0, chunk,
-                                                        (flags & CTQW_FLAG_NO_COMPENSATION) ? 0 : 1, law, s));
+                                                        (flags & CTQW_FLAG_NO_COMPENSATION) ? 0 : 1, law, work, s));
             s0 += chunk;
         }
     }

@@ -267,9 +267,10 @@ int launch_group_sum(const ctqw_hamiltonian *h, const double *grad, double *out,
 // rounding error in and out; when snap is not null the state after every
 // snap_every-th step before the last is stored to slot q = step/snap_every - 1
 // of snap (consecutive states, the layout of psi).  The launch covers
-// realizations r0 .. r0 + R_run - 1, dealt out in turn to one cluster per
-// resident slot; it keeps nothing in the handle, so calls on several streams
-// do not meet.
+// realizations r0 .. r0 + R_run - 1 with one cluster per resident slot.  Where
+// there are more of them than clusters, these take them from the counter `work`
+// in device memory of the call (which the launch zeroes on its stream; null: in
+// turn); nothing is kept in the handle, so calls on several streams do not meet.
 bool fused_rows_supported(const ctqw_hamiltonian *h, int dtype);
 bool fused_rows_switching_supported(const ctqw_hamiltonian *h, int dtype);
 // Picks the split of a lattice over warps, CTAs and the cluster for the
@@ -283,13 +284,13 @@ int plan_fused_rows(ctqw_hamiltonian *h);
 int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled);
 int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap,
                              int snap_every, double dt, int K, int64_t n_steps, int compensated,
-                             int shape, int test_timeout, int r0, int R_run, cudaStream_t s);
+                             int shape, int test_timeout, int r0, int R_run, int *work, cudaStream_t s);
 // The same with switching noise: the Hamiltonian update of `law` after every
 // step (step0 is the first step's number), in the kernel; the handle holds the
 // parameters after the last one.  All realizations.
 int launch_taylor_fused_rows_switching(const ctqw_hamiltonian *h, void *psi, void *lo, double dt, int K,
                                        int64_t step0, int64_t n_steps, int compensated, const SwitchLaw &law,
-                                       cudaStream_t s);
+                                       int *work, cudaStream_t s);
 
 // Fused row-wavefront Taylor propagation (m = 2, c64, open chains): every
 // Taylor term of a step on chip, psi streamed once per step; lo: the carried

@@ -37,6 +37,13 @@ static __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank
     return r;
 }
 
+// 32-bit load from the shared memory of a CTA of the cluster (a map_rank address).
+static __device__ __forceinline__ int ld_shared_cluster_s32(uint32_t raddr) {
+    int v;
+    asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(raddr) : "memory");
+    return v;
+}
+
 static __device__ __forceinline__ void mbar_init(uint32_t mb, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(count) : "memory");
 }

@@ -4,13 +4,14 @@
 // One thread-block cluster owns one realization at a time for all steps of
 // the launch (the order-K Taylor polynomial of Algorithm 3, Sec. 2.3, applied
 // n_steps times).  The grid holds only as many clusters as are resident at
-// once, and cluster q of n takes the realizations q, q + n, q + 2 n, ..., so the
-// SMs a cluster holds stay its own until the launch ends.  (A counter in the
-// handle, from which a cluster took its next realization, was shared by calls
-// that overlap on one handle: they stepped each other's realizations twice or
-// not at all.  All take the same time, so the counter gained nothing: 1024
-// realizations of N = 256, 50 steps: 47.93 ms with it, 47.91 without; 1000 rings
-// of N = 100, 100 steps: 21.75 and 21.83; one of N = 64, 10 steps: 75.8 and 73.5 us.)
+// once, and each takes realization after realization, so the SMs a cluster
+// holds stay its own until the launch ends.  They come from a counter in the
+// call's own workspace (one in the handle would be shared by calls that overlap
+// on it), or, where there is one for each cluster or no room for the counter,
+// in turn.  The counter is for clusters of unequal speed, which share their SMs
+// with others or with the tiles of the second stream: 20 steps of 600 x N = 200
+// 10.6 ms with it and 11.2 in turn on one stream, and in turn up to 17.8 with
+// the tiles; with SMs of their own (1024 x N = 256, 50 steps) 47.9 either way.
 // The N x N tile is split into row slabs, one per CTA; every warp owns RL
 // whole rows and each lane CL adjacent columns of them (N <= 32 CL), so a warp
 // covers full rows: neighbours along x2 are in the lane's registers or one
@@ -47,7 +48,7 @@
 // barrier a stage (K = 16, site-updates/s, one stream): N = 64 1.17e12 ->
 // 1.23e12, N = 128 1.27e12 -> 1.33e12, N = 192 1.01e12 -> 1.23e12, N = 256
 // 9.1e11 -> 1.11e12; N = 100, on the register tiles before, 4.4e11 -> 7.6e11;
-// one realization of N = 64, 10 steps: 129 us -> 74 us.
+// one realization of N = 64, 10 steps: 129 us -> 73 us.
 //
 // Control flow: the stages of a step are a first one (from psi), middle ones
 // in pairs and a final one, with no per-stage dispatch.  A row tests the few
@@ -94,6 +95,7 @@ struct RowsArgs {
     unsigned long long wait_limit_ns;
     int test_timeout;
     int r0, R_run;          // realizations r0 .. r0 + R_run - 1
+    int *work;              // counter they are taken from, zero at the launch; null: cluster by cluster in turn
     // switching noise: the law, the number of the first step, and the
     // parameters to leave the updated values in
     SwitchLaw law;
@@ -161,6 +163,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
     __shared__ __align__(8) unsigned long long mbar[2][2];      // halo rows: [parity][above, below]
     __shared__ __align__(8) unsigned long long mbar_edge;       // the CTA's warps have published a stage
     __shared__ __align__(8) unsigned long long mbar_never;
+    __shared__ int next_r;
 
     const int rank = (int)cluster_rank();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -274,6 +277,7 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
             for (int sd = 0; sd < 2; ++sd) mbar_init(smem_u32(&mbar[q][sd]), 1);
         mbar_init(mb_edge, my_warps > 0 ? my_warps : 1);
         mbar_init(smem_u32(&mbar_never), 1);
+        next_r = a.r0 + (int)blockIdx.x / C - (int)gridDim.x / C;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     cluster_barrier();
@@ -282,6 +286,16 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
 
     const long long n_steps = a.n_steps;
     const int K = a.K;
+    // this cluster's next realization, which CTA 0 reads from its counter (or
+    // counts on by itself) and the others from CTA 0.  Every warp of the cluster
+    // is done with the last one's shared memory when it returns.
+    auto next = [&]() -> int {
+        if (rank == 0 && threadIdx.x == 0) next_r = a.work ? a.r0 + atomicAdd(a.work, 1) : next_r + (int)gridDim.x / C;
+        cluster_barrier();
+        const int r = ld_shared_cluster_s32(map_rank(smem_u32(&next_r), 0));
+        cluster_barrier();
+        return r;
+    };
     // edge rows of the warp and of its neighbours, by parity (with one CTA the
     // slab's edges are each other's neighbours)
     const bool push_up = C > 1 && top, push_dn = C > 1 && bottom;
@@ -391,9 +405,8 @@ __global__ void __launch_bounds__(32 * MAXW, 1) taylor_fused_rows_kernel(const _
                 Q[i][k + 1] = pack2(h1.x, h1.y);
             }
         };
-        const int r_end = a.r0 + a.R_run, clusters = (int)gridDim.x / C;
-        for (int r = a.r0 + (int)blockIdx.x / C; r < r_end; r += clusters) {
-            cluster_barrier();   // every warp is done with the last one's shared memory
+        const int r_end = a.r0 + a.R_run;
+        for (int r = next(); r < r_end; r = next()) {
             load_realization(r);
             if (SWITCH)
                 cluster_barrier();   // every CTA has read the parameters that CTA 0 overwrites when it is done
@@ -668,7 +681,7 @@ int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) 
 }
 
 static int launch_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap, int snap_every, double dt, int K,
-                       int64_t n_steps, int compensated, int shape, int test_timeout, int r0, int R_run,
+                       int64_t n_steps, int compensated, int shape, int test_timeout, int r0, int R_run, int *work,
                        const SwitchLaw *law, int64_t step0, cudaStream_t s) {
     RowsShape f;
     if (!rows_shape_of(h, shape, f)) {
@@ -739,19 +752,21 @@ static int launch_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *sna
     }
     // one cluster per resident slot
     cfg.gridDim = dim3((unsigned)(std::min(R_run, clusters) * f.C));
+    a.work = R_run > clusters ? work : nullptr;
+    if (a.work) CTQW_CUDA_TRY(cudaMemsetAsync(a.work, 0, sizeof(int), s));
     CTQW_CUDA_TRY(cudaLaunchKernelEx(&cfg, f.kern, a));
     return CTQW_OK;
 }
 
 int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap, int snap_every, double dt,
                              int K, int64_t n_steps, int compensated, int shape, int test_timeout, int r0,
-                             int R_run, cudaStream_t s) {
-    return launch_rows(h, psi, lo, snap, snap_every, dt, K, n_steps, compensated, shape, test_timeout, r0, R_run, nullptr,
-                       0, s);
+                             int R_run, int *work, cudaStream_t s) {
+    return launch_rows(h, psi, lo, snap, snap_every, dt, K, n_steps, compensated, shape, test_timeout, r0, R_run, work,
+                       nullptr, 0, s);
 }
 
 int launch_taylor_fused_rows_switching(const ctqw_hamiltonian *h, void *psi, void *lo, double dt, int K,
                                        int64_t step0, int64_t n_steps, int compensated, const SwitchLaw &law,
-                                       cudaStream_t s) {
-    return launch_rows(h, psi, lo, nullptr, 0, dt, K, n_steps, compensated, 0, 0, 0, h->R, &law, step0, s);
+                                       int *work, cudaStream_t s) {
+    return launch_rows(h, psi, lo, nullptr, 0, dt, K, n_steps, compensated, 0, 0, 0, h->R, work, &law, step0, s);
 }

@@ -119,3 +119,37 @@ def test_a_call_beside_another_calls_capture(ctqw):
     ctqw.ctqw_check_status(h)
     assert np.array_equal(psis[0].cpu().numpy(), expect[0])
     h.close()
+
+
+@pytest.mark.parametrize("outputs", ["PNE", "P", "E", ""])
+@pytest.mark.parametrize("N,R,states", [(200, 60, 3), (64, 700, 1), (64, 700, 2), (64, 700, 5), (256, 40, 3), (256, 150, 3)])
+def test_where_the_counter_lies(ctqw, N, R, states, outputs):
+    # more realizations than clusters: their counter lies in the workspace or
+    # in a sample that is written later, whatever these leave room for (launches
+    # of several sampling intervals, the last one cut off); against a workspace
+    # with room for it behind the states.
+    w = cw.get("bosons_n256_u2").with_(N=N, R=R, K=5, sites=(N // 2 - 1, N // 2))
+    every, steps = 2, 17
+    h = ctqw.build_for_workload(w)
+    rng = np.random.default_rng(R)
+    v = rng.standard_normal(h.total_amplitudes) + 1j * rng.standard_normal(h.total_amplitudes)
+    v = torch.from_numpy((v / np.linalg.norm(v) * np.sqrt(R)).astype(np.complex64)).cuda()
+    full = ctqw._outputs(h, h.n_obs(steps, every), True, True, True, "cuda")
+    for o in full:
+        o.fill_(7.0)
+    got = [o if c in outputs else None for c, o in zip("PNE", full)]
+    flags = ctqw.FLAG_ONE_STREAM if R != 150 else 0
+    psi = v.clone()
+    ws = torch.empty(states * 8 * h.total_amplitudes, dtype=torch.uint8, device="cuda")
+    ctqw.ctqw_propagate_taylor(h, psi, cw.C64, w.dt, w.K, steps, every, *got, flags, ws)
+    ctqw.ctqw_check_status(h)
+    ref = v.clone()
+    room = torch.empty(3 * 8 * h.total_amplitudes + 16, dtype=torch.uint8, device="cuda")
+    again = ctqw._outputs(h, h.n_obs(steps, every), True, True, True, "cuda")
+    ctqw.ctqw_propagate_taylor(h, ref, cw.C64, w.dt, w.K, steps, every, *again, flags, room)
+    ctqw.ctqw_check_status(h)
+    h.close()
+    assert torch.equal(psi, ref)
+    for a, b in zip(got, again):
+        if a is not None:   # the same terms in another order: FP64 sums of order 10
+            assert float((a - b).abs().max()) <= 1e-12
