@@ -306,6 +306,9 @@ int launch_taylor_wavefront(const ctqw_hamiltonian *h, void *psi, void *lo, doub
 bool tiled_supported(const ctqw_hamiltonian *h, int dtype, int shape);
 int tiled_depth(int shape);
 int tiled_default_shape(const ctqw_hamiltonian *h, int K);   // the register tiles' region and depth for the sizes
+// Microseconds a stage that one round of tile blocks takes on any SMs (default
+// shape, one size); *blocks of them a realization, *resident on an SM.
+double tiled_round_us(const ctqw_hamiltonian *h, int K, int *blocks, int *resident);
 int launch_taylor_tiled(const ctqw_hamiltonian *h, int shape, const void *w_in, const void *psi,
                         void *w_out, void *lo, double dt, int j0, int n_stages, int final,
                         int compensated, cudaStream_t s);

@@ -640,12 +640,6 @@ int plan_fused_rows(ctqw_hamiltonian *h) {
     return CTQW_OK;
 }
 
-// Tiled-to-fused throughput ratio per SM on two bosons at N = 256, K = 16
-// (register tiles 4.43e11 site-updates/s on 152 SMs, the full-row clusters
-// 1.11e12 on the 120 that hold them: 0.32).  1024 realizations, 50 steps: 62
-// rounds of clusters 47.8 ms, 63 48.4; 0.39 gives 62.
-static constexpr double kTiledPerSmRatio = 0.39;
-
 int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) {
     *R_tiled = 0;
     if (shape != 0 || h->rows_clusters < 1 || h->group_N.size() != 1 ||
@@ -657,20 +651,30 @@ int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled) 
     const int used = std::min(n_sm, (clusters * h->rows_C + per_sm - 1) / per_sm);
     const int idle = n_sm - used;
     if (idle * 16 < n_sm) return CTQW_OK;   // under 1/16 of the SMs idle: not worth a second stream
-    // the rounds of resident clusters with the least time of the longer part,
-    // a stage: so many rounds, against the tiles' throughput on the SMs left over
-    // and what a launch takes however few tiles it has (17 us for 8 stages: 1 of
-    // 24 x N = 192 on the tiles made 20 steps of K = 16 0.70 ms instead of 0.41).
-    // A share by throughput alone also gave: 77 x N = 192 1.27 ms, now 0.85; 20 x
-    // N = 256 0.96, now 0.53; 40 x N = 160 1.15, now 0.53.
-    constexpr double kTiledStageUs = 2.2;
-    const double tiled_us = h->rows_stage_us * used / (clusters * kTiledPerSmRatio * idle);   // a realization
+    // few SMs idle (clusters of 5 CTAs leave 12): at the launch the tiles may hold
+    // an SM that a cluster needs, so only shares that take well under the clusters'
+    // time (of 581 x N = 145 21 on the tiles: 60 steps 7.34 to 8 ms instead of 7.55;
+    // 24 of 640 x 156: no gain; clusters of 6 leave 14: no such loss)
+    const double margin = idle * 12 < n_sm ? 1.6 : 1.0;
+    // two CTAs an SM: tiles that hold half an SM when the clusters are launched
+    // keep some of them out for the whole launch (20 steps of K = 16, one stream
+    // and with 8% on the tiles: 600 x N = 200 10.5 and 12.0 to 13.7 ms, 350 x 196
+    // 6.3 and 6.8 to 8.3, 200 x 200 3.7 and 3.5 to 4.8)
+    if (per_sm > 1) return CTQW_OK;
+    // the rounds of resident clusters with the least time of the longer part, a
+    // stage: so many rounds of clusters, against so many rounds of tile blocks on
+    // the SMs left over
+    int blocks = 0;   // of a realization, and resident on an SM
+    int resident = 1;
+    const double round_us = tiled_round_us(h, K, &blocks, &resident);
     const int most = (h->R + clusters - 1) / clusters;
     int R_f = h->R;
     double best = most * h->rows_stage_us;
     for (int rounds = std::max(1, most / 2); rounds < most; ++rounds) {
-        const double t = std::max(rounds * h->rows_stage_us,
-                                  std::max(kTiledStageUs, (h->R - rounds * clusters) * tiled_us));
+        const int64_t all = (int64_t)(h->R - rounds * clusters) * blocks, at_once = idle * resident;
+        double tile_rounds = (double)(all / at_once);
+        if (all % at_once) tile_rounds += 0.6 + 0.4 * (double)(all % at_once) / at_once;   // fewer blocks an SM, a little sooner
+        const double t = std::max(rounds * h->rows_stage_us, margin * tile_rounds * round_us);
         if (t < best) {
             best = t;
             R_f = rounds * clusters;

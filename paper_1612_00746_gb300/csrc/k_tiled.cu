@@ -876,9 +876,10 @@ int tiled_depth(int shape) {
 // N = 512 4.99e11 against 5.03e11.
 // Where every tile finds an SM of its own, launches are all that counts: the
 // 64 x 64 regions at the even split of the fewest launches.
+static constexpr double kTileFixed = 1180.0, kRowStage = 27.0, kTallRate = 0.94;
+
 int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
     static const int by_depth[9] = {4, 10, 5, 9, 3, 8, 7, 6, 4};   // 64 x 64 regions
-    constexpr double kTileFixed = 1180.0, kRowStage = 27.0, kTallRate = 0.94;
     int best = by_depth[8];
     double best_cost = 0.0;
     auto consider = [&](int shape) {
@@ -920,6 +921,25 @@ int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
     if (even8 == 8) consider(13);
     if (even8 == 7) consider(14);
     return best;
+}
+
+// A round of blocks (24 warps an SM) beside the clusters takes 4.45 ns for each
+// instruction of a tile's warp (tiled_default_shape), and a fifth more at odd N,
+// whose copies are of 8 bytes, where a step is several launches.  So the best
+// share of R x N, K measured (realizations on the tiles, and what others cost): 1024 x
+// 256, 16: 94 (64 +2.5%, 109 +2.4%); 300 x 240, 5: 30 (15 +3%); 600 x 192, 16: 25 (2 +3%);
+// 356 x 237, 12: 26 (41 +4%); 181 x 221, 12: 16 (31 +4%); 286 x 187, 4: 10 (0 +5%).
+// With all SMs to themselves the tiles take 5.3 ns.
+double tiled_round_us(const ctqw_hamiltonian *h, int K, int *blocks, int *resident) {
+    constexpr double kInstructionUs = 4.45e-3;
+    TiledShape f;
+    tiled_shape_for(tiled_default_shape(h, K), f);
+    double rate = settle_columns(h, f);
+    if (h->Nmax % 2 && K > f.D) rate *= 1.2;
+    *blocks = ((h->Nmax + f.TMAX - 1) / f.TMAX) * ((h->Nmax + f.TMAX2 - 1) / f.TMAX2);
+    *resident = f.threads > 256 ? 2 : 3;
+    const int launches = (K + f.D - 1) / f.D;
+    return kInstructionUs * rate / (f.threads > 256 ? kTallRate : 1.0) * (launches * kTileFixed / K + 8.0 * kRowStage);
 }
 
 int launch_taylor_tiled_range(const ctqw_hamiltonian *h, int shape, const void *w_in, const void *psi,
