@@ -76,7 +76,8 @@ extern "C" {
  * through a pipeline; open chains, N in {64, 128, 192, 256}, also ragged,
  * K <= 16 with N + 1 > 2K + 8; needs ctqw_workspace_size bytes of workspace,
  * one c64 state, or allocates it stream-ordered when workspace_dev is NULL).
- * An index with no compiled shape returns CTQW_EUNSUPPORTED. */
+ * k = 4..8 read pairs of amplitudes: psi_dev and workspace_dev on a 16-byte
+ * boundary, else CTQW_EINVAL.  An index with no compiled shape returns CTQW_EUNSUPPORTED. */
 #define CTQW_FUSED_SHAPE_SHIFT 8
 #define CTQW_FUSED_SHAPE(k) (((uint32_t)(k) & 0xFu) << CTQW_FUSED_SHAPE_SHIFT)
 #define CTQW_SHAPE_WAVEFRONT 8
@@ -354,7 +355,8 @@ int ctqw_propagate_rk4(const ctqw_hamiltonian *h, int32_t dtype, void *psi_dev, 
  * device, complex128 (interleaved re, im), group g's N_g x N_g block
  * row-major starting at element sum_{g' < g} N_g'^2 (the order of
  * ctqw_output_layout's groups); overwritten (zeroed on the stream first).
- * CTQW_C64 with every group's N a multiple of 16 (up to 2048) runs on the
+ * CTQW_C64 with every group's N a multiple of 16 (up to 2048) and psi_dev on a
+ * 16-byte boundary runs on the
  * tensor cores (tcgen05, TF32): each FP32 amplitude is split into two TF32
  * pieces and every product formed from three piece products (~2^-22
  * relative), accumulated in FP32 in tensor memory over at most 256 k and
@@ -510,8 +512,9 @@ int ctqw_inject_no_clusters(ctqw_hamiltonian *h);
  * are the fastest index, amplitude s (x_m fastest, as above) of realization
  * r at s Rp + r with Rp = R rounded up to a multiple of 4 (the padding
  * realizations stay zero), so that the kernels read every neighbour as one
- * coalesced row across realizations, four realizations per thread.  The topology is stored once as the CSR of the
- * one-particle graph; the N^m x (mk + 1) many-particle topology of Sec. 2
+ * coalesced row across realizations, four realizations per thread; c64 states
+ * and workspaces start on a 16-byte boundary (else CTQW_EINVAL where a kernel
+ * reads them so).  The topology is stored once as the CSR of the one-particle graph; the N^m x (mk + 1) many-particle topology of Sec. 2
  * is regenerated inside the kernels.
  * ------------------------------------------------------------------------ */
 typedef struct ctqw_graph ctqw_graph;   /* opaque, owned by the library */

@@ -497,6 +497,7 @@ static int propagate_wavefront(const ctqw_hamiltonian *h, int32_t dtype, void *p
                        "256} with N + 1 > 2K + 8, and K <= 16");
         return CTQW_EUNSUPPORTED;
     }
+    CTQW_TRY(check_pairs_aligned("wavefront path", psi_dev, workspace_dev));
     const size_t need = wavefront_workspace_bytes(h);
     void *lo = workspace_dev;
     bool own = false;
@@ -894,6 +895,7 @@ static int propagate_taylor_impl(const ctqw_hamiltonian *h, int32_t dtype, void 
             return CTQW_EINVAL;
         }
     }
+    if (fused && shape >= 4) CTQW_TRY(check_pairs_aligned("banded fused path", psi_dev));
     CTQW_TRY(zero_outputs(h, n_obs, P_mean_dev, norm_dev, energy_dev, s));
     if (fused) {
         // shape index 0..3: full-row kernel; 4..7: the banded kernel (shape - 4)
@@ -1301,7 +1303,8 @@ int ctqw_one_body_density(const ctqw_hamiltonian *h, int32_t dtype, const void *
     if (dtype != CTQW_C64 && dtype != CTQW_C128) { ctqw_set_error("dtype %d", dtype); return CTQW_EINVAL; }
     cudaStream_t s = (cudaStream_t)stream;
     CTQW_CUDA_TRY(cudaMemsetAsync(rho_dev, 0, 2 * sizeof(double) * (size_t)h->joint_width, s));
-    if (h->density_method == 0 && one_body_density_tc_supported(h, dtype))
+    // the tensor-core kernel loads two amplitudes at a time
+    if (h->density_method == 0 && one_body_density_tc_supported(h, dtype) && ((uintptr_t)psi_dev & 15) == 0)
         return launch_one_body_density_tc(h, psi_dev, rho_dev, s);
     return launch_one_body_density(h, dtype, psi_dev, rho_dev, s);
 }

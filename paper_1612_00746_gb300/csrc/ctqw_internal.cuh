@@ -119,6 +119,15 @@ int launch_norm_check(const ctqw_hamiltonian *h, const double *norm, int64_t n_o
         if (_e != cudaSuccess) return ctqw_cuda_fail(_e, #call); \
     } while (0)
 
+// EINVAL unless the buffers of a kernel that reads pairs of c64 amplitudes
+// start on 16 bytes (null ones do).
+template <typename... Ptr>
+inline int check_pairs_aligned(const char *what, Ptr... p) {
+    if (((0 | ... | (uintptr_t)p) & 15) == 0) return CTQW_OK;
+    ctqw_set_error("%s: psi and workspace must start on a 16-byte boundary", what);
+    return CTQW_EINVAL;
+}
+
 // Propagate a nonzero status of a library call.
 #define CTQW_TRY(expr)                  \
     do {                                \

@@ -483,6 +483,7 @@ int launch_graph_init_state(const ctqw_graph *g, const int32_t *sites_d, int dty
 
 int launch_graph_horner_stage(const ctqw_graph *g, int rb, int re, const void *in, const void *psi,
                               void *out, double coef, cudaStream_t s) {
+    CTQW_TRY(check_pairs_aligned("graph stage", in, psi, out));
     const Launch l = graph_launch(g, rb, re);
     auto k = g->m == 2 ? graph_horner_stage_kernel<2> : graph_horner_stage_kernel<3>;
     k<<<l.grid, l.block, 0, s>>>(graph_view(g, rb, re), g->eps32, g->w32, (const float2 *)in,
@@ -493,6 +494,7 @@ int launch_graph_horner_stage(const ctqw_graph *g, int rb, int re, const void *i
 
 int launch_graph_horner_final(const ctqw_graph *g, int rb, int re, const void *w2, void *psi, void *lo,
                               double dt, cudaStream_t s) {
+    CTQW_TRY(check_pairs_aligned("graph stage", w2, psi, lo));
     const Launch l = graph_launch(g, rb, re);
     auto k = g->m == 2 ? graph_horner_final_kernel<2> : graph_horner_final_kernel<3>;
     k<<<l.grid, l.block, 0, s>>>(graph_view(g, rb, re), g->eps32, g->w32, (const float2 *)w2, (float2 *)psi,
@@ -503,6 +505,7 @@ int launch_graph_horner_final(const ctqw_graph *g, int rb, int re, const void *w
 
 int launch_graph_taylor_term(const ctqw_graph *g, int rb, int re, int dtype, const void *in, void *out,
                              const void *psi, void *acc, double coef, int first, cudaStream_t s) {
+    CTQW_TRY(check_pairs_aligned("graph stage", in, out, psi, acc));
     const Launch l = graph_launch(g, rb, re);
     if (dtype == CTQW_C64) {
         auto k = g->m == 2 ? graph_taylor_term_kernel<float, 2> : graph_taylor_term_kernel<float, 3>;
@@ -519,6 +522,7 @@ int launch_graph_taylor_term(const ctqw_graph *g, int rb, int re, int dtype, con
 
 int launch_graph_rk4_stage(const ctqw_graph *g, int rb, int re, int dtype, const void *in, void *next,
                            const void *psi, void *acc, double a, double b, int first, cudaStream_t s) {
+    CTQW_TRY(check_pairs_aligned("graph stage", in, next, psi, acc));
     const Launch l = graph_launch(g, rb, re);
     if (dtype == CTQW_C64) {
         auto k = g->m == 2 ? graph_rk4_stage_kernel<float, 2> : graph_rk4_stage_kernel<float, 3>;
@@ -536,6 +540,7 @@ int launch_graph_rk4_stage(const ctqw_graph *g, int rb, int re, int dtype, const
 int launch_graph_observables(const ctqw_graph *g, int rb, int re, int dtype, const void *psi,
                              double *P_mean, double *norm, double *energy, cudaStream_t s) {
     if (!P_mean && !norm && !energy) return CTQW_OK;
+    CTQW_TRY(check_pairs_aligned("graph observables", psi));
     const int n_rows = (int)(g->D / g->N);
     const dim3 grid((unsigned)((n_rows + kRows - 1) / kRows), (unsigned)((re - rb + 127) / 128));
     const dim3 block(32, kObsWarps);
