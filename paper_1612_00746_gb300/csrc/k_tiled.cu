@@ -861,57 +861,48 @@ int tiled_depth(int shape) {
     return tiled_shape_for(shape, s) ? s.D : 0;
 }
 
-// The register tiles' depth (and region) for this handle and order: the
-// least of launches x tiles x (kTileFixed + 8 kRowStage stages), the warp
-// instructions of a tile, over the depths 1..8.  A tile costs a fixed part
-// (loads, coefficients, the compensated update) and its rows' stages; deeper
-// launches are fewer but leave a smaller tile, and where N is little more
-// than a whole number of tiles the next shallower one covers it with fewer.
-// The two constants are from the 64 x 64 tiles' counters at depths 8 and 4
-// (2918 and 2049 warp instructions a tile and warp).  Measured, K = 16
-// (site-updates/s at depths 8 / 4): N = 1024 5.16e11 / 5.02e11, N = 256
-// 4.20e11 / 4.43e11, N = 128 4.02e11 / 3.11e11, N = 100 2.45e11 / 3.73e11.
-// The 96 x 64 regions (depth 7 and 8 only) run at 0.94 of the rate a region
-// point and are taken where they save more than that: N = 1024 5.44e11,
-// N = 512 4.99e11 against 5.03e11.
-// Where every tile finds an SM of its own, launches are all that counts: the
-// 64 x 64 regions at the even split of the fewest launches.
-static constexpr double kTileFixed = 1180.0, kRowStage = 27.0, kTallRate = 0.94;
+// The register tiles' depth (and region) for this handle and order: the least
+// time by a model over the depths 1..8.  A launch takes kLaunch, and its tiles
+// run in rounds of three blocks an SM, each of them a fixed part (loads,
+// coefficients, the compensated update) and a part for every stage; the last
+// round takes half a round and the rest by how full it is.  So deeper launches
+// are fewer but leave a smaller tile, the next shallower depth may cover the
+// lattice with fewer tiles, and where the tiles do not fill the SMs the launches
+// are what counts.  The constants, in warp instructions, are fitted to 450
+// calls at every depth (N = 20..1150, also ragged, 3 to 10000 tiles, K = 3..20): the
+// choice is 0.3% above the best depth on average, 12% at most.  By the number of
+// tiles alone it was 1.2%, up to 47% where they do not fill the SMs (10 steps of R
+// x N, K: 7 x 277, 7 299 us, now 224; 6 x 318, 17 606 and 481; 6 x 501, 8 498 and 437).
+// The 96 x 64 regions (depth 7 and 8 only, two blocks an SM) run at 0.94 of the
+// rate a region point.
+static constexpr double kTileFixed = 1180.0, kTileStage = 170.0, kLaunch = 1000.0, kTallRate = 0.94;
 
 int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
     static const int by_depth[9] = {4, 10, 5, 9, 3, 8, 7, 6, 4};   // 64 x 64 regions
-    int best = by_depth[8];
+    int best = by_depth[8], n_sm = 152;
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device);
     double best_cost = 0.0;
     auto consider = [&](int shape) {
         TiledShape f;
         if (!tiled_shape_for(shape, f)) return;
         const double rate = settle_columns(h, f);
-        double tiles = 0.0;
+        int64_t tiles = 0;
         for (size_t g = 0; g < h->group_N.size(); ++g) {
             const int N = h->group_N[g];
-            tiles += (double)h->group_count[g] * ((N + f.TMAX - 1) / f.TMAX) * ((N + f.TMAX2 - 1) / f.TMAX2);
+            tiles += (int64_t)h->group_count[g] * ((N + f.TMAX - 1) / f.TMAX) * ((N + f.TMAX2 - 1) / f.TMAX2);
         }
         const int launches = (K + f.D - 1) / f.D;
-        double cost = rate * tiles * (f.threads / 256.0) * (launches * kTileFixed + 8.0 * kRowStage * K);
-        if (f.threads > 256) cost /= kTallRate;
+        const bool tall = f.threads > 256;   // two blocks an SM, else three
+        const int64_t at_once = (tall ? 2 : 3) * n_sm, rest = tiles % at_once;
+        const double rounds = (double)(tiles / at_once) + (rest ? 0.5 + 0.5 * (double)rest / (double)at_once : 0.0);
+        const double cost = launches * kLaunch +
+                            rate * rounds / (tall ? kTallRate : 1.0) * (launches * kTileFixed + kTileStage * K);
         if (best_cost == 0.0 || cost < best_cost) {
             best = shape;
             best_cost = cost;
         }
     };
     const int few = (K + 7) / 8, even8 = (K + few - 1) / few;
-    {
-        TiledShape f;
-        int n_sm = 152;
-        tiled_shape_for(by_depth[even8], f);
-        settle_columns(h, f);
-        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, h->device);
-        int64_t tiles = 0;
-        for (size_t g = 0; g < h->group_N.size(); ++g)
-            tiles += (int64_t)h->group_count[g] * ((h->group_N[g] + f.TMAX - 1) / f.TMAX) *
-                     ((h->group_N[g] + f.TMAX2 - 1) / f.TMAX2);
-        if (tiles <= n_sm) return by_depth[even8];
-    }
     for (int d = 8; d >= 1; --d) {
         // only depths that split the stages evenly: another one does the same
         // launches on smaller tiles
@@ -924,14 +915,15 @@ int tiled_default_shape(const ctqw_hamiltonian *h, int K) {
 }
 
 // A round of blocks (24 warps an SM) beside the clusters takes 4.45 ns for each
-// instruction of a tile's warp (tiled_default_shape), and a fifth more at odd N,
+// instruction of a tile's warp (1180 a launch and 216 a stage, from the counters
+// of the 64 x 64 tiles at depths 8 and 4: 2918 and 2049), and a fifth more at odd N,
 // whose copies are of 8 bytes, where a step is several launches.  So the best
 // share of R x N, K measured (realizations on the tiles, and what others cost): 1024 x
 // 256, 16: 94 (64 +2.5%, 109 +2.4%); 300 x 240, 5: 30 (15 +3%); 600 x 192, 16: 25 (2 +3%);
 // 356 x 237, 12: 26 (41 +4%); 181 x 221, 12: 16 (31 +4%); 286 x 187, 4: 10 (0 +5%).
 // With all SMs to themselves the tiles take 5.3 ns.
 double tiled_round_us(const ctqw_hamiltonian *h, int K, int *blocks, int *resident) {
-    constexpr double kInstructionUs = 4.45e-3;
+    constexpr double kInstructionUs = 4.45e-3, kFixed = 1180.0, kStage = 216.0;
     TiledShape f;
     tiled_shape_for(tiled_default_shape(h, K), f);
     double rate = settle_columns(h, f);
@@ -939,7 +931,7 @@ double tiled_round_us(const ctqw_hamiltonian *h, int K, int *blocks, int *reside
     *blocks = ((h->Nmax + f.TMAX - 1) / f.TMAX) * ((h->Nmax + f.TMAX2 - 1) / f.TMAX2);
     *resident = f.threads > 256 ? 2 : 3;
     const int launches = (K + f.D - 1) / f.D;
-    return kInstructionUs * rate / (f.threads > 256 ? kTallRate : 1.0) * (launches * kTileFixed / K + 8.0 * kRowStage);
+    return kInstructionUs * rate / (f.threads > 256 ? kTallRate : 1.0) * (launches * kFixed / K + kStage);
 }
 
 int launch_taylor_tiled_range(const ctqw_hamiltonian *h, int shape, const void *w_in, const void *psi,
