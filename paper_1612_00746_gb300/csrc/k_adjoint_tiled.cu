@@ -461,11 +461,12 @@ ChainShape chain_shape() {
     return s;
 }
 
-// Whether every buffer of the launch starts on a 16-byte boundary.
-bool chain_aligned16(const ChainArgs &a) {
+// Whether every buffer of the launch starts on a 16-byte boundary (and its 16-byte
+// copies are not all of two addresses, which is slow).
+bool chain_aligned16(const ctqw_hamiltonian *h, const ChainArgs &a) {
     uintptr_t all = (uintptr_t)a.in | (uintptr_t)a.q | (uintptr_t)a.out;
     for (int i = 0; i < kMaxLevels; ++i) all |= (uintptr_t)a.lev[i] | (uintptr_t)a.mlev[i];
-    return (all & 15) == 0;
+    return (all & 15) == 0 && h->group_N[0] > 2;
 }
 
 // Depth for K levels: the fewest launches at depth <= 8, the levels split
@@ -535,7 +536,7 @@ int launch_adjoint_phi_chain(const ctqw_hamiltonian *h, int K, double dt, void *
         a.in = (const float2 *)levels[a0];
         a.a_in = a0;
         a.n_stages = n;
-        a.aligned16 = chain_aligned16(a);
+        a.aligned16 = chain_aligned16(h, a);
         int off = 0;
         for (size_t g = 0; g < h->group_N.size(); ++g) {
             const int N = h->group_N[g], cnt = h->group_count[g];
@@ -571,7 +572,7 @@ int launch_adjoint_mu_chain(const ctqw_hamiltonian *h, int K, double dt, const v
         a.n_stages = n;
         a.init = init ? 1 : 0;
         a.final = final ? 1 : 0;
-        a.aligned16 = chain_aligned16(a);
+        a.aligned16 = chain_aligned16(h, a);
         int off = 0;
         for (size_t g = 0; g < h->group_N.size(); ++g) {
             const int N = h->group_N[g], cnt = h->group_count[g];
