@@ -1042,7 +1042,13 @@ static int propagate_rk4_impl(const ctqw_hamiltonian *h, int32_t dtype, void *ps
     cudaStream_t s = (cudaStream_t)stream;
     // RK4's update map is the order-4 Taylor polynomial of exp(-i H dt)
     // (Sec. 2.3): the Taylor path of the handle evaluates it directly
-    if (!(flags & (CTQW_FLAG_PLAIN | CTQW_FLAG_RENORMALIZE))) {
+    // (except rings of a few sites that only the tiles take, a tile each: many
+    // more of them than run at once cost more than four stages.  20 steps, tiles
+    // and stages: 614 x N = 6 0.54 and 0.39 ms, 614 x 14 0.53 and 0.56, 2000 x 14 1.20 and
+    // 0.87, 2000 x 22 1.24 and 1.12, 946 x 22 0.72 and 0.76)
+    const bool tiny = dtype == CTQW_C64 && h->m == 2 && h->uniform && !fused_rows_supported(h, dtype) && h->Nmax <= 24 &&
+                      h->R > 57 * std::max(8, h->Nmax);
+    if (!tiny && !(flags & (CTQW_FLAG_PLAIN | CTQW_FLAG_RENORMALIZE))) {
         // a tuning shape only means something at the sizes that have them
         if (!fused_taylor_supported(h, dtype)) flags &= ~(0xFu << CTQW_FUSED_SHAPE_SHIFT);
         return propagate_taylor_impl(h, dtype, psi_dev, dt, 4, n_steps, obs_every, P_mean_dev,
