@@ -291,6 +291,10 @@ int ctqw_graph_propagate_taylor(const ctqw_graph *g, int32_t dtype, void *psi_de
                     CTQW_TRY(sample(g, rb, re, dtype, psi_dev, obs++, P_mean_dev, norm_dev, energy_dev, s));
                 if (step == n_steps) break;
                 const void *in = psi_dev;
+                if (K == 1) {   // the only stage reads its neighbours from a copy
+                    CTQW_CUDA_TRY(cudaMemcpyAsync(wa, psi_dev, sb, cudaMemcpyDeviceToDevice, s));
+                    in = wa;
+                }
                 void *out = wa;
                 for (int j = K; j >= 2; --j) {
                     CTQW_TRY(launch_graph_horner_stage(g, rb, re, in, psi_dev, out, dt / j, s));
