@@ -953,7 +953,16 @@ static int propagate_switching_impl(const ctqw_hamiltonian *h, int32_t dtype, vo
     sw.on = true;
     sw.seed = seed;
     sw.p = p_switch;
-    if (!(flags & CTQW_FLAG_PLAIN) && fused_rows_switching_supported(h, dtype)) {
+    // Clusters where a launch has stages enough: it loads and stores every state,
+    // and after each step rebuilds the coefficients, 20 to 30 us a realization.  The
+    // tiles take less below about N / 12 stages a sampling interval (half of that
+    // where every realization has its cluster at once).  A sample a step, clusters
+    // and tiles: 916 x N = 211, K = 7 43.6 and 26.8 ms (21 steps); 998 x 211, K = 15 16.8 and
+    // 11.5 (6); 168 x 160, K = 14 1.12 and 1.27; 413 x 256, K = 1 4.9 and 3.0; 5 x 256, K = 13
+    // 0.26 and 0.30; 1020 x 58, K = 9, every second step 1.2 and 1.6 (12).
+    const int64_t stages = K * (obs_every > 0 ? std::min<int64_t>(obs_every, n_steps) : n_steps);
+    const bool enough = stages * (h->R <= h->rows_switch_clusters ? 24 : 12) >= h->Nmax;
+    if (!(flags & CTQW_FLAG_PLAIN) && fused_rows_switching_supported(h, dtype) && enough) {
         // the clusters redraw the parameters themselves after every step; a
         // launch per sampling interval, since a sample uses H of its step
         CTQW_TRY(zero_outputs(h, n_samples(n_steps, obs_every), P_mean_dev, norm_dev, energy_dev, s));

@@ -40,7 +40,9 @@ def _oracle(w, r, psi):
     return psi, eps, J
 
 
-@pytest.mark.parametrize("K", [1, 2, 6])
+# (orders of 12 and more a launch run on the clusters at these sizes, the
+# lower ones on the tiles)
+@pytest.mark.parametrize("K", [1, 2, 6, 12, 14])
 @pytest.mark.parametrize("N,R,steps", [(256, 1, 6), (256, 4, 4), (256, 20, 2), (128, 3, 4), (200, 2, 4)])
 def test_a_launch_after_every_step(ctqw, N, R, steps, K):
     w = cw.get("bosons_n256_u2").with_(N=N, R=R, K=K, n_steps=steps, obs_every=1, sites=(N // 2 - 1, N // 2))
