@@ -577,30 +577,30 @@ static int propagate_per_term(const ctqw_hamiltonian *h, int32_t dtype, void *ps
         return CTQW_OK;
     }
     void *wa = ws, *wb = ws + sb;
+    void *cur = psi_dev;   // the state; with K = 1, whose only stage cannot work in place, psi and wa in turn
     int64_t obs = 0;
     for (int64_t step = 0; step <= n_steps; ++step) {
         if (obs_every > 0 && step % obs_every == 0) {
-            CTQW_TRY(launch_observables(h, dtype, psi_dev, P_mean_dev ? P_mean_dev + obs * h->p_width : nullptr,
+            CTQW_TRY(launch_observables(h, dtype, cur, P_mean_dev ? P_mean_dev + obs * h->p_width : nullptr,
                                         nullptr, norm_dev ? norm_dev + obs * h->R : nullptr,
                                         energy_dev ? energy_dev + obs * h->R : nullptr, s));
             ++obs;
         }
         if (step == n_steps) break;
-        const void *in = psi_dev;
-        if (K == 1) {   // the only stage reads its neighbours from a copy
-            CTQW_CUDA_TRY(cudaMemcpyAsync(wa, psi_dev, sb, cudaMemcpyDeviceToDevice, s));
-            in = wa;
-        }
+        const void *in = cur;
         void *out = wa;
-        for (int j = K; j >= 1; --j) {
-            void *o = j == 1 ? psi_dev : out;
-            CTQW_TRY(launch_horner_f64(h, in, psi_dev, o, dt / j, s));
-            in = o;
+        for (int j = K; j >= 2; --j) {
+            CTQW_TRY(launch_horner_f64(h, in, cur, out, dt / j, s));
+            in = out;
             out = (out == wa) ? wb : wa;
         }
-        if (sw.renorm) CTQW_TRY(launch_renormalize(h, dtype, psi_dev, nullptr, s));
+        void *next = K > 1 ? cur : (cur == psi_dev ? wa : psi_dev);
+        CTQW_TRY(launch_horner_f64(h, in, cur, next, dt, s));
+        cur = next;
+        if (sw.renorm) CTQW_TRY(launch_renormalize(h, dtype, cur, nullptr, s));
         if (sw.on) CTQW_TRY(launch_switch_params(h, sw.seed, (uint64_t)step, sw.p, s));
     }
+    if (cur != psi_dev) CTQW_CUDA_TRY(cudaMemcpyAsync(psi_dev, cur, sb, cudaMemcpyDeviceToDevice, s));
     return CTQW_OK;
 }
 
