@@ -2,6 +2,8 @@
 // one launch per Taylor term (or RK4 stage) over all realizations at once
 // (the realization x node loop collapsed into one grid, Sec. 2.2).  These
 // are the plain path: every term streams the iterate and psi through HBM.
+#include <algorithm>
+
 #include "ctqw_internal.cuh"
 #include "stencil.cuh"
 
@@ -158,8 +160,10 @@ int launch_horner_f64(const ctqw_hamiltonian *h, const void *in, const void *psi
         const int tx = N >= 256 ? 256 : ((N + 31) / 32) * 32, ty = 256 / tx;
         const int64_t cols = (N + tx - 1) / tx;
         // longer walks scale and reload less, but the FP64 pipes of all SMs
-        // have to get work: at least six blocks an SM, or one row a thread
-        int rows = kF64Rows;
+        // have to get work: at least six blocks an SM, or one row a thread.  No
+        // more rows than give every thread row some of them (1953 x N = 11 with
+        // switching noise, 19 steps of K = 12: 8.3 ms with 16, 5.5 with 2)
+        int rows = std::min(kF64Rows, (N + ty - 1) / ty);
         while (rows > 1 && (int64_t)((N + ty * rows - 1) / (ty * rows)) * cols * cnt < 912) rows /= 2;
         for (int done = 0; done < cnt; done += 65535) {
             const int part = cnt - done < 65535 ? cnt - done : 65535;
