@@ -461,12 +461,12 @@ ChainShape chain_shape() {
     return s;
 }
 
-// Whether every buffer of the launch starts on a 16-byte boundary (and its 16-byte
-// copies are not all of two addresses, which is slow).
+// Whether every buffer of the launch starts on a 16-byte boundary (and the lattice is
+// large enough that the 16-byte copies are not of a few addresses, which is slow).
 bool chain_aligned16(const ctqw_hamiltonian *h, const ChainArgs &a) {
     uintptr_t all = (uintptr_t)a.in | (uintptr_t)a.q | (uintptr_t)a.out;
     for (int i = 0; i < kMaxLevels; ++i) all |= (uintptr_t)a.lev[i] | (uintptr_t)a.mlev[i];
-    return (all & 15) == 0 && h->group_N[0] > 2;
+    return (all & 15) == 0 && h->Nmax > 6;
 }
 
 // Depth for K levels: the fewest launches at depth <= 8, the levels split

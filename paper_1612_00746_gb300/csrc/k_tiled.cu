@@ -968,9 +968,9 @@ int launch_taylor_tiled_range(const ctqw_hamiltonian *h, int shape, const void *
     a.n_stages = n_stages;
     a.final = final;
     a.compensated = compensated;
-    // (at N = 2 all 16-byte copies of a block would be of two addresses: a launch
-    // takes 27 us instead of 11)
-    a.aligned16 = (((uintptr_t)w_in | (uintptr_t)psi | (uintptr_t)w_out | (uintptr_t)lo) & 15) == 0 && h->group_N[0] > 2;
+    // (with a few sites the 16-byte copies of a block are of few addresses: at N = 2
+    // a launch takes 27 us instead of 11, at N = 6 up to 12% more, at N = 8 no more)
+    a.aligned16 = (((uintptr_t)w_in | (uintptr_t)psi | (uintptr_t)w_out | (uintptr_t)lo) & 15) == 0 && h->Nmax > 6;
     CTQW_CUDA_TRY(cudaFuncSetAttribute((const void *)f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)f.smem));
     const int G = (int)h->group_N.size();
