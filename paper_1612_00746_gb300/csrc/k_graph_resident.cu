@@ -324,12 +324,14 @@ cudaLaunchConfig_t resident_config(cudaLaunchAttribute *attr, int CL, int thread
 // of a thread 100 + 60 for each link read there + 400 for each in another CTA,
 // and a barrier.  It is within 20 % of what those took.  None where one launch
 // a stage is faster: that takes some 5 us and 24 links + 40 bytes an amplitude
-// at 19.6 TB/s (links the most of a node), measured the same way; so graphs of
-// many links that cluster CTAs cannot hold near each other stay there.
+// at 19.6 TB/s (links of the mean node: only here every node is padded to the
+// most links), measured the same way; so graphs of many or uneven links that
+// cluster CTAs cannot hold near each other stay there (127 x 222 nodes of 0 to 8
+// links, 2.9 on average, K = 17, 5 steps: 5.1 ms with a launch a stage, 6.3 here).
 int plan_graph_resident(ctqw_graph *g, const int32_t *row_ptr, const int32_t *col, int max_deg) {
     g->res_CL = 0;
     if (g->m != 2) return CTQW_OK;
-    double least = ((24.0 * max_deg + 40.0) * g->D * g->R / 19.6e12 + 5e-6) * 1.92e9;
+    double least = ((24.0 * row_ptr[g->N] / g->N + 40.0) * g->D * g->R / 19.6e12 + 5e-6) * 1.92e9;
     int n_sm = 0;
     CTQW_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, g->device));
     bool enough = false;   // realizations for every SM already
