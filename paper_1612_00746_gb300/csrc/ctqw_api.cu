@@ -784,8 +784,8 @@ static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double
     // in memory of this call that nothing else uses meanwhile: behind the slots;
     // in a slot without a snapshot, at realization 0, which is never on the tiles;
     // or, with snapshots in all of them, the norm or energy of realization 0 in
-    // the sample that follows the launch.  Where there is none of these, the last
-    // slot is left free.
+    // the first of these samples, which is taken after the launch.  Where there is
+    // none of these, the last slot is left free.
     int *const behind = wsb - (size_t)(slots + 1) * sb >= sizeof(int) ? (int *)(w + (size_t)(slots + 1) * sb) : nullptr;
     double *const later = norm_dev ? norm_dev : energy_dev;
     const bool counted = R_f > h->rows_clusters;
@@ -810,8 +810,8 @@ static int propagate_fused_rows(const ctqw_hamiltonian *h, void *psi_dev, double
         int *work = behind;
         double *borrowed = nullptr;
         if (!work && counted && slots > 0) {
-            if (inside == slots && chunk % obs_every == 0 && later) {
-                borrowed = later + ((s0 + chunk) / obs_every) * h->R;
+            if (inside == slots && later) {
+                borrowed = later + (s0 / obs_every + 1) * h->R;
                 work = (int *)borrowed;
             } else {
                 if (inside == slots) chunk = inside-- * obs_every;
