@@ -20,6 +20,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import multiprocessing as mp
 import os
 import statistics
@@ -213,6 +214,23 @@ def fused_traffic(workload: str):
     return ent.get("dram_bytes_per_launch")
 
 
+def fp64_on_chip(N: int, R: int) -> bool:
+    """Whether two-particle FP64 states of one size stay on chip (mirrors
+    resident_f64_ctas of the library: its model of a stage's time, us)."""
+    best, on = 4.1 + 2.6e-5 * R * N * N, False
+    for most in (16, 8, 4):
+        rows = -(-N // most)
+        ctas = -(-N // rows)
+        if -(-rows * N // 256) > 8 or 32 * (rows + 2) * N + 8 * N > 226 * 1024:
+            continue
+        share = (math.ceil((R + 6) // 7 * ctas / 19) if ctas > 8
+                 else max(math.ceil(R * ctas / 148), 2 if R > 120 // ctas else 1))
+        t = 0.5 + 0.0029 * rows * N * share
+        if t < best:
+            best, on = t, True
+    return on
+
+
 def propagation_path(w, dtype, flags, switching=False):
     """Which kernels ctqw_propagate_taylor runs for this workload (mirrors the library)."""
     from paper_1612_00746_gb300 import ctqw
@@ -222,8 +240,9 @@ def propagation_path(w, dtype, flags, switching=False):
         return "plain"
     on_clusters = (dtype == ctqw.C64 and w.m == 2 and w.ragged_sizes is None and w.N <= 256
                    and (not w.periodic or w.N % 4 == 0))
-    if switching:
-        return "rows" if on_clusters else "tiled" if dtype == ctqw.C64 and w.m == 2 else "plain"
+    if switching:   # on the clusters with stages enough a launch
+        enough = w.K * (w.obs_every or w.n_steps) * 12 >= w.N
+        return "rows" if on_clusters and enough else "tiled" if dtype == ctqw.C64 and w.m == 2 else "plain"
     if shape == ctqw.SHAPE_WAVEFRONT:
         return "wavefront"
     if shape >= 9:
@@ -232,6 +251,9 @@ def propagation_path(w, dtype, flags, switching=False):
         return "rows" if shape < 4 else "banded"
     if dtype == ctqw.C64 and w.m == 2 and shape == 0:
         return "tiled"   # the library's default for the other two-particle FP32 handles
+    if (dtype == ctqw.C128 and w.m == 2 and w.ragged_sizes is None and fp64_on_chip(w.N, w.R)
+            and w.K * (w.obs_every or w.n_steps) > 2):
+        return "resident64"
     return "plain"
 
 
@@ -245,7 +267,7 @@ def roofline_of(w, dtype, flags, units, kernel_ms, peaks, traffic, switching=Fal
     compensated final stage), against the measured copy bandwidth; three
     particles take two stages a launch and are bound by the FP32 pipe.  The FP64
     per-term kernels move 48 bytes per site-update but are bound by the FP64
-    pipe (2 DFMA per SM per cycle).
+    pipe (2 DFMA per SM per cycle); small FP64 states stay on chip.
     """
     from paper_1612_00746_gb300 import ctqw
 
@@ -268,10 +290,13 @@ def roofline_of(w, dtype, flags, units, kernel_ms, peaks, traffic, switching=Fal
         flops_per_unit = 8 * w.m + 4
         achieved = units * flops_per_unit / sec / 1e12
         peak = alu_peak(fp64=True)
+        on_chip = path == "resident64"
         return with_measured({"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                              "frac": achieved / peak, "traffic": None, "kernel": "horner2_f64_kernel",
+                              "frac": achieved / peak, "traffic": None,
+                              "kernel": "resident_f64_kernel" if on_chip else f"horner{w.m}_f64_kernel",
                               "kernel_ms": kernel_ms, "flops_per_site_update": flops_per_unit,
-                              "hbm_gbs_achieved": units * 48.0 / sec / 1e9, "bytes_per_site_update": 48.0,
+                              "hbm_gbs_achieved": None if on_chip else units * 48.0 / sec / 1e9,
+                              "bytes_per_site_update": None if on_chip else 48.0,
                               "peak_basis": f"{SM_COUNT} SMs x 2 DFMA x 2 flop x 2070 MHz (FP64, derived)",
                               "timing": "the whole propagate call (observables kernels included)"}, "fp64")
     if w.m == 3 and not flags & ctqw.FLAG_PLAIN:
@@ -477,6 +502,9 @@ def run_ours(args):
         # stages a launch) + one observables kernel per sample
         pairs = w.m == 3 and dtype == ctqw.C64 and not args.flags & ctqw.FLAG_PLAIN
         launches_per_step = 1 + w.n_steps * (-(-w.K // 2) if pairs else w.K) + n_obs
+    elif path == "resident64":
+        # init_state + a launch per sampling interval + one observables kernel per sample
+        launches_per_step = 1 + (-(-w.n_steps // w.obs_every) if w.obs_every else 1) + n_obs
     elif path == "tiled":
         # ceil(K / D) launches per step and size group, observables, init
         launches8 = -(-w.K // 8)
@@ -743,7 +771,7 @@ def run_ours(args):
         "gpu_launches": launches_per_step * args.steps,
         "fused_split": ({"clusters_realizations": w.R - split, "tiles_realizations": split,
                          "what": "the last realizations on the register tiles on a second stream, "
-                                 "on the SMs no 16-CTA cluster can hold"} if path == "rows" else None),
+                                 "on the SMs no cluster can hold"} if path == "rows" else None),
         "one_stream": one_stream,
         "roofline": roofline,
         "e2e": e2e,

@@ -62,7 +62,8 @@ extern "C" {
                                           error word) by its norm: the corrective action of the norm check of
                                           Algorithms 2 and 3 (Sec. 2.2: RK4 does not conserve the norm).  Runs
                                           on the per-term path (workspace as CTQW_FLAG_PLAIN), two extra
-                                          launches per step; sampled norms are then 1 up to rounding */
+                                          launches per step; sampled norms are then 1 up to rounding.  The
+                                          norms lie in the handle: such calls on one handle must not overlap */
 #define CTQW_FLAG_TEST_WAIT_TIMEOUT 0x8 /* failure-path test: the fused kernel first waits on an mbarrier that
                                            nothing completes, gives up after 1 ms and flags the handle */
 #define CTQW_FLAG_ONE_STREAM 0x10      /* fused path: run every realization on the clusters, on the caller's
@@ -87,7 +88,7 @@ extern "C" {
  * iterate in shared memory (tile <= 56, D = 4); i = 1 keeps it in registers
  * on 64 x 128 regions (4 columns a lane), D = 8; i = 2 on 96 x 64 regions
  * (12 warps), D = 8; i = 3..6 on 64 x 64 regions (2 columns a lane),
- * D = 4, 8, 2, 7 (tile 64 - 2D).  Needs the per-term workspace (3 states). */
+ * D = 4, 8, 2, 7 (tile 64 - 2D, at odd D and even N two columns less).  Needs the per-term workspace (3 states). */
 #define CTQW_SHAPE_TILED(i) (9 + (i))
 
 typedef struct ctqw_hamiltonian ctqw_hamiltonian;   /* opaque, owned by the library */
@@ -269,14 +270,15 @@ int ctqw_propagate_taylor(const ctqw_hamiltonian *h, int32_t dtype, void *psi_de
  * How many realizations the fused path of ctqw_propagate_taylor (and of
  * ctqw_propagate_rk4, at K = 4) hands to the register tiles on the handle's
  * second stream, given a workspace of at least 3 states: the last *R_tiled
- * realizations.  A 16-CTA cluster (two particles, N = 256) needs 8 SMs of
- * one GPC, so the SMs left over in each GPC hold no cluster; the tiles get
- * the share of realizations that their throughput on those SMs can finish
- * in the time the clusters take for the rest (whole rounds of the resident
- * clusters), if that is sooner than the clusters alone.  0 when fewer than 1/16 of the SMs are left over, when the
- * handle has no fused path, with CTQW_FLAG_ONE_STREAM, CTQW_FLAG_PLAIN or
- * CTQW_FLAG_RENORMALIZE, or with a shape flag.  Queries the device's
- * occupancy; launches nothing.  Errors: CTQW_EINVAL for a null handle or
+ * realizations.  A cluster (two particles, N = 256: 8 CTAs, one an SM) needs
+ * its SMs in one GPC, so the SMs left over in each GPC hold no cluster; the
+ * tiles get the share of realizations that they can finish on those SMs in
+ * the time the clusters take for the rest (whole rounds of the resident
+ * clusters), if that is sooner than the clusters alone.  0 when fewer than
+ * 1/16 of the SMs are left over, when two CTAs of the clusters share an SM,
+ * when the handle has no fused path, with CTQW_FLAG_ONE_STREAM,
+ * CTQW_FLAG_PLAIN or CTQW_FLAG_RENORMALIZE, or with a shape flag.  Launches
+ * nothing.  Errors: CTQW_EINVAL for a null handle or
  * pointer or K outside 1..30.
  */
 int ctqw_fused_split(const ctqw_hamiltonian *h, int32_t K, uint32_t flags, int32_t *R_tiled);
@@ -295,8 +297,10 @@ int ctqw_fused_split(const ctqw_hamiltonian *h, int32_t K, uint32_t flags, int32
  * to its right (never the absent wrap bond of an open chain).
  * The call first restores the parameters as built, so equal arguments give
  * equal results; afterwards the handle holds the parameters after the last
- * update (ctqw_get_params).  Paths: two particles in CTQW_C64 on the fused
- * cluster kernel where ctqw_propagate_taylor uses it (the clusters redraw
+ * update (ctqw_get_params).  Calls that overlap on one handle are not
+ * allowed: the parameters are the handle's.  Paths: two particles in CTQW_C64 on the fused
+ * cluster kernel where ctqw_propagate_taylor uses it and a sampling interval
+ * has stages enough (the clusters redraw
  * their realization's parameters after every step, a launch per sampling
  * interval), else on the temporally blocked tiles; everything else (or
  * CTQW_FLAG_PLAIN) one launch per term; all need 3 states of workspace
@@ -335,8 +339,9 @@ int ctqw_propagate_exact(const ctqw_hamiltonian *h, int32_t dtype, void *psi_dev
  * corrected.  This update map is the order-4 Taylor polynomial of
  * exp(-i H dt) (Sec. 2.3: order-n RK and order-n Taylor coincide for the
  * exponential); the call evaluates that polynomial as ctqw_propagate_taylor
- * with K = 4 does.  With CTQW_FLAG_PLAIN (or CTQW_FLAG_RENORMALIZE) one
- * launch per stage runs the four stages above.  Both need the workspace of
+ * with K = 4 does.  With CTQW_FLAG_PLAIN (or CTQW_FLAG_RENORMALIZE), and for
+ * many CTQW_C64 rings of up to 24 sites, one launch per stage runs the four
+ * stages above.  Both need the workspace of
  * ctqw_workspace_size(method = 1).
  */
 int ctqw_propagate_rk4(const ctqw_hamiltonian *h, int32_t dtype, void *psi_dev, double dt,
@@ -580,7 +585,8 @@ int ctqw_graph_workspace_size(const ctqw_graph *g, int32_t dtype, size_t *bytes)
  * Advance every realization by n_steps order-K Taylor steps (Sec. 2.3,
  * Algorithm 3), one launch per term over all realizations; m = 2 in CTQW_C64
  * on graphs whose two iterates fit on chip (a few hundred nodes of at most 8
- * links), where that is faster, one launch per sampling interval.  CTQW_C128 runs
+ * links), where that is faster, one launch per sampling interval of more than
+ * two stages.  CTQW_C128 runs
  * the terms in the order of Algorithm 3; CTQW_C64 the same polynomial in
  * Horner form with the state update compensated (the carried rounding
  * error lives in the third workspace state), as the chain's per-term path.

@@ -737,7 +737,7 @@ static int side_can_follow(const ctqw_hamiltonian *h, cudaStream_t s, bool *can)
 // the slots inside).  Without observables it is one launch.  With no
 // workspace, one of 3 states is allocated stream-ordered.
 //
-// A 16-CTA cluster needs 8 SMs of one GPC, so some SMs hold no cluster.
+// A cluster (N = 256: 8 CTAs, one an SM) needs its SMs in one GPC, so some SMs hold none.
 // With S >= 2 the last realizations (fused_rows_split) run meanwhile on the
 // register tiles on the handle's side stream, forked from and joined to the
 // caller's stream: the tiles use slots 1 and 2 of their own realizations as

@@ -288,8 +288,9 @@ bool fused_rows_switching_supported(const ctqw_hamiltonian *h, int dtype);
 int plan_fused_rows(ctqw_hamiltonian *h);
 // How many realizations (the last ones) to run on the register tiles on the
 // handle's side stream while the clusters run the rest: the SMs that hold no
-// cluster (a 16-CTA cluster needs 8 SMs of one GPC) take a share matched to
-// their throughput.  0 when under 1/16 of the SMs would be idle.
+// cluster (N = 256: 8 CTAs, one an SM of one GPC) take a share that takes them no
+// longer.  0 when under 1/16 of the SMs would be idle, and where two CTAs of the
+// clusters share an SM.
 int fused_rows_split(const ctqw_hamiltonian *h, int shape, int K, int *R_tiled);
 int launch_taylor_fused_rows(const ctqw_hamiltonian *h, void *psi, void *lo, void *snap,
                              int snap_every, double dt, int K, int64_t n_steps, int compensated,

@@ -50,6 +50,9 @@
 // 9.1e11 -> 1.11e12; N = 100, on the register tiles before, 4.4e11 -> 7.6e11;
 // one realization of N = 64, 10 steps: 129 us -> 73 us.
 //
+// (At 4 columns a lane 16 warps leave 128 registers, and a thread spills 56 bytes,
+// 100 with switching noise; the other widths spill nothing.)
+//
 // Control flow: the stages of a step are a first one (from psi), middle ones
 // in pairs and a final one, with no per-stage dispatch.  A row tests the few
 // columns that the diagonal x1 = x2 can meet it in; a step loop compiled per

@@ -259,7 +259,9 @@ __global__ void __launch_bounds__(256) taylor_tiled_kernel(const __grid_constant
 // tile, both by cp.async into shared memory (a lane reads back only slots it
 // filled itself, so they need no barrier).  The row coefficients are 8-byte
 // broadcasts: 16-byte ones cost twice the shared-memory wavefronts, and that
-// pipe is the bound (78% busy; 8 warps x 3 blocks an SM).  The ragged batch
+// pipe is the bound (78% busy; 8 warps x 3 blocks an SM; at their 80 registers a
+// thread spills 44 bytes, loaded 88 to 128 bytes at a time and 324 for odd N,
+// through the same pipe).  The ragged batch
 // of 512 realizations, N = 128..1024, K = 8, 20 steps: 97.5 ms with the
 // error words read in the final stage and psi read twice, 79.9 ms with both
 // fetched at the start, 74.2 ms with the 8-byte coefficients and the regions
